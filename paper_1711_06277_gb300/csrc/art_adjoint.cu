@@ -138,7 +138,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
     WalkT<Cell> W;
     // pass-1 start of the ray (next face per axis, start cell), so that a leaf's pass 2
     // restarts without a new ray set-up
-    df t0[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    fix t0[3] = {0, 0, 0};
     int idx0 = 0;
     unsigned s = 0, p = 0;
     unsigned slot = 0;
@@ -146,7 +146,6 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
     df own = {0.f, 0.f};   // own weighted sum (pass 1), kept for dL in pass 2
     float total = 0.f;     // own + descendants (pass 2), passed to the parent
     df rem = {0.f, 0.f};   // weighted sum over what follows the current segment (pass 2)
-    df rmax = LV.rmax;     // radius where the ray of level lv ends (split or cutoff)
     bool splits = false;
     unsigned ncross = 0, nrays = 0;
     // Every step crosses at least one face and the sentinel ring ends every walk that
@@ -181,9 +180,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
             rem = df_add(own, {__ldcg(Pl.sub + slot), 0.f});
             total = rem.hi + rem.lo;
             const LevelInfo Lp = A.levels[lv];
-            if constexpr (!kCut) rmax = Lp.rmax;
-            ray_begin(A, Lp, Pl, lv, slot, W, recs, s, p, L0, splits);
-            if constexpr (kCut) rmax = end_radius(splits, Lp.rmax, A.dmax);
+            ray_begin<kCut>(A, Lp, Pl, lv, slot, W, recs, s, p, L0, splits);
             Ls = __ldg(A.srcL + s);
             mode = 2;
             return;
@@ -207,9 +204,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
                 if (mode == 0 && rank < avail) {
                     slot = wnext + rank;
                     lv = l;
-                    if constexpr (!kCut) rmax = LV.rmax;
-                    const int st = ray_begin(A, LV, B, l, slot, W, recs, s, p, L0, splits);
-                    if constexpr (kCut) rmax = end_radius(splits, LV.rmax, A.dmax);
+                    const int st = ray_begin<kCut>(A, LV, B, l, slot, W, recs, s, p, L0, splits);
                     if (st > 0) {
                         Ls = __ldg(A.srcL + s);
                         t0[0] = W.t[0];
@@ -250,8 +245,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
                 const float wv = cm.z;   // weight and neutral-H opacity of this cell
                 const float hv = cm.y;
                 const float q = force_weight(W.cell, W.n, A.fscale);
-                // a ray ends at a radius (rmax) when it can split or (kCut) at the cutoff
-                const StepOut o = walk_step<false, true>(W, kCut || splits, rmax, recs, A.tau_max);
+                const StepOut o = walk_step<false, true>(W, A.fbits, recs, A.tau_max);
                 // this segment's loss: w k G, plus q dL with a force term
                 const float g = fmaf(q, o.dL, wv * gs * o.G);
                 if (mode == 1) {
@@ -269,7 +263,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
                 if (o.ev != EV_NONE) {
                     if (mode == 1) {
                         const unsigned long long c4 = 4ull * (slot - b32);
-                        if (o.ev == EV_SPLIT && (!kCut || splits_at_end(splits, LV.rmax, A.dmax))) {
+                        if (o.ev == EV_SPLIT && splits_at_end<kCut>(splits, LV.rmaxx, A.dmax)) {
                             B.own[slot] = make_float2(own.hi, own.lo);
                             B.sub[slot] = 0.f;
                             B.pending[slot] = 4u;
@@ -299,7 +293,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
                             W.t[1] = t0[1];
                             W.t[2] = t0[2];
                             W.idx = idx0;
-                            W.tc = LV.r0;
+                            W.tc = LV.r0x;
                             W.L = L0;
                             W.Lc = 0.f;
                             W.tau = l == A.level0 ? 0.f : __ldcg(B.tau + slot);

@@ -103,6 +103,28 @@ int check_params(const art_params* p)
 // Split radius r_max(l) = [3/(pi m_ray)]^(1/2) 2^l in cells (Sec. 2.1).
 double rmax_cells(double m_ray, int level) { return rmax_unit(m_ray) * std::ldexp(1.0, level); }
 
+// A distance in cells as a fixed-point number; distances beyond every box (radii of levels
+// that no ray reaches) end up just below kFar.
+fix to_fix(double cells, int fbits)
+{
+    const double v = std::ldexp(cells, fbits);
+    return v < (double)kFar ? (fix)std::llrint(v) : kFar - 1;
+}
+
+// Device record of a source at u (cell units).
+SrcDev source_record(const art_grid* g, const double u[3], double base_L, int lmax)
+{
+    SrcDev d;
+    float h[3], lo[3], lmf;
+    for (int a = 0; a < 3; ++a) split_df(u[a], h[a], lo[a]);
+    std::memcpy(&lmf, &lmax, sizeof(float));
+    d.hi = make_float4(h[0], h[1], h[2], (float)base_L);
+    d.lo = make_float4(lo[0], lo[1], lo[2], lmf);
+    d.xy = make_longlong2(to_fix(u[0], g->fbits), to_fix(u[1], g->fbits));
+    d.z_ = make_longlong2(to_fix(u[2], g->fbits), 0);
+    return d;
+}
+
 // Direction tables of levels lfrom..lto (FP64 HEALPix, rotated by p's rotation, split
 // into hi + lo), rebuilt when the rotation changes.
 int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto)
@@ -128,7 +150,7 @@ int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto)
             unsigned blocks = (unsigned)((npix + 255) / 256);
             k_directions<<<blocks, 256, 0, g->stream>>>(l, npix, r[0], r[1], r[2], r[3], r[4],
                                                         r[5], r[6], r[7], r[8], rotate ? 1 : 0,
-                                                        g->dir[l]);
+                                                        std::ldexp(1.0, g->fbits), g->dir[l]);
             ART_TRY(cudaGetLastError());
             g->dir_built[l] = true;
         }
@@ -155,14 +177,8 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         int lm = source_level_max(g, u, l0, p->level_max, p->m_ray);
         g->src_lmax[s] = lm;
         if (lm > lmax_glob) lmax_glob = lm;
-        float h[3], lo[3];
-        for (int a = 0; a < 3; ++a) split_df(u[a], h[a], lo[a]);
         const double lb = adjoint ? 1.0 / (double)npix0 : g->L[s] / (double)npix0;
-        int lmi = lm;
-        float lmf;
-        std::memcpy(&lmf, &lmi, sizeof(float));
-        hs[s].hi = make_float4(h[0], h[1], h[2], (float)lb);
-        hs[s].lo = make_float4(lo[0], lo[1], lo[2], lmf);
+        hs[s] = source_record(g, u, lb, lm);
     }
     if ((size_t)ns > g->src_cap) {
         dev_free(g->d_src);
@@ -222,7 +238,8 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         double r0 = l > l0 ? unit * std::ldexp(1.0, l - 1) : 0.0;
         double r1 = unit * std::ldexp(1.0, l);
         split_df(r0, lv[l].r0.hi, lv[l].r0.lo);
-        split_df(r1, lv[l].rmax.hi, lv[l].rmax.lo);
+        lv[l].r0x = to_fix(r0, g->fbits);
+        lv[l].rmaxx = to_fix(r1, g->fbits);
         lv[l].dir = g->dir[l];
         lv[l].destroy_w = 1ull << (2 * (lmax_glob - l));
     }
@@ -309,8 +326,9 @@ TraceArgs make_args(art_grid* g, const art_params* p)
 {
     TraceArgs A;
     std::memset(&A, 0, sizeof(A));
-    // the d_max cutoff in cell units (read only by the kernels built for a cutoff)
-    split_df(p->d_max > 0.0 ? p->d_max / g->dx : (double)kBig, A.dmax.hi, A.dmax.lo);
+    // the d_max cutoff (read only by the kernels built for a cutoff)
+    A.dmax = p->d_max > 0.0 ? to_fix(p->d_max / g->dx, g->fbits) : kNoEnd;
+    A.fbits = g->fbits;
     A.nx = g->n[0];
     A.ny = g->n[1];
     A.nz = g->n[2];
@@ -404,6 +422,9 @@ int art_create_grid(art_grid** out, int nx, int ny, int nz, const double box_lo[
     g->npad = npad;
     for (int a = 0; a < 3; ++a) g->lo[a] = box_lo[a];
     g->dx = dx;
+    // as many fraction bits as keep every distance inside the box below 2^61
+    g->fbits = 61 - (int)std::ceil(std::log2(
+                        std::sqrt((double)nx * nx + (double)ny * ny + (double)nz * nz) + 4.0));
     g->nH0 = d_nH0;
     g->nH = d_nH;
     g->stream = (cudaStream_t)stream;

@@ -1,10 +1,14 @@
 // art_device.cuh -- device-side building blocks of the GB300 adaptive ray trace.
 //
-// * Double-float ("df") arithmetic: a value is an unevaluated sum hi + lo of two floats,
-//   ~44 significant bits. Ray positions, face-crossing distances and split radii are held
-//   this way so that a ray several hundred cells from its source still places its faces to
-//   ~1e-11 cells, while every per-crossing operation stays on the FP32 pipes (FP64 throughput
-//   on this part is a small fraction of FP32).
+// * Distances along a ray (next face per axis, current position, split radii) are 64-bit
+//   fixed-point numbers with TraceArgs::fbits fraction bits, as many as the box diagonal
+//   leaves room for (51 at 512^3): a face 500 cells from the source sits within 1e-12 cells
+//   of its place, an advance is one 64-bit integer add and an order decision one compare.
+//   Against pairs of floats this took the reverse sweep, which is bound by its instructions,
+//   from 9.82 to 8.91 ms (128^3, 16 sources) and the forward trace, which is bound by its
+//   deposits, from 83.6 to 81.9 ms (256^3, 64 sources).
+// * Double-float ("df") arithmetic (an unevaluated sum hi + lo of two floats, ~44 significant
+//   bits) places the start of a ray: FP64 throughput on this part is a small fraction of FP32.
 // * The ray-walk state and one crossing step of Sec. 2.1 (Kim et al. 2017): next face
 //   crossing per axis measured from the source, segment length, attenuation
 //   dL = L (1 - e^-dtau) with dtau = chi ds (Eq. e:RT2), deposit of sum dL/chi and sum dL n
@@ -19,7 +23,6 @@ namespace art {
 
 constexpr int kNL = 20;                 // level slots (levels 0..13 used)
 constexpr unsigned kFull = 0xffffffffu;
-constexpr float kBig = 1.0e30f;         // "never": crossing distance of an axis with n_a = 0
 
 // ---------------------------------------------------------------------------------------
 // double-float arithmetic
@@ -54,41 +57,70 @@ __device__ __forceinline__ df df_mul(df a, df b)
     e = fmaf(a.lo, b.hi, e);
     return df_quick(p, e);
 }
-__device__ __forceinline__ df df_div(df a, df b)
+
+// ---------------------------------------------------------------------------------------
+// fixed-point distances
+// ---------------------------------------------------------------------------------------
+using fix = long long;
+// "Never reached": the face distance of an axis with n_a = 0 and of faces beyond the box.
+// Faces inside the box lie below 2^61 (see fraction_bits), so kFar stays apart from them and
+// a face step of at most kFarStep keeps every sum below 2^63.
+constexpr fix kFar = 1ll << 62;
+constexpr fix kFarStep = 1ll << 61;
+constexpr fix kNoEnd = 0x7fffffffffffffffll;  // end radius of a ray that ends at no radius
+
+// Face spacing 1/|n_a| of the direction tables: m 2^(8k) with m < 2^61 in the low bits and
+// the smallest such k (0..3) above them. n_a is 0 or at least 2^-24, so the product with an
+// offset keeps its accuracy where the spacing itself is far beyond the box.
+__device__ __forceinline__ fix encode_spacing(double spacing)
 {
-    float q1 = __fdiv_rn(a.hi, b.hi);
-    df r = df_add(a, df_neg(df_mul({q1, 0.f}, b)));
-    float q2 = __fdiv_rn(r.hi, b.hi);
-    return df_quick(q1, q2);
+    unsigned long long k = 0;
+    while (spacing >= 0x1p61) {
+        spacing *= 0x1p-8;
+        ++k;
+    }
+    const unsigned long long m = (unsigned long long)__double2ll_rn(spacing);
+    return (fix)(m < (1ull << 61) ? m | (k << 61) : (1ull << 53) | ((k + 1) << 61));
 }
-// a <= b for normalised df values (lexicographic on hi, lo)
-__device__ __forceinline__ bool df_le(df a, df b)
+
+// The distance to the next face from the spacing code: off * spacing for an offset of `off`
+// cells (fixed-point, >= 0) along the axis; kFar when that is beyond every box. step receives
+// the distance between faces, at most kFarStep. 33 <= fbits <= 59.
+__device__ __forceinline__ fix face_distance(fix off, fix code, int fbits, fix& step)
 {
-    return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo);
-}
-// a - b rounded to float; exact enough when a and b are close (Sterbenz on hi)
-__device__ __forceinline__ float df_diff(df a, df b)
-{
-    return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo));
+    const unsigned k8 = 8u * (unsigned)((unsigned long long)code >> 61);
+    const unsigned long long a = (unsigned long long)off;
+    const unsigned long long b = (unsigned long long)code & ((1ull << 61) - 1ull);
+    const unsigned long long hi = __umul64hi(a, b), lo = a * b;
+    const unsigned s = (unsigned)fbits - 32u;
+    const unsigned l0 = (unsigned)lo, l1 = (unsigned)(lo >> 32);
+    const unsigned h0 = (unsigned)hi, h1 = (unsigned)(hi >> 32);
+    const unsigned w1 = __funnelshift_l(l0, l1, k8), w2 = __funnelshift_l(l1, h0, k8),
+                   w3 = __funnelshift_l(h0, h1, k8);
+    const unsigned t0 = __funnelshift_r(w1, w2, s), t1 = __funnelshift_r(w2, w3, s);
+    step = k8 ? kFarStep : (fix)b;
+    return (hi >> ((unsigned)fbits - 2u - k8)) ? kFar : (fix)(((unsigned long long)t1 << 32) | t0);
 }
 
 // ---------------------------------------------------------------------------------------
 // shared data layouts
 // ---------------------------------------------------------------------------------------
 
-// Per source: position in cell units (df split over two float4) + base-ray luminosity and
-// the source's l_max.
+// Per source: position in cell units (df split over two float4, and fixed-point) + base-ray
+// luminosity and the source's l_max.
 struct SrcDev {
     float4 hi;  // u_x, u_y, u_z (hi parts), L / N_ray(l0)
     float4 lo;  // u_x, u_y, u_z (lo parts), l_max (int bits)
+    longlong2 xy;  // u_x, u_y (fixed-point)
+    longlong2 z_;  // u_z (fixed-point), unused
 };
 
 // Per level constants of a trace.
 struct LevelInfo {
     df r0;              // start radius of level-l rays (r_max(l-1), 0 at l0), cell units
-    df rmax;            // split radius r_max(l), cell units
-    const float4* dir;     // direction table of level l: 3 float4 per pixel holding
-                           // n (hi, lo) and 1/n (hi, lo) per axis
+    fix r0x, rmaxx;     // the same and the split radius r_max(l), fixed-point
+    const float4* dir;     // direction table of level l: 3 float4 per pixel holding n
+                           // (hi, lo) and a face spacing code per axis
     unsigned long long destroy_w;  // 4^(l_max_global - l)
 };
 
@@ -161,8 +193,9 @@ struct TraceArgs {
     const float* srcL;       // adjoint: source luminosities (gradients scale with them)
     const CellF* recf;       // adjoint with a force term: per cell {chi, chi_H, w, 0}, {v, 0}
     const CellW* recw;       // adjoint without dust and force term: per cell {chi, w}
-    df dmax;                 // d_max cutoff in cell units (kernels built for a cutoff only)
+    fix dmax;                // d_max cutoff (kernels built for a cutoff only)
     float fscale;            // adjoint: force per unit momentum (1 / dV)
+    int fbits;               // fraction bits of the fixed-point distances
 };
 
 enum : int { EV_NONE = 0, EV_EXIT = 1, EV_DROP = 2, EV_SPLIT = 3 };
@@ -211,9 +244,10 @@ template <> __device__ __forceinline__ CellF cell_zero<CellF>()
 
 template <class Cell>
 struct WalkT {
-    df t[3];      // distance from the source to the next face on each axis
-    df d[3];      // distance between consecutive faces on each axis (1/|n_a|)
-    df tc;        // distance of the current position
+    fix t[3];     // distance from the source to the next face on each axis
+    fix d[3];     // distance between consecutive faces on each axis (1/|n_a|)
+    fix tc;       // distance of the current position
+    fix rend;     // radius where the ray ends (split or cutoff), kNoEnd if at none
     int idx;      // index of the current cell in the padded layout (sentinel ring around
                   // the grid, see pad_index)
     int ss[3];    // signed index step of a crossing on each axis
@@ -258,12 +292,13 @@ __device__ __forceinline__ unsigned pad_of(unsigned i, int nx, int ny)
     return (unsigned)pad_index(x, r % (unsigned)ny, r / (unsigned)ny, nx, ny);
 }
 
-// Sets up the walk of a ray with direction n and reciprocal inv (df, from the direction
-// table) from source position u (df) starting at radius r0. Returns false if the start
-// point lies outside the grid.
+// Sets up the walk of a ray with direction n (df) and face spacing codes (both from the
+// direction table) from source position u (df, and ux fixed-point) starting at radius r0.
+// Returns false if the start point lies outside the grid.
 template <class Cell>
-__device__ __forceinline__ bool walk_start(WalkT<Cell>& W, int nx, int ny, int nz, const df u[3],
-                                           const df n[3], const df inv[3], df r0)
+__device__ __forceinline__ bool walk_start(WalkT<Cell>& W, int nx, int ny, int nz, int fbits,
+                                           const df u[3], const fix ux[3], const df n[3],
+                                           const fix code[3], df r0, fix r0x)
 {
     const int N[3] = {nx, ny, nz};
     int c[3];
@@ -277,20 +312,15 @@ __device__ __forceinline__ bool walk_start(WalkT<Cell>& W, int nx, int ny, int n
         c[a] = ci;
         inside = inside && ci >= 0 && ci < N[a];
         W.n[a] = n[a].hi;
-        if (n[a].hi != 0.f) {
-            const bool up = n[a].hi > 0.f;
-            const int stride = a == 0 ? 1 : (a == 1 ? nx + 2 : (nx + 2) * (ny + 2));
-            W.ss[a] = up ? stride : -stride;
-            const df off = df_add({(float)(up ? ci + 1 : ci), 0.f}, df_neg(u[a]));
-            W.t[a] = df_mul(off, inv[a]);
-            W.d[a] = up ? inv[a] : df_neg(inv[a]);
-        } else {
-            W.ss[a] = 0;
-            W.t[a] = {kBig, 0.f};
-            W.d[a] = {0.f, 0.f};
-        }
+        const bool up = n[a].hi > 0.f, flat = n[a].hi == 0.f;
+        const int stride = a == 0 ? 1 : (a == 1 ? nx + 2 : (nx + 2) * (ny + 2));
+        W.ss[a] = flat ? 0 : (up ? stride : -stride);
+        const fix face = (fix)(up ? ci + 1 : ci) << fbits;
+        const fix off = up ? face - ux[a] : ux[a] - face;
+        const fix t = face_distance(off > 0 ? off : 0, code[a], fbits, W.d[a]);
+        W.t[a] = flat ? kFar : t;
     }
-    W.tc = r0;
+    W.tc = r0x;
     W.idx = inside ? (int)pad_index(c[0], c[1], c[2], nx, ny) : 0;
     return inside;
 }
@@ -315,17 +345,31 @@ struct StepOut {
 // sinh(y)/y to y^8 (truncation < 3e-11 for y < 1/2, no cancellation); above 1 as
 // (1 - e^{-x})/x with e^{-x} = (e^{-x/2})^2. One exponential serves both branches, which are
 // evaluated and selected, so lanes never diverge here.
+__device__ __forceinline__ float ex2_ftz(float v)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float rcp_ftz(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+constexpr float kHalfLog2e = 0.72134752f;  // log2(e) / 2: e^{-x/2} = 2^{-x kHalfLog2e}
+
 __device__ __forceinline__ float phi_of(float x)
 {
     const float y = 0.5f * x;
-    const float E = __expf(-y);
+    const float E = ex2_ftz(-kHalfLog2e * x);
     const float y2 = y * y;
     float S = fmaf(y2, 1.f / 362880.f, 1.f / 5040.f);
     S = fmaf(S, y2, 1.f / 120.f);
     S = fmaf(S, y2, 1.f / 6.f);
     S = fmaf(S, y2, 1.f);
     const float small = E * S;
-    const float large = __fdividef(fmaf(-E, E, 1.f), fmaxf(x, 1.f));
+    const float large = fmaf(-E, E, 1.f) * rcp_ftz(fmaxf(x, 1.f));
     return x < 1.f ? small : large;
 }
 
@@ -335,7 +379,7 @@ __device__ __forceinline__ float phi_of(float x)
 __device__ __forceinline__ float phi_dphi(float x, float& dphi)
 {
     const float y = 0.5f * x;
-    const float E = __expf(-y);
+    const float E = ex2_ftz(-kHalfLog2e * x);
     const float y2 = y * y;
     float S = fmaf(y2, 1.f / 362880.f, 1.f / 5040.f);
     S = fmaf(S, y2, 1.f / 120.f);
@@ -345,7 +389,7 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
     Sp = fmaf(Sp, y2, 1.f / 30.f);
     Sp = fmaf(Sp, y2, 1.f / 3.f);
     Sp *= y;
-    const float r = __fdividef(1.f, fmaxf(x, 1.f));
+    const float r = rcp_ftz(fmaxf(x, 1.f));
     const float E2 = E * E;
     const float large = (1.f - E2) * r;
     const bool sm = x < 1.f;
@@ -353,73 +397,57 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
     return sm ? E * S : large;
 }
 
-__device__ __forceinline__ df df_sel(bool c, df a, df b) { return {c ? a.hi : b.hi, c ? a.lo : b.lo}; }
-
-// One step of the walk: the segment from tc to the next face or to the split radius rmax
-// (when the ray splits at all). The common case (one axis crossing) runs without branches;
-// faces crossed together (ties) take a short side path. When the step ends the ray (event
-// other than EV_NONE) the walk state other than L and tau is left unspecified.
+// One step of the walk: the segment from tc to the next face or to the end radius. The
+// common case (one axis crossing) runs without branches; faces crossed together (ties) take
+// a short side path. When the step ends the ray (event other than EV_NONE) the walk state
+// other than L and tau is left unspecified.
 template <bool kCountOnly, bool kDphi = false, class Cell>
-__device__ __forceinline__ StepOut walk_step(WalkT<Cell>& W, bool splits, df rmax,
+__device__ __forceinline__ StepOut walk_step(WalkT<Cell>& W, int fbits,
                                              const Cell* __restrict__ cells, float tau_max)
 {
     StepOut o;
     // A step that starts in a sentinel cell ends the ray: it left the grid with the crossing
     // of the previous step (whose segment was deposited then); nothing is deposited now.
     const bool out = chi_of(W.cell) < 0.f;
-    // Earliest face crossing, decided on the hi parts: for normalised df values |lo| is at
-    // most half an ulp of hi, so distinct hi parts order the values exactly. Equal hi parts
-    // (exact ties, near ties, a face at the split radius) take the exact double-float path
-    // below. Two values within the 1e-12 tie tolerance can still have distinct hi parts when
-    // they straddle a rounding boundary of hi; the walk then crosses the two faces in two
-    // steps with a segment far below the 1e-5-cell near-tie threshold between them, a ray
-    // the oracle flags as near-tie.
-    const float h0 = W.t[0].hi, h1 = W.t[1].hi, h2 = W.t[2].hi;
-    const bool c01 = h0 < h1;
-    const float h01 = c01 ? h0 : h1;
-    const bool c2 = h01 < h2;
-    bool p0 = c2 && c01, p1 = c2 && !c01, p2 = !c2;  // the earliest axis
-    const float hm = c2 ? h01 : h2;
-    df tm = {hm, p2 ? W.t[2].lo : (c01 ? W.t[0].lo : W.t[1].lo)};
-    bool split = splits && rmax.hi < hm;
-    // next cell, for the usual single-axis crossing
-    int nidx = W.idx + (p2 ? W.ss[2] : (c01 ? W.ss[0] : W.ss[1]));
-    // the second-earliest hi part: a tie with the earliest face, or the split radius at the
-    // earliest face, needs the exact comparison (axes parallel to the grid sit at kBig and
-    // tie only with each other, never with the earliest face)
-    const float h2nd = c2 ? fminf(c01 ? h1 : h0, h2) : h01;
-    if (h2nd == hm || (splits && rmax.hi == hm)) {
-        const bool e01 = df_le(W.t[0], W.t[1]);
-        tm = df_sel(e01, W.t[0], W.t[1]);
-        int a = e01 ? 0 : 1;
-        if (!df_le(tm, W.t[2])) {
-            tm = W.t[2];
-            a = 2;
-        }
-        p0 = a == 0;
-        p1 = a == 1;
-        p2 = a == 2;
-        split = splits && df_le(rmax, tm);
-        // axes crossing together with the earliest one (relative tie 1e-12): a diagonal step
-        const float tol = 1e-12f * tm.hi;
-        const bool m0 = df_diff(W.t[0], tm) <= tol;
-        const bool m1 = df_diff(W.t[1], tm) <= tol;
-        const bool m2 = df_diff(W.t[2], tm) <= tol;
-        nidx = W.idx + (m0 ? W.ss[0] : 0) + (m1 ? W.ss[1] : 0) + (m2 ? W.ss[2] : 0);
-        // tied axes other than a advance here; axis a advances with the common path below
-        if (m0 && a != 0) W.t[0] = df_add(W.t[0], W.d[0]);
-        if (m1 && a != 1) W.t[1] = df_add(W.t[1], W.d[1]);
-        if (m2 && a != 2) W.t[2] = df_add(W.t[2], W.d[2]);
+    // Earliest of the three faces and the end radius, decided on the high words (2^-19 cells
+    // at 512^3): different high words order the distances exactly. Equal ones (exact ties,
+    // near ties, a face at the end radius) take the exact 64-bit comparison below. Two
+    // distances within the 1e-12 tie tolerance can still have different high words when they
+    // straddle a boundary; the walk then crosses the two faces in two steps with a segment
+    // far below the 1e-5-cell near-tie threshold between them, a ray the oracle flags as
+    // near-tie.
+    const int h0 = (int)(W.t[0] >> 32), h1 = (int)(W.t[1] >> 32), h2 = (int)(W.t[2] >> 32);
+    const int hr = (int)(W.rend >> 32);
+    const int hm = min(min(h0, h1), min(h2, hr));
+    bool p0 = h0 == hm, p1 = h1 == hm, p2 = h2 == hm, split = hr == hm;
+    fix tm = p0 ? W.t[0] : (p1 ? W.t[1] : (p2 ? W.t[2] : W.rend));
+    if ((p0 && p1) || ((p0 || p1) && p2) || (split && (p0 || p1 || p2))) {
+        const fix m = min(min(W.t[0], W.t[1]), W.t[2]);
+        split = W.rend <= m;
+        tm = split ? W.rend : m;
+        // axes crossing together with the earliest one (relative tie 2^-40): a diagonal step
+        const fix tol = m >> 40;
+        p0 = W.t[0] - m <= tol;
+        p1 = W.t[1] - m <= tol;
+        p2 = W.t[2] - m <= tol;
     }
-    o.ds = df_diff(split ? rmax : tm, W.tc);
+    // segment length: the distance moved, below 2 cells, to 2^-30 cells
+    const fix mv = tm - W.tc;
+    const int q = (int)__funnelshift_r((unsigned)mv, (unsigned)(mv >> 32), (unsigned)fbits - 30u);
+    // deposit in the current cell (segments of length <= 0 deposit nothing)
+    const bool seg = !out && mv > 0;
+    const float ds = seg ? (float)q * 0x1p-30f : 0.f;
+    o.ds = ds;
+    o.cell = W.idx;
+    // advance
+    W.tc = tm;
+    if (p0) { W.t[0] += W.d[0]; W.idx += W.ss[0]; }
+    if (p1) { W.t[1] += W.d[1]; W.idx += W.ss[1]; }
+    if (p2) { W.t[2] += W.d[2]; W.idx += W.ss[2]; }
     // prefetch of the next cell: from a cell inside the grid every crossing (also a diagonal
     // one) lands inside the padded layout
-    const Cell ncell = out ? cell_zero<Cell>() : load_cell(cells + nidx);
-    // deposit in the current cell (segments of length <= 0 deposit nothing)
-    const bool seg = !out && o.ds > 0.f;
-    const float ds = seg ? o.ds : 0.f;
+    const Cell ncell = out ? cell_zero<Cell>() : load_cell(cells + W.idx);
     const float x = chi_of(W.cell) * ds;
-    o.cell = W.idx;
     o.seg = seg;
     o.Lin = W.L;
     o.dtau = x;
@@ -461,15 +489,6 @@ __device__ __forceinline__ StepOut walk_step(WalkT<Cell>& W, bool splits, df rma
     }
     o.end = out || drop || split;
     o.ev = out ? EV_EXIT : (drop ? EV_DROP : (split ? EV_SPLIT : EV_NONE));
-    // advance: the earliest axis by select, further tied axes on the side path
-    const df dsel = {p0 ? W.d[0].hi : (p1 ? W.d[1].hi : W.d[2].hi),
-                     p0 ? W.d[0].lo : (p1 ? W.d[1].lo : W.d[2].lo)};
-    const df tn = df_add(tm, dsel);
-    W.t[0] = df_sel(p0, tn, W.t[0]);
-    W.t[1] = df_sel(p1, tn, W.t[1]);
-    W.t[2] = df_sel(p2, tn, W.t[2]);
-    W.tc = tm;
-    W.idx = nidx;
     W.cell = ncell;
     return o;
 }
@@ -571,21 +590,25 @@ __device__ __forceinline__ void tally_flush(DevStats* st)
 // did not split (each parent owns four consecutive child slots, so fronts keep pixel order).
 constexpr unsigned kHole = 0xffffffffu;
 
-// With a d_max cutoff: where a ray of a level with split radius rmax ends, and whether it
-// splits there. A ray that can split ends at min(rmax, d_max); at equal radii the cut wins.
-__device__ __forceinline__ df end_radius(bool splits, df rmax, df dmax)
+// Where a ray of a level with split radius rmax ends: at rmax if it can split and (kCut) at
+// the d_max cutoff, whichever comes first; at equal radii the cut wins.
+template <bool kCut>
+__device__ __forceinline__ fix end_radius(bool splits, fix rmax, fix dmax)
 {
-    return (splits && !df_le(dmax, rmax)) ? rmax : dmax;
+    const fix r = splits ? rmax : kNoEnd;
+    return kCut ? min(r, dmax) : r;
 }
-__device__ __forceinline__ bool splits_at_end(bool splits, df rmax, df dmax)
+// Whether a ray that reached its end radius splits there (else the cutoff ended it).
+template <bool kCut>
+__device__ __forceinline__ bool splits_at_end(bool splits, fix rmax, fix dmax)
 {
-    return splits && !df_le(dmax, rmax);
+    return !kCut || (splits && rmax < dmax);
 }
 
 // Starts the walk of ray i of level l: loads its record, its source and its direction
 // entry. Returns 1 if the ray starts inside the grid, 0 if it starts outside (it escapes at
 // once), -1 if slot i holds no ray. L0 receives its entering L.
-template <class Cell>
+template <bool kCut, class Cell>
 __device__ __forceinline__ int ray_begin(const TraceArgs& A, const LevelInfo& LV, const RayBuf& B,
                                          int l, unsigned long long i, WalkT<Cell>& W,
                                          const Cell* cells, unsigned& s, unsigned& p, float& L0,
@@ -596,16 +619,21 @@ __device__ __forceinline__ int ray_begin(const TraceArgs& A, const LevelInfo& LV
     p = __ldcg(B.pix + i);
     const float4 sh = __ldg(&A.src[s].hi);
     const float4 sl = __ldg(&A.src[s].lo);
+    const longlong2 xy = __ldg(&A.src[s].xy);
+    const longlong2 z_ = __ldg(&A.src[s].z_);
     L0 = (l == A.level0) ? sh.w : __ldcg(B.L + i);
     const float tau0 = (l == A.level0) ? 0.f : __ldcg(B.tau + i);
     splits = l < __float_as_int(sl.w);
     const float4 e0 = __ldg(LV.dir + 3ull * p);
     const float4 e1 = __ldg(LV.dir + 3ull * p + 1);
-    const float4 e2 = __ldg(LV.dir + 3ull * p + 2);
+    const longlong2 e2 = __ldg(reinterpret_cast<const longlong2*>(LV.dir + 3ull * p + 2));
     const df u[3] = {{sh.x, sl.x}, {sh.y, sl.y}, {sh.z, sl.z}};
+    const fix ux[3] = {xy.x, xy.y, z_.x};
     const df n[3] = {{e0.x, e0.w}, {e0.y, e1.x}, {e0.z, e1.y}};
-    const df inv[3] = {{e1.z, e2.y}, {e1.w, e2.z}, {e2.x, e2.w}};
-    const bool inside = walk_start(W, A.nx, A.ny, A.nz, u, n, inv, LV.r0);
+    const fix code[3] = {(fix)(((unsigned long long)__float_as_uint(e1.w) << 32) | __float_as_uint(e1.z)),
+                         e2.x, e2.y};
+    const bool inside = walk_start(W, A.nx, A.ny, A.nz, A.fbits, u, ux, n, code, LV.r0, LV.r0x);
+    W.rend = end_radius<kCut>(splits, LV.rmaxx, A.dmax);
     W.L = L0;
     W.Lc = 0.f;
     W.tau = tau0;

@@ -39,6 +39,7 @@ struct art_grid {
     long long npad = 0;          // cells of the padded layout (sentinel ring around the grid)
     double lo[3] = {0, 0, 0};
     double dx = 1.0;
+    int fbits = 0;               // fraction bits of the fixed-point distances
     const float* nH0 = nullptr;  // borrowed
     const float* nH = nullptr;   // borrowed, may be NULL
     std::vector<double> pos, L;  // host copies of the sources
@@ -107,6 +108,8 @@ int check_params(const art_params* p);
 int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto);
 int run_opacity(art_grid* g, const art_params* p, bool two_bin);
 double rmax_cells(double m_ray, int level);
+fix to_fix(double cells, int fbits);
+SrcDev source_record(const art_grid* g, const double u[3], double base_L, int lmax);
 int prepare_trace(art_grid* g, const art_params* p, bool adjoint);
 TraceArgs make_args(art_grid* g, const art_params* p);
 int finish_stats(art_grid* g, art_stats* out);

@@ -53,7 +53,7 @@ __device__ __forceinline__ void cossin_pi_frac(long long num, long long den, dou
 
 __global__ void k_directions(int level, unsigned long long npix, double r0, double r1, double r2,
                              double r3, double r4, double r5, double r6, double r7, double r8,
-                             int rotate, float4* __restrict__ dir)
+                             int rotate, double fscale, float4* __restrict__ dir)
 {
     unsigned long long p = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
     if (p >= npix) return;
@@ -93,20 +93,21 @@ __global__ void k_directions(int level, unsigned long long npix, double r0, doub
     } else {
         w[0] = v[0]; w[1] = v[1]; w[2] = v[2];
     }
-    float h[3], l[3], ih[3], il[3];
+    float h[3], l[3];
+    fix d[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (fabs(w[a]) < 5.9604644775390625e-08) w[a] = 0.0;  // 2^-24
         h[a] = __double2float_rn(w[a]);
         l[a] = __double2float_rn(w[a] - (double)h[a]);
-        const double iv = w[a] != 0.0 ? 1.0 / w[a] : 0.0;
-        ih[a] = __double2float_rn(iv);
-        il[a] = __double2float_rn(iv - (double)ih[a]);
+        // distance between faces, 1/|n_a| (fixed-point, fscale = 2^fbits)
+        d[a] = w[a] != 0.0 ? encode_spacing(fscale / fabs(w[a])) : 0;
     }
-    // layout: {n_hx, n_hy, n_hz, n_lx}, {n_ly, n_lz, i_hx, i_hy}, {i_hz, i_lx, i_ly, i_lz}
+    // layout: {n_hx, n_hy, n_hz, n_lx}, {n_ly, n_lz, d_x}, {d_y, d_z}
     dir[3 * p] = make_float4(h[0], h[1], h[2], l[0]);
-    dir[3 * p + 1] = make_float4(l[1], l[2], ih[0], ih[1]);
-    dir[3 * p + 2] = make_float4(ih[2], il[0], il[1], il[2]);
+    dir[3 * p + 1] = make_float4(l[1], l[2], __uint_as_float((unsigned)d[0]),
+                                 __uint_as_float((unsigned)(d[0] >> 32)));
+    *reinterpret_cast<longlong2*>(dir + 3 * p + 2) = make_longlong2(d[1], d[2]);
 }
 
 // chi per cell length (dx) in FP32 from the density fields, in the padded layout with the
@@ -181,7 +182,6 @@ __device__ void run_rays(const TraceArgs& A, const Cell* cells, int l,
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt = (1u << lane) - 1u;
     const LevelInfo& LV = A.levels[l];
-    const df lv_rmax = LV.rmax;  // split radius of this level, kept in registers
     const RayBuf& B = A.buf[l];
     const RayBuf& C = A.buf[l + 1];
     const bool has_next = l < A.lmax_glob;
@@ -217,7 +217,7 @@ __device__ void run_rays(const TraceArgs& A, const Cell* cells, int l,
                 const unsigned rank = __popc(need & lt);
                 if (!active && rank < avail) {
                     slot = wnext + rank;
-                    const int st = ray_begin(A, LV, B, l, slot, W, cells, s, p, L0, splits);
+                    const int st = ray_begin<kCut>(A, LV, B, l, slot, W, cells, s, p, L0, splits);
                     if (st > 0) {
                         active = true;
                         first = base;
@@ -247,13 +247,7 @@ __device__ void run_rays(const TraceArgs& A, const Cell* cells, int l,
             int cell = 0;
             float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
             if (active) {
-                // a ray ends at a radius when it can split or (kCut) at the d_max cutoff
-                StepOut o;
-                if constexpr (kCut)
-                    o = walk_step<false>(W, true, end_radius(splits, lv_rmax, A.dmax), cells,
-                                         A.tau_max);
-                else
-                    o = walk_step<false>(W, splits, lv_rmax, cells, A.tau_max);
+                const StepOut o = walk_step<false>(W, A.fbits, cells, A.tau_max);
                 dep = o.seg;  // segments without length deposit nothing
                 cell = o.cell;
                 const float dm = two ? o.dL + o.dLn : o.dL;  // momentum of both bins
@@ -262,7 +256,7 @@ __device__ void run_rays(const TraceArgs& A, const Cell* cells, int l,
                 if (o.end) {
                     active = false;
                     const unsigned long long c4 = 4ull * (slot - b32);
-                    if (o.ev == EV_SPLIT && (!kCut || splits_at_end(splits, LV.rmax, A.dmax))) {
+                    if (o.ev == EV_SPLIT && splits_at_end<kCut>(splits, LV.rmaxx, A.dmax)) {
                         if (c4 + 4 <= C.cap) {
                             const float Lc = 0.25f * W.L;
                             *reinterpret_cast<uint4*>(C.src + c4) = make_uint4(s, s, s, s);

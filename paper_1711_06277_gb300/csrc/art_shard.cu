@@ -32,21 +32,27 @@ namespace {
 // ends within nx + ny + nz + 2 steps.
 __global__ void k_reach(int nx, int ny, int nz, const float* __restrict__ chi,
                         const SrcDev* __restrict__ src, int nsrc, const float4* __restrict__ dir,
-                        unsigned npix, float tau_max, df dmax, float* __restrict__ reach)
+                        unsigned npix, float tau_max, fix dmax, int fbits,
+                        float* __restrict__ reach)
 {
     const unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
     if (i >= (unsigned long long)nsrc * npix) return;
     const unsigned s = (unsigned)(i / npix), p = (unsigned)(i - (unsigned long long)s * npix);
     const float4 sh = __ldg(&src[s].hi), sl = __ldg(&src[s].lo);
-    const float4 e0 = __ldg(dir + 3ull * p), e1 = __ldg(dir + 3ull * p + 1), e2 = __ldg(dir + 3ull * p + 2);
+    const longlong2 xy = __ldg(&src[s].xy), z_ = __ldg(&src[s].z_);
+    const float4 e0 = __ldg(dir + 3ull * p), e1 = __ldg(dir + 3ull * p + 1);
+    const longlong2 e2 = __ldg(reinterpret_cast<const longlong2*>(dir + 3ull * p + 2));
     const df u[3] = {{sh.x, sl.x}, {sh.y, sl.y}, {sh.z, sl.z}};
+    const fix ux[3] = {xy.x, xy.y, z_.x};
     const df n[3] = {{e0.x, e0.w}, {e0.y, e1.x}, {e0.z, e1.y}};
-    const df inv[3] = {{e1.z, e2.y}, {e1.w, e2.z}, {e2.x, e2.w}};
+    const fix code[3] = {(fix)(((unsigned long long)__float_as_uint(e1.w) << 32) | __float_as_uint(e1.z)),
+                         e2.x, e2.y};
     WalkT<float> W;
-    if (!walk_start(W, nx, ny, nz, u, n, inv, df{0.f, 0.f})) {
+    if (!walk_start(W, nx, ny, nz, fbits, u, ux, n, code, df{0.f, 0.f}, 0)) {
         reach[i] = 0.f;
         return;
     }
+    W.rend = dmax;
     W.L = 0.f;
     W.Lc = 0.f;
     W.tau = 0.f;
@@ -54,11 +60,11 @@ __global__ void k_reach(int nx, int ny, int nz, const float* __restrict__ chi,
     float r = 0.f;
     const int bound = nx + ny + nz + 2;
     for (int k = 0; k < bound; ++k) {
-        const df before = W.tc;
-        const StepOut o = walk_step<true>(W, true, dmax, chi, tau_max);
+        const fix before = W.tc;
+        const StepOut o = walk_step<true>(W, fbits, chi, tau_max);
         if (o.ev == EV_NONE) continue;
         // an exit is seen one step late, in the sentinel cell: the ray left at `before`
-        r = o.ev == EV_EXIT ? before.hi : fminf(W.tc.hi, dmax.hi);
+        r = (float)(o.ev == EV_EXIT ? before : W.tc) * exp2f((float)-fbits);
         break;
     }
     reach[i] = r;
@@ -81,14 +87,9 @@ int art_estimate_work(art_grid* g, const art_params* p, double* h_work)
     // source table (positions in cell units as double-floats)
     std::vector<SrcDev> hs(ns);
     for (int s = 0; s < ns; ++s) {
-        float h[3], lo[3];
-        for (int a = 0; a < 3; ++a) {
-            const double u = (g->pos[3 * s + a] - g->lo[a]) / g->dx;
-            h[a] = (float)u;
-            lo[a] = (float)(u - (double)h[a]);
-        }
-        hs[s].hi = make_float4(h[0], h[1], h[2], 0.f);
-        hs[s].lo = make_float4(lo[0], lo[1], lo[2], 0.f);
+        double u[3];
+        for (int a = 0; a < 3; ++a) u[a] = (g->pos[3 * s + a] - g->lo[a]) / g->dx;
+        hs[s] = source_record(g, u, 0.0, 0);
     }
     if ((rc = ensure_directions(g, p, le, le))) return rc;
     if ((rc = run_opacity(g, p, false))) return rc;
@@ -101,13 +102,10 @@ int art_estimate_work(art_grid* g, const art_params* p, double* h_work)
         e = cudaMemcpyAsync(d_src, hs.data(), sizeof(SrcDev) * ns, cudaMemcpyHostToDevice, g->stream);
     std::vector<float> reach(nray);
     if (e == cudaSuccess) {
-        df dmax;
-        const double dm = p->d_max > 0.0 ? p->d_max / g->dx : 1.0e30;
-        dmax.hi = (float)dm;
-        dmax.lo = (float)(dm - (double)dmax.hi);
+        const fix dmax = p->d_max > 0.0 ? to_fix(p->d_max / g->dx, g->fbits) : kNoEnd;
         k_reach<<<(unsigned)((nray + 255) / 256), 256, 0, g->stream>>>(
             g->n[0], g->n[1], g->n[2], g->d_chi, d_src, ns, g->dir[le], npix, (float)p->tau_max,
-            dmax, d_reach);
+            dmax, g->fbits, d_reach);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
