@@ -70,9 +70,12 @@ typedef struct {
     double rot[9];       /* row-major rotation of the ray directions (with ART_F_ROTATE) */
     unsigned flags;      /* ART_F_* */
     int schedule;        /* ART_SCHED_* */
-    int block_threads;   /* threads per block of the trace kernels (0 = library choice) */
-    int chunk;           /* rays a warp takes from the queue at a time (0 = library choice) */
-    long long queue_capacity; /* rays per level buffer beyond l0 (0 = library choice) */
+    int block_threads;   /* threads per block of the trace kernels (0 = library choice; at most
+                            128 in the forward trace, 256 in the reverse sweep) */
+    int chunk;           /* rays a warp of the reverse sweep takes from the queue at a time
+                            (0 = library choice; the forward trace takes 32 lanes' worth) */
+    long long queue_capacity; /* rays per level buffer beyond l0 (0 = library choice; the
+                            persistent trace holds at least 16) */
     double wait_limit_s; /* bound on any device-side wait (grid barrier); 0 = library default
                             (60 s); a negative value makes every wait give up at once. A
                             block waits at a barrier while the slowest block finishes its

@@ -147,7 +147,8 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
     float total = 0.f;     // own + descendants (pass 2), passed to the parent
     df rem = {0.f, 0.f};   // weighted sum over what follows the current segment (pass 2)
     bool splits = false;
-    unsigned ncross = 0, nrays = 0;
+    fix rend = kNoEnd;     // radius where the ray of level lv ends (split or cutoff)
+    unsigned ncross = 0, nrays = 0, nstep = 0;
     // Every step crosses at least one face and the sentinel ring ends every walk that
     // leaves the grid, so walks end by construction. As a safety net the warp counts its
     // rounds of steps (ART_ADJ_STEPS each) and gives up past a bound far beyond any phase
@@ -180,7 +181,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
             rem = df_add(own, {__ldcg(Pl.sub + slot), 0.f});
             total = rem.hi + rem.lo;
             const LevelInfo Lp = A.levels[lv];
-            ray_begin<kCut>(A, Lp, Pl, lv, slot, W, recs, s, p, L0, splits);
+            ray_begin<kCut>(A, Lp, Pl, lv, slot, W, recs, s, p, L0, splits, rend);
             Ls = __ldg(A.srcL + s);
             mode = 2;
             return;
@@ -204,7 +205,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
                 if (mode == 0 && rank < avail) {
                     slot = wnext + rank;
                     lv = l;
-                    const int st = ray_begin<kCut>(A, LV, B, l, slot, W, recs, s, p, L0, splits);
+                    const int st = ray_begin<kCut>(A, LV, B, l, slot, W, recs, s, p, L0, splits, rend);
                     if (st > 0) {
                         Ls = __ldg(A.srcL + s);
                         t0[0] = W.t[0];
@@ -245,7 +246,7 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
                 const float wv = cm.z;   // weight and neutral-H opacity of this cell
                 const float hv = cm.y;
                 const float q = force_weight(W.cell, W.n, A.fscale);
-                const StepOut o = walk_step<false, true>(W, A.fbits, recs, A.tau_max);
+                const StepOut o = walk_step(W, rend, A.unit, (int)A.npad, recs, A.tau_max, nstep);
                 // this segment's loss: w k G, plus q dL with a force term
                 const float g = fmaf(q, o.dL, wv * gs * o.G);
                 if (mode == 1) {
@@ -295,7 +296,6 @@ __device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* curso
                             W.idx = idx0;
                             W.tc = LV.r0x;
                             W.L = L0;
-                            W.Lc = 0.f;
                             W.tau = l == A.level0 ? 0.f : __ldcg(B.tau + slot);
                             W.cell = load_cell(recs + idx0);
                             mode = 2;
@@ -517,16 +517,16 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     // without dust the neutral-H opacity is the opacity: an 8-byte record serves
     const bool light = !d_v && sd_dx == 0.0;
     if (light) {
-        if (!g->d_recw && (rc = status_of(cudaMalloc((void**)&g->d_recw, sizeof(CellW) * g->npad))))
+        if (!g->d_recw && (rc = status_of(cudaMalloc((void**)&g->d_recw, sizeof(CellW) * (g->npad + 1)))))
             return rc;
         k_pack_cells_w<<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, sH_dx, d_w, g->d_recw);
     } else if (d_v) {
-        if (!g->d_recf && (rc = status_of(cudaMalloc((void**)&g->d_recf, sizeof(CellF) * g->npad))))
+        if (!g->d_recf && (rc = status_of(cudaMalloc((void**)&g->d_recf, sizeof(CellF) * (g->npad + 1)))))
             return rc;
         k_pack_cells_f<<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH_dx, sd_dx, d_w,
                                                     d_v, g->d_recf);
     } else {
-        if (!g->d_rec && (rc = status_of(cudaMalloc((void**)&g->d_rec, sizeof(float4) * g->npad))))
+        if (!g->d_rec && (rc = status_of(cudaMalloc((void**)&g->d_rec, sizeof(float4) * (g->npad + 1)))))
             return rc;
         k_pack_cells<<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH_dx, sd_dx, d_w,
                                                   g->d_rec);

@@ -158,6 +158,51 @@ int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto)
     return ART_OK;
 }
 
+// Front of level l with room for `need` rays of a reverse sweep.
+static int ensure_adjoint_front(art_grid* g, int l, unsigned long long need)
+{
+    RayBuf& b = g->buf[l];
+    if (need > g->buf_cap[l]) {
+        dev_free(b.src); dev_free(b.pix); dev_free(b.L); dev_free(b.tau);
+        dev_free(b.parent); dev_free(b.own); dev_free(b.sub); dev_free(b.pending);
+        b = RayBuf{};
+        g->buf_cap[l] = 0;
+        int rc = dev_alloc(&b.src, need);
+        if (!rc) rc = dev_alloc(&b.pix, need);
+        if (!rc) rc = dev_alloc(&b.L, need);
+        if (!rc) rc = dev_alloc(&b.tau, need);
+        if (!rc) rc = dev_alloc(&b.parent, need);
+        if (!rc) rc = dev_alloc(&b.own, need);
+        if (!rc) rc = dev_alloc(&b.sub, need);
+        if (!rc) rc = dev_alloc(&b.pending, need);
+        if (rc) return rc;
+        g->buf_cap[l] = need;
+    }
+    b.cap = need;  // the capacity this sweep may use
+    return ART_OK;
+}
+
+// Front of level l with room for `need` quads of a forward trace.
+static int ensure_quads(art_grid* g, int l, unsigned long long need, bool two_bin)
+{
+    QuadBuf& q = g->quad[l];
+    if (need > g->quad_cap[l]) {
+        dev_free(q.rec);
+        dev_free(q.recn);
+        q = QuadBuf{};
+        g->quad_cap[l] = 0;
+        const int rc = dev_alloc(&q.rec, need);
+        if (rc) return rc;
+        g->quad_cap[l] = need;
+    }
+    if (two_bin && !q.recn) {
+        const int rc = dev_alloc(&q.recn, g->quad_cap[l]);
+        if (rc) return rc;
+    }
+    q.cap = need;  // the capacity this trace may use
+    return ART_OK;
+}
+
 // Source table, per-source l_max, direction tables, level constants and ray buffers for a
 // trace with parameters p. Allocates only when something grew or changed.
 int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
@@ -221,7 +266,7 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
                                     cudaMemcpyHostToDevice, g->stream));
         }
         if (!g->d_chi2) {
-            int rc = dev_alloc(&g->d_chi2, g->npad);
+            int rc = dev_alloc(&g->d_chi2, g->npad + 1);
             if (rc) return rc;
         }
     }
@@ -248,53 +293,26 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         ART_TRY(cudaMemcpyAsync(g->d_levels, g->h_levels, sizeof(lv), cudaMemcpyHostToDevice,
                                 g->stream));
     }
-    // --- ray buffers: level l0 holds every base ray of the batch; deeper levels hold at
-    // most the queue capacity (persistent) or one source's whole front (plain)
+    // --- fronts: deeper levels hold at most the queue capacity (persistent) or one source's
+    // whole front (plain); the base level of a forward trace needs no storage
     const bool plain = p->schedule == ART_SCHED_PLAIN;
-    long long qcap = p->queue_capacity > 0 ? p->queue_capacity : (64ll << 20);
+    const long long qcap = p->queue_capacity > 0 ? p->queue_capacity : (64ll << 20);
     for (int l = l0; l <= lmax_glob; ++l) {
         unsigned long long need;
         const unsigned long long front = 12ull << (2 * l);  // rays of one source at level l
-        if (l == l0) need = plain ? npix0 : (unsigned long long)ns * npix0;
+        if (l == l0) need = (unsigned long long)ns * npix0;
         else if (plain) need = p->queue_capacity > 0 ? (unsigned long long)qcap : front;
         else need = std::min<unsigned long long>((unsigned long long)qcap, (unsigned long long)ns * front);
         need = (need + 3) & ~3ull;
-        const bool want_adj = adjoint && !g->buf_adj[l];
-        const bool want_2bin = g->two_bin && !adjoint && !g->buf_2bin[l];
-        if (need > g->buf_cap[l] || want_adj || want_2bin) {
-            RayBuf& b = g->buf[l];
-            dev_free(b.src); dev_free(b.pix); dev_free(b.L); dev_free(b.tau);
-            dev_free(b.Ln); dev_free(b.taun);
-            dev_free(b.parent); dev_free(b.own); dev_free(b.sub); dev_free(b.pending);
-            b = RayBuf{};
-            g->buf_cap[l] = 0;
-            const unsigned long long cap = std::max(need, g->buf_cap_req[l]);
-            int rc = dev_alloc(&b.src, cap);
-            if (!rc) rc = dev_alloc(&b.pix, cap);
-            if (!rc) rc = dev_alloc(&b.L, cap);
-            if (!rc) rc = dev_alloc(&b.tau, cap);
-            if (!rc && (adjoint || g->buf_adj[l])) {
-                rc = dev_alloc(&b.parent, cap);
-                if (!rc) rc = dev_alloc(&b.own, cap);
-                if (!rc) rc = dev_alloc(&b.sub, cap);
-                if (!rc) rc = dev_alloc(&b.pending, cap);
-                g->buf_adj[l] = true;
-            }
-            if (!rc && ((g->two_bin && !adjoint) || g->buf_2bin[l])) {
-                rc = dev_alloc(&b.Ln, cap);
-                if (!rc) rc = dev_alloc(&b.taun, cap);
-                g->buf_2bin[l] = true;
-            }
-            if (rc) return rc;
-            g->buf_cap[l] = cap;
-            g->buf_cap_req[l] = cap;
+        int rc = ART_OK;
+        if (adjoint) {
+            rc = ensure_adjoint_front(g, l, need);
+        } else if (l > l0) {
+            // in the persistent schedule a phase takes a quarter of the next front's quads
+            const unsigned long long quads = plain ? need / 4 : std::max(need / 4, 4ull);
+            rc = ensure_quads(g, l, quads, g->two_bin);
         }
-        g->buf[l].cap = need;  // the capacity this trace may use
-    }
-    for (int l = lmax_glob + 1; l < kNL; ++l) {
-        RayBuf keep = g->buf[l];
-        keep.cap = 0;
-        g->buf[l] = keep;
+        if (rc) return rc;
     }
     g->prep_valid = true;
     g->prep_version = g->src_version;
@@ -329,6 +347,7 @@ TraceArgs make_args(art_grid* g, const art_params* p)
     // the d_max cutoff (read only by the kernels built for a cutoff)
     A.dmax = p->d_max > 0.0 ? to_fix(p->d_max / g->dx, g->fbits) : kNoEnd;
     A.fbits = g->fbits;
+    A.unit = (float)std::ldexp(1.0, -g->fbits);
     A.nx = g->n[0];
     A.ny = g->n[1];
     A.nz = g->n[2];
@@ -342,7 +361,14 @@ TraceArgs make_args(art_grid* g, const art_params* p)
     A.acc = g->d_acc;
     A.src = g->d_src;
     A.levels = g->d_levels;
-    for (int l = 0; l < kNL; ++l) A.buf[l] = g->buf[l];
+    for (int l = 0; l < kNL; ++l) {
+        A.buf[l] = g->buf[l];
+        A.quad[l] = g->quad[l];
+        if (l > g->lmax_glob) A.buf[l].cap = A.quad[l].cap = 0;
+    }
+    A.base_quads = 3u << (2 * p->level0);
+    A.nsrc = (unsigned)g->L.size();
+    A.npad = (unsigned)g->npad;
     A.sched = g->d_sched;
     A.stats = g->d_stats;
     double ws = p->wait_limit_s == 0.0 ? kDefaultWaitS : p->wait_limit_s;
@@ -430,7 +456,7 @@ int art_create_grid(art_grid** out, int nx, int ny, int nz, const double box_lo[
     g->stream = (cudaStream_t)stream;
     int rc = cuda_status(cudaGetDevice(&g->device));
     if (!rc) rc = cuda_status(cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device));
-    if (!rc) rc = dev_alloc(&g->d_chi, npad);
+    if (!rc) rc = dev_alloc(&g->d_chi, npad + 1);
     if (!rc) rc = dev_alloc(&g->d_acc, npad);
     if (!rc) rc = dev_alloc(&g->d_levels, kNL);
     if (!rc) rc = dev_alloc(&g->d_sched, 1);
@@ -516,9 +542,8 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     ART_TRY(cudaMemsetAsync(g->d_sched, 0, sizeof(Sched), g->stream));
     const int ns = (int)g->L.size();
     const int l0 = p->level0;
-    const unsigned npix0 = 12u << (2 * l0);
-    // block size: the caller's (or 256), at most what the trace kernels are built for
-    const int threads = std::min(p->block_threads > 0 ? p->block_threads : 256, kTraceMaxThreads);
+    // block size: the caller's (or 128), at most what the trace kernels are built for
+    const int threads = std::min(p->block_threads > 0 ? p->block_threads : 128, kTraceMaxThreads);
     TraceArgs A = make_args(g, p);
     if (p->schedule == ART_SCHED_PLAIN) {
         int per_sm = 0;
@@ -530,17 +555,11 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
         const int grid = per_sm * g->sms;
         for (int s = 0; s < ns; ++s) {
             k_reset_counts<<<1, 32, 0, g->stream>>>(g->d_sched);
-            k_inject<<<(npix0 + 255) / 256, 256, 0, g->stream>>>(s, 1, npix0, g->buf[l0],
-                                                                  &g->d_sched->count[l0]);
             for (int l = l0; l <= g->src_lmax[s]; ++l)
-                kern<<<grid, threads, 0, g->stream>>>(A, l);
+                kern<<<grid, threads, 0, g->stream>>>(A, l, (unsigned)s);
         }
         ART_TRY(cudaGetLastError());
     } else {
-        unsigned long long nb = (unsigned long long)ns * npix0;
-        k_inject<<<(unsigned)((nb + 255) / 256), 256, 0, g->stream>>>(0, ns, npix0, g->buf[l0],
-                                                                     &g->d_sched->count[l0]);
-        ART_TRY(cudaGetLastError());
         int per_sm = 0;
         const bool cut = p->d_max > 0.0;
         auto kern = g->two_bin
@@ -611,9 +630,10 @@ void art_destroy_grid(art_grid* g)
     dev_free(g->d_dL_scratch);
     for (int l = 0; l < kNL; ++l) {
         dev_free(g->dir[l]);
+        dev_free(g->quad[l].rec);
+        dev_free(g->quad[l].recn);
         RayBuf& b = g->buf[l];
         dev_free(b.src); dev_free(b.pix); dev_free(b.L); dev_free(b.tau);
-        dev_free(b.Ln); dev_free(b.taun);
         dev_free(b.parent); dev_free(b.own); dev_free(b.sub); dev_free(b.pending);
     }
     if (g->h_stats) cudaFreeHost(g->h_stats);

@@ -124,19 +124,24 @@ struct LevelInfo {
     unsigned long long destroy_w;  // 4^(l_max_global - l)
 };
 
-// SoA ray buffer of one level: source index, nested pixel, entering L and tau.
+// Adjoint fronts, SoA per level: source index, nested pixel, entering L and tau.
 struct RayBuf {
     unsigned* src;
     unsigned* pix;
     float* L;
     float* tau;
-    float* Ln;          // two-bin traces: entering L and tau of the non-ionizing bin
-    float* taun;
-    // adjoint extras (NULL in forward traces)
     unsigned* parent;   // slot of the parent in the level above
     float2* own;        // weighted sum over the ray's own segments (pass 1), double-float
     float* sub;         // weighted sum over the ray's descendants (added by the children)
     unsigned* pending;  // children of a split ray still to finish
+    unsigned long long cap;
+};
+
+// Forward fronts: one record per quad, the four children of a split ray, {source, pixel of
+// the first child, entering L of each child (bits), tau (bits)}; two-bin traces add {Ln, taun}.
+struct QuadBuf {
+    uint4* rec;
+    float2* recn;
     unsigned long long cap;
 };
 
@@ -162,7 +167,7 @@ struct Sched {
     unsigned long long count[kNL];   // rays held in the level buffer (a stack, top = count)
     unsigned long long cursor[kNL];  // next ray of the current phase / launch
     unsigned long long phase_begin, phase_end;
-    int phase_level, phase_kind, done, pad;
+    int phase_level, phase_width, phase_strided, done, started, pad;
     unsigned bar_count, bar_gen;
 };
 
@@ -185,7 +190,11 @@ struct TraceArgs {
     float4* acc;             // per-cell accumulator (sum L ds phi, sum dL n), padded
     const SrcDev* src;
     const LevelInfo* levels;
-    RayBuf buf[kNL];
+    RayBuf buf[kNL];         // adjoint fronts
+    QuadBuf quad[kNL];       // forward fronts (levels beyond l0)
+    unsigned base_quads;     // quads of level l0 per source (3 * 4^l0)
+    unsigned nsrc;
+    unsigned npad;           // cells of the padded layout; cell npad is the end marker
     Sched* sched;
     DevStats* stats;
     long long wait_ns;       // bound of a grid-barrier wait (<0: give up at once)
@@ -196,6 +205,7 @@ struct TraceArgs {
     fix dmax;                // d_max cutoff (kernels built for a cutoff only)
     float fscale;            // adjoint: force per unit momentum (1 / dV)
     int fbits;               // fraction bits of the fixed-point distances
+    float unit;              // 2^-fbits, their unit in cells
 };
 
 enum : int { EV_NONE = 0, EV_EXIT = 1, EV_DROP = 2, EV_SPLIT = 3 };
@@ -242,24 +252,22 @@ template <> __device__ __forceinline__ CellF cell_zero<CellF>()
     return {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
 }
 
-template <class Cell>
-struct WalkT {
+// Where a ray is on its way through the grid.
+struct Path {
     fix t[3];     // distance from the source to the next face on each axis
     fix d[3];     // distance between consecutive faces on each axis (1/|n_a|)
     fix tc;       // distance of the current position
-    fix rend;     // radius where the ray ends (split or cutoff), kNoEnd if at none
     int idx;      // index of the current cell in the padded layout (sentinel ring around
                   // the grid, see pad_index)
     int ss[3];    // signed index step of a crossing on each axis
+};
+
+template <class Cell>
+struct WalkT : Path {
     float n[3];   // direction (hi parts) for momentum deposits
     float L, tau;
-    float Lc;        // photon ledger: the rounding error of this walk's L updates (see
-                     // walk_step); tallied with the ray, never used for deposits
-    float Ln, taun;  // non-ionizing bin (two-bin traces only)
-    float Lnc;       // the same compensation for Ln
     Cell cell;    // record of the current cell (prefetched)
 };
-using Walk = WalkT<float>;
 
 // Cell records are stored with a ring of sentinel cells around the nx*ny*nz grid (opacity
 // < 0): cell (i, j, k) sits at (i + 1) + (nx + 2) ((j + 1) + (ny + 2) (k + 1)). A ray leaves
@@ -271,6 +279,7 @@ __host__ __device__ __forceinline__ long long pad_index(long long i, long long j
     return (i + 1) + (long long)(nx + 2) * ((j + 1) + (long long)(ny + 2) * (k + 1));
 }
 constexpr float kSentinel = -1.0f;
+constexpr float kEnded = -2.0f;  // opacity of the end marker, the cell after the padded layout
 
 // Coordinates of padded cell q (see pad_index; padded grids hold fewer than 2^31 cells):
 // false for the sentinel ring, else the cell's index in the caller's nx*ny*nz layout.
@@ -292,11 +301,10 @@ __device__ __forceinline__ unsigned pad_of(unsigned i, int nx, int ny)
     return (unsigned)pad_index(x, r % (unsigned)ny, r / (unsigned)ny, nx, ny);
 }
 
-// Sets up the walk of a ray with direction n (df) and face spacing codes (both from the
+// Sets up the path of a ray with direction n (df) and face spacing codes (both from the
 // direction table) from source position u (df, and ux fixed-point) starting at radius r0.
 // Returns false if the start point lies outside the grid.
-template <class Cell>
-__device__ __forceinline__ bool walk_start(WalkT<Cell>& W, int nx, int ny, int nz, int fbits,
+__device__ __forceinline__ bool path_start(Path& W, int nx, int ny, int nz, int fbits,
                                            const df u[3], const fix ux[3], const df n[3],
                                            const fix code[3], df r0, fix r0x)
 {
@@ -311,7 +319,6 @@ __device__ __forceinline__ bool walk_start(WalkT<Cell>& W, int nx, int ny, int n
         if (p.hi == f && (p.lo < 0.f || (p.lo == 0.f && n[a].hi < 0.f))) ci -= 1;
         c[a] = ci;
         inside = inside && ci >= 0 && ci < N[a];
-        W.n[a] = n[a].hi;
         const bool up = n[a].hi > 0.f, flat = n[a].hi == 0.f;
         const int stride = a == 0 ? 1 : (a == 1 ? nx + 2 : (nx + 2) * (ny + 2));
         W.ss[a] = flat ? 0 : (up ? stride : -stride);
@@ -327,24 +334,16 @@ __device__ __forceinline__ bool walk_start(WalkT<Cell>& W, int nx, int ny, int n
 
 // Outcome of one crossing step: the deposit to make (in cell, when seg) and the event.
 struct StepOut {
-    int cell;     // the cell the segment lies in (padded layout)
+    int cell;     // the cell the segment lies in (padded layout), negative without a segment
     bool seg;     // the segment has positive length: deposit and count it
-    bool end;     // the ray ends with this step (ev != EV_NONE)
     float ds;     // segment length (cell units), > 0 when seg
-    float dtau;
     float Lin;
     float G;      // L_in ds phi(dtau)
     float dL;     // L_in (1 - e^-dtau)
-    float phi;    // (1 - e^-dtau)/dtau
-    float dphi;   // d phi / d dtau (filled by walk_step<kCountOnly, true> only)
-    float dLn;    // two-bin traces: loss of the non-ionizing bin (chi_n = n_H sigma_d)
+    float dphi;   // d phi / d dtau
     int ev;
 };
 
-// (1 - e^-x)/x for x >= 0. Below 1 as e^{-x/2} sinh(x/2)/(x/2), the even series of
-// sinh(y)/y to y^8 (truncation < 3e-11 for y < 1/2, no cancellation); above 1 as
-// (1 - e^{-x})/x with e^{-x} = (e^{-x/2})^2. One exponential serves both branches, which are
-// evaluated and selected, so lanes never diverge here.
 __device__ __forceinline__ float ex2_ftz(float v)
 {
     float r;
@@ -359,18 +358,52 @@ __device__ __forceinline__ float rcp_ftz(float v)
 }
 constexpr float kHalfLog2e = 0.72134752f;  // log2(e) / 2: e^{-x/2} = 2^{-x kHalfLog2e}
 
-__device__ __forceinline__ float phi_of(float x)
+// Arithmetic on the values of one ray (float) or of two rays side by side (float2, which this
+// part adds and multiplies in one instruction).
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b)
 {
-    const float y = 0.5f * x;
-    const float E = ex2_ftz(-kHalfLog2e * x);
-    const float y2 = y * y;
-    float S = fmaf(y2, 1.f / 362880.f, 1.f / 5040.f);
-    S = fmaf(S, y2, 1.f / 120.f);
-    S = fmaf(S, y2, 1.f / 6.f);
-    S = fmaf(S, y2, 1.f);
-    const float small = E * S;
-    const float large = fmaf(-E, E, 1.f) * rcp_ftz(fmaxf(x, 1.f));
-    return x < 1.f ? small : large;
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);  // exact product: one rounding
+}
+template <class V> __device__ __forceinline__ V vset(float v);
+template <> __device__ __forceinline__ float vset<float>(float v) { return v; }
+template <> __device__ __forceinline__ float2 vset<float2>(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float vex2(float v) { return ex2_ftz(v); }
+__device__ __forceinline__ float2 vex2(float2 v) { return make_float2(ex2_ftz(v.x), ex2_ftz(v.y)); }
+__device__ __forceinline__ float vrcp_max1(float v) { return rcp_ftz(fmaxf(v, 1.f)); }
+__device__ __forceinline__ float2 vrcp_max1(float2 v)
+{
+    return make_float2(rcp_ftz(fmaxf(v.x, 1.f)), rcp_ftz(fmaxf(v.y, 1.f)));
+}
+__device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ float2 vmax(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
+__device__ __forceinline__ float& vget(float& v, int) { return v; }
+__device__ __forceinline__ float& vget(float2& v, int j) { return j ? v.y : v.x; }
+__device__ __forceinline__ float vget(const float& v, int) { return v; }
+__device__ __forceinline__ float vget(const float2& v, int j) { return j ? v.y : v.x; }
+
+// phi(x) = (1 - e^-x)/x for x >= 0. Below 1 as E sinh(y)/y with y = x/2 and E = e^{-y}, the even
+// series of sinh(y)/y to y^8 (truncation < 3e-11 for y < 1/2, no cancellation); above 1 as
+// (1 - E^2)/x. One exponential serves both. The first form falls below phi above 1 (its series
+// is cut short; NaN where it overflows against E = 0) and the second, with x replaced by
+// max(x, 1), falls below phi below 1, so phi is the larger of the two and lanes never diverge.
+template <class V>
+__device__ __forceinline__ V phi_of(V x)
+{
+    const V E = vex2(vmul(x, vset<V>(-kHalfLog2e)));
+    const V x2 = vmul(x, x);
+    V S = vfma(x2, vset<V>(1.f / 92897280.f), vset<V>(1.f / 322560.f));
+    S = vfma(S, x2, vset<V>(1.f / 1920.f));
+    S = vfma(S, x2, vset<V>(1.f / 24.f));
+    S = vfma(S, x2, vset<V>(1.f));
+    const V large = vmul(vfma(vmul(E, vset<V>(-1.f)), E, vset<V>(1.f)), vrcp_max1(x));
+    return vmax(vmul(E, S), large);
 }
 
 // phi(x) and phi'(x) from the same exponential (the reverse sweep needs both). Below 1, with
@@ -397,115 +430,160 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
     return sm ? E * S : large;
 }
 
-// One step of the walk: the segment from tc to the next face or to the end radius. The
-// common case (one axis crossing) runs without branches; faces crossed together (ties) take
-// a short side path. When the step ends the ray (event other than EV_NONE) the walk state
-// other than L and tau is left unspecified.
-template <bool kCountOnly, bool kDphi = false, class Cell>
-__device__ __forceinline__ StepOut walk_step(WalkT<Cell>& W, int fbits,
-                                             const Cell* __restrict__ cells, float tau_max)
+// The geometric part of a step: the segment from tc to the next face or to the end radius
+// rend (split or cutoff, kNoEnd if at none), and the advance of the walk to its end; at rend
+// the next cell is the end marker npad. ds is the length (cell units; unit = 2^-fbits) and key
+// the cell of the segment, 0 and `none` where there is nothing to deposit: the length is not
+// positive or the ray has ended (chi < 0, or depth > limit). Deposits are counted in ncross;
+// x is chi ds. walk_move_load also replaces chi by the opacity at the start of the next
+// cell's record, unless the ray has ended.
+//
+// The earliest of the three faces and the end radius is decided on the high words (2^-19
+// cells at 512^3): different high words order the distances exactly. Equal ones (exact ties,
+// near ties, a face at the end radius), and segments too short to show in the high words,
+// take the exact 64-bit comparison on the side path, where axes that cross within 2^-40 of
+// the distance of the earliest one step together (a diagonal step). Two distances within that
+// tolerance can still have different high words when they straddle a boundary; the walk then
+// crosses the two faces in two steps with a segment far below the 1e-5-cell near-tie
+// threshold between them, a ray the oracle flags as near-tie.
+//
+// Written in PTX because the predicates of the choice then also predicate the advance: from
+// C++ the compiler made branches of it (15 per ray and step instead of the one for ties,
+// 97.0 against 65.7 ms on 256^3 / 64 sources). The side path finishes the move by itself:
+// joined before the advance, with the predicates of both paths, every step paid 18 more
+// instructions (14.3 against 12.2 ms on 256^3 / 16 sources).
+//   operands: 0-2 t, 3 tc, 4 idx, 5 ncross, 6 ds, 7 key, 8 x, 9 chi, 10-12 d, 13-15 ss,
+//   16 rend, 17 unit, 18 none, 19 npad, 20 depth, 21 limit
+#define ART_MOVE_ADVANCE \
+    "sub.s64 mv, m, %3;\n\t" \
+    "mov.b64 %3, m;\n\t" \
+    "cvt.rn.f32.s64 %6, mv;\n\t" \
+    "mul.f32 %6, %6, %17;\n\t" \
+    "selp.f32 %6, %6, 0f00000000, pa;\n\t" \
+    "mul.f32 %8, %9, %6;\n\t" \
+    "selp.b32 %7, %4, %18, pa;\n\t" \
+    "@pa add.u32 %5, %5, 1;\n\t" \
+    "@p0 add.s64 %0, %0, %10;\n\t" \
+    "@p1 add.s64 %1, %1, %11;\n\t" \
+    "@p2 add.s64 %2, %2, %12;\n\t" \
+    "@p0 add.s32 %4, %4, %13;\n\t" \
+    "@p1 add.s32 %4, %4, %14;\n\t" \
+    "@p2 add.s32 %4, %4, %15;\n\t" \
+    "@ps mov.b32 %4, %19;\n\t"
+#define ART_MOVE_PTX \
+    "{\n\t" \
+    ".reg .pred p0, p1, p2, ps, ta, tb, tc, po, pa;\n\t" \
+    ".reg .b32 l0, l1, l2, lr, h0, h1, h2, hr, hm, lm, cl, ch;\n\t" \
+    ".reg .b64 m, tol, d, mv, at;\n\t" \
+    "mov.b64 {l0, h0}, %0;\n\t" \
+    "mov.b64 {l1, h1}, %1;\n\t" \
+    "mov.b64 {l2, h2}, %2;\n\t" \
+    "mov.b64 {lr, hr}, %16;\n\t" \
+    "mov.b64 {cl, ch}, %3;\n\t" \
+    "setp.geu.f32 po, %9, 0f00000000;\n\t" \
+    "setp.leu.and.f32 po, %20, %21, po;\n\t" \
+    "min.s32 hm, h0, h1;\n\t" \
+    "min.s32 hm, hm, h2;\n\t" \
+    "min.s32 hm, hm, hr;\n\t" \
+    "setp.eq.s32 p0, h0, hm;\n\t" \
+    "setp.eq.s32 p1, h1, hm;\n\t" \
+    "setp.eq.s32 p2, h2, hm;\n\t" \
+    "setp.eq.s32 ps, hr, hm;\n\t" \
+    "and.pred ta, p0, p1;\n\t" \
+    "or.pred tb, p0, p1;\n\t" \
+    "and.pred tc, tb, p2;\n\t" \
+    "or.pred ta, ta, tc;\n\t" \
+    "or.pred tb, tb, p2;\n\t" \
+    "and.pred tc, tb, ps;\n\t" \
+    "or.pred ta, ta, tc;\n\t" \
+    "setp.le.or.s32 ta, hm, ch, ta;\n\t" \
+    "and.pred ta, ta, po;\n\t" \
+    "@ta bra tie_%=;\n\t" \
+    "selp.b32 lm, l2, lr, p2;\n\t" \
+    "selp.b32 lm, l1, lm, p1;\n\t" \
+    "selp.b32 lm, l0, lm, p0;\n\t" \
+    "mov.b64 m, {lm, hm};\n\t" \
+    "mov.pred pa, po;\n\t" \
+    ART_MOVE_ADVANCE \
+    "bra moved_%=;\n\t" \
+    "tie_%=:\n\t" \
+    "min.s64 m, %0, %1;\n\t" \
+    "min.s64 m, m, %2;\n\t" \
+    "shr.s64 tol, m, 40;\n\t" \
+    "sub.s64 d, %0, m;\n\t" \
+    "setp.le.s64 p0, d, tol;\n\t" \
+    "sub.s64 d, %1, m;\n\t" \
+    "setp.le.s64 p1, d, tol;\n\t" \
+    "sub.s64 d, %2, m;\n\t" \
+    "setp.le.s64 p2, d, tol;\n\t" \
+    "setp.le.s64 ps, %16, m;\n\t" \
+    "selp.b64 m, %16, m, ps;\n\t" \
+    "setp.gt.and.s64 pa, m, %3, po;\n\t" \
+    ART_MOVE_ADVANCE \
+    "moved_%=:\n\t"
+#define ART_MOVE_OPERANDS                                                                      \
+        : "+l"(W.t[0]), "+l"(W.t[1]), "+l"(W.t[2]), "+l"(W.tc), "+r"(W.idx), "+r"(ncross),     \
+          "=&f"(ds), "=&r"(key), "=&f"(x), "+f"(chi)                                           \
+        : "l"(W.d[0]), "l"(W.d[1]), "l"(W.d[2]), "r"(W.ss[0]), "r"(W.ss[1]), "r"(W.ss[2]),     \
+          "l"(rend), "f"(unit), "r"(none), "r"(npad), "f"(depth), "f"(limit)
+
+__device__ __forceinline__ void walk_move(Path& W, fix rend, float unit, float chi, float depth,
+                                          float limit, int none, int npad, float& ds, float& x,
+                                          int& key, unsigned& ncross)
+{
+    asm(ART_MOVE_PTX "}" ART_MOVE_OPERANDS);
+}
+
+template <class Cell>
+__device__ __forceinline__ void walk_move_load(Path& W, fix rend, float unit, float& chi,
+                                               float depth, float limit, int none, int npad,
+                                               const Cell* cells, float& ds, float& x, int& key,
+                                               unsigned& ncross)
+{
+    asm(ART_MOVE_PTX
+        "mad.wide.s32 at, %4, %22, %23;\n\t"
+        "@po ld.global.nc.f32 %9, [at];\n\t"
+        "}"
+        ART_MOVE_OPERANDS, "n"((int)sizeof(Cell)), "l"(cells));
+}
+
+// One step of a walk of the reverse sweep (and of the work estimate, which passes L = 0): the
+// segment, its attenuation and the next cell's record. When the step ends the ray (event other
+// than EV_NONE) the walk state other than L and tau is left unspecified.
+template <class Cell>
+__device__ __forceinline__ StepOut walk_step(WalkT<Cell>& W, fix rend, float unit, int npad,
+                                             const Cell* __restrict__ cells, float tau_max,
+                                             unsigned& ncross)
 {
     StepOut o;
     // A step that starts in a sentinel cell ends the ray: it left the grid with the crossing
     // of the previous step (whose segment was deposited then); nothing is deposited now.
     const bool out = chi_of(W.cell) < 0.f;
-    // Earliest of the three faces and the end radius, decided on the high words (2^-19 cells
-    // at 512^3): different high words order the distances exactly. Equal ones (exact ties,
-    // near ties, a face at the end radius) take the exact 64-bit comparison below. Two
-    // distances within the 1e-12 tie tolerance can still have different high words when they
-    // straddle a boundary; the walk then crosses the two faces in two steps with a segment
-    // far below the 1e-5-cell near-tie threshold between them, a ray the oracle flags as
-    // near-tie.
-    const int h0 = (int)(W.t[0] >> 32), h1 = (int)(W.t[1] >> 32), h2 = (int)(W.t[2] >> 32);
-    const int hr = (int)(W.rend >> 32);
-    const int hm = min(min(h0, h1), min(h2, hr));
-    bool p0 = h0 == hm, p1 = h1 == hm, p2 = h2 == hm, split = hr == hm;
-    fix tm = p0 ? W.t[0] : (p1 ? W.t[1] : (p2 ? W.t[2] : W.rend));
-    if ((p0 && p1) || ((p0 || p1) && p2) || (split && (p0 || p1 || p2))) {
-        const fix m = min(min(W.t[0], W.t[1]), W.t[2]);
-        split = W.rend <= m;
-        tm = split ? W.rend : m;
-        // axes crossing together with the earliest one (relative tie 2^-40): a diagonal step
-        const fix tol = m >> 40;
-        p0 = W.t[0] - m <= tol;
-        p1 = W.t[1] - m <= tol;
-        p2 = W.t[2] - m <= tol;
-    }
-    // segment length: the distance moved, below 2 cells, to 2^-30 cells
-    const fix mv = tm - W.tc;
-    const int q = (int)__funnelshift_r((unsigned)mv, (unsigned)(mv >> 32), (unsigned)fbits - 30u);
-    // deposit in the current cell (segments of length <= 0 deposit nothing)
-    const bool seg = !out && mv > 0;
-    const float ds = seg ? (float)q * 0x1p-30f : 0.f;
-    o.ds = ds;
-    o.cell = W.idx;
-    // advance
-    W.tc = tm;
-    if (p0) { W.t[0] += W.d[0]; W.idx += W.ss[0]; }
-    if (p1) { W.t[1] += W.d[1]; W.idx += W.ss[1]; }
-    if (p2) { W.t[2] += W.d[2]; W.idx += W.ss[2]; }
+    float x;
+    walk_move(W, rend, unit, chi_of(W.cell), 0.f, 0.f, -1, npad, o.ds, x, o.cell, ncross);
+    const bool split = W.idx == npad;
+    o.seg = o.cell >= 0;
     // prefetch of the next cell: from a cell inside the grid every crossing (also a diagonal
     // one) lands inside the padded layout
     const Cell ncell = out ? cell_zero<Cell>() : load_cell(cells + W.idx);
-    const float x = chi_of(W.cell) * ds;
-    o.seg = seg;
+    const float ph = phi_dphi(x, o.dphi);
     o.Lin = W.L;
-    o.dtau = x;
-    if (!kCountOnly) {
-        float ph;
-        if constexpr (kDphi) ph = phi_dphi(x, o.dphi);
-        else ph = phi_of(x);
-        o.phi = ph;
-        o.G = W.L * ds * ph;
-        o.dL = W.L * x * ph;
-        // L - dL, and its rounding error (Fast2Sum, dL <= L) kept for the photon ledger:
-        // where a cell is nearly transparent dL falls below half an ulp of L, so the
-        // deposited dL never leaves L. The deposits keep using L itself, whose relative
-        // accuracy survives strong attenuation (L + Lc carries the absolute error of all
-        // deposits instead); only the tallies of retired rays take L + Lc.
-        const float Lnew = __fsub_rn(W.L, o.dL);
-        W.Lc = __fadd_rn(W.Lc, __fsub_rn(__fsub_rn(W.L, Lnew), o.dL));
-        W.L = Lnew;
-    } else {
-        o.phi = 1.f;
-        o.G = 0.f;
-        o.dL = 0.f;
-    }
+    o.G = W.L * o.ds * ph;
+    o.dL = W.L * x * ph;
+    W.L -= o.dL;
     W.tau += x;
-    bool drop;
-    if constexpr (TwoBin<Cell>::value) {
-        // second bin on the same ray; the packet is used up once its dust-only depth (never
-        // the larger one) passes tau_max
-        const float xn = W.cell.y * ds;
-        o.dLn = W.Ln * xn * phi_of(xn);
-        const float Lnnew = __fsub_rn(W.Ln, o.dLn);
-        W.Lnc = __fadd_rn(W.Lnc, __fsub_rn(__fsub_rn(W.Ln, Lnnew), o.dLn));
-        W.Ln = Lnnew;
-        W.taun += xn;
-        drop = seg && W.taun > tau_max;
-    } else {
-        o.dLn = 0.f;
-        drop = seg && W.tau > tau_max;
-    }
-    o.end = out || drop || split;
+    const bool drop = o.seg && W.tau > tau_max;
     o.ev = out ? EV_EXIT : (drop ? EV_DROP : (split ? EV_SPLIT : EV_NONE));
     W.cell = ncell;
     return o;
 }
 
 // Merges the deposits of lanes that hit the same cell (runs of equal cell index in lane
-// order) and issues one reduction per run. Used only for the first segment of base-level
-// rays, which all start in their source's cell: at l0 = 8 that is 786,432 deposits into one
-// cell per source, whose FP32 sum the merge keeps accurate. Warp-uniform.
-__device__ __forceinline__ void red_v4(float4* q, float4 v)
-{
-    float* p = reinterpret_cast<float*>(q);
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y),
-                 "f"(v.z), "f"(v.w)
-                 : "memory");
-}
-
-__device__ __forceinline__ void deposit_merged(float4* __restrict__ acc, int cell, float4 v)
+// order) into the first lane of each run and takes them from the others. Used only for the
+// first segment of base-level rays, which all start in their source's cell: at l0 = 8 that is
+// 786,432 deposits into one cell per source, whose FP32 sum the merge keeps accurate.
+// Warp-uniform.
+__device__ __forceinline__ void merge_lanes(int& cell, float4& v)
 {
     const unsigned lane = threadIdx.x & 31u;
     const int prev = __shfl_up_sync(kFull, cell, 1);
@@ -523,18 +601,28 @@ __device__ __forceinline__ void deposit_merged(float4* __restrict__ acc, int cel
             v.x += ox; v.y += oy; v.z += oz; v.w += ow;
         }
     }
-    if (cell >= 0 && !dup) red_v4(acc + cell, v);
+    if (dup) cell = -1;
 }
 
-// One 16-byte vector reduction (G, dL n) into the accumulator of `cell` (none if < 0).
-// Merging equal cells across lanes first was measured slower than letting L2 combine them.
-__device__ __forceinline__ void deposit(float4* __restrict__ acc, int cell, float4 v)
+// Adds the deposit of ray b to that of ray a where both lie in the same cell (key: the cell,
+// or a negative number of the ray's own without a deposit), leaving ray b without one.
+__device__ __forceinline__ void merge_pair(int key_a, float4& a, int& key_b, const float4& b,
+                                           int none)
 {
-    if (cell >= 0) red_v4(acc + cell, v);
+    asm("{\n\t.reg .pred q;\n\tsetp.eq.s32 q, %5, %4;\n\t@q add.f32 %0, %0, %6;\n\t"
+        "@q add.f32 %1, %1, %7;\n\t@q add.f32 %2, %2, %8;\n\t@q add.f32 %3, %3, %9;\n\t"
+        "@q mov.b32 %4, %10;\n\t}"
+        : "+f"(a.x), "+f"(a.y), "+f"(a.z), "+f"(a.w), "+r"(key_b)
+        : "r"(key_a), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w), "r"(none));
 }
-__device__ __forceinline__ void deposit_if(float4* __restrict__ acc, bool dep, int cell, float4 v)
+
+// One reduction into the accumulator of cell `key`, none if it is negative.
+__device__ __forceinline__ void red_v4_if(float4* __restrict__ acc, int key, float4 v)
 {
-    if (dep) red_v4(acc + cell, v);
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %1, 0;\n\t"
+                 "@q red.global.add.v4.f32 [%0], {%2, %3, %4, %5};\n\t}"
+                 :: "l"(acc + key), "r"(key), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
 }
 
 // ---------------------------------------------------------------------------------------
@@ -605,6 +693,19 @@ __device__ __forceinline__ bool splits_at_end(bool splits, fix rmax, fix dmax)
     return !kCut || (splits && rmax < dmax);
 }
 
+// One entry of a direction table: n (df) and the face spacing code per axis.
+__device__ __forceinline__ void load_direction(const float4* e, df n[3], fix code[3])
+{
+    const float4 e0 = __ldg(e), e1 = __ldg(e + 1);
+    const longlong2 e2 = __ldg(reinterpret_cast<const longlong2*>(e + 2));
+    n[0] = {e0.x, e0.w};
+    n[1] = {e0.y, e1.x};
+    n[2] = {e0.z, e1.y};
+    code[0] = (fix)(((unsigned long long)__float_as_uint(e1.w) << 32) | __float_as_uint(e1.z));
+    code[1] = e2.x;
+    code[2] = e2.y;
+}
+
 // Starts the walk of ray i of level l: loads its record, its source and its direction
 // entry. Returns 1 if the ray starts inside the grid, 0 if it starts outside (it escapes at
 // once), -1 if slot i holds no ray. L0 receives its entering L.
@@ -612,7 +713,7 @@ template <bool kCut, class Cell>
 __device__ __forceinline__ int ray_begin(const TraceArgs& A, const LevelInfo& LV, const RayBuf& B,
                                          int l, unsigned long long i, WalkT<Cell>& W,
                                          const Cell* cells, unsigned& s, unsigned& p, float& L0,
-                                         bool& splits)
+                                         bool& splits, fix& rend)
 {
     s = __ldcg(B.src + i);
     if (s == kHole) return -1;
@@ -624,24 +725,18 @@ __device__ __forceinline__ int ray_begin(const TraceArgs& A, const LevelInfo& LV
     L0 = (l == A.level0) ? sh.w : __ldcg(B.L + i);
     const float tau0 = (l == A.level0) ? 0.f : __ldcg(B.tau + i);
     splits = l < __float_as_int(sl.w);
-    const float4 e0 = __ldg(LV.dir + 3ull * p);
-    const float4 e1 = __ldg(LV.dir + 3ull * p + 1);
-    const longlong2 e2 = __ldg(reinterpret_cast<const longlong2*>(LV.dir + 3ull * p + 2));
+    const float4* e = LV.dir + 3ull * p;
     const df u[3] = {{sh.x, sl.x}, {sh.y, sl.y}, {sh.z, sl.z}};
     const fix ux[3] = {xy.x, xy.y, z_.x};
-    const df n[3] = {{e0.x, e0.w}, {e0.y, e1.x}, {e0.z, e1.y}};
-    const fix code[3] = {(fix)(((unsigned long long)__float_as_uint(e1.w) << 32) | __float_as_uint(e1.z)),
-                         e2.x, e2.y};
-    const bool inside = walk_start(W, A.nx, A.ny, A.nz, A.fbits, u, ux, n, code, LV.r0, LV.r0x);
-    W.rend = end_radius<kCut>(splits, LV.rmaxx, A.dmax);
+    df n[3];
+    fix code[3];
+    load_direction(e, n, code);
+    const bool inside = path_start(W, A.nx, A.ny, A.nz, A.fbits, u, ux, n, code, LV.r0, LV.r0x);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) W.n[a] = n[a].hi;
+    rend = end_radius<kCut>(splits, LV.rmaxx, A.dmax);
     W.L = L0;
-    W.Lc = 0.f;
     W.tau = tau0;
-    if constexpr (TwoBin<Cell>::value) {
-        W.Ln = (l == A.level0) ? __ldg(A.srcLn + s) : __ldcg(B.Ln + i);
-        W.Lnc = 0.f;
-        W.taun = (l == A.level0) ? 0.f : __ldcg(B.taun + i);
-    }
     W.cell = inside ? load_cell(cells + W.idx) : cell_zero<Cell>();
     return inside ? 1 : 0;
 }
@@ -674,7 +769,9 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
-__device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long wait_ns)
+// The block that arrives last runs `last` (one thread) before it releases the others.
+template <class F>
+__device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long wait_ns, F last)
 {
     __shared__ int s_ok;
     __syncthreads();
@@ -685,6 +782,8 @@ __device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long 
         __threadfence();
         const unsigned arrived = atomicAdd(&sc->bar_count, 1u) + 1u;
         if (arrived == gridDim.x) {
+            __threadfence();
+            last();
             atomicExch(&sc->bar_count, 0u);
             __threadfence();
             atomicAdd(&sc->bar_gen, 1u);
@@ -696,7 +795,7 @@ __device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long 
                     ok = 0;
                     break;
                 }
-                __nanosleep(200);
+                __nanosleep(40);
             }
         }
         __threadfence();
@@ -705,6 +804,10 @@ __device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long 
     }
     __syncthreads();
     return s_ok != 0;
+}
+__device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long wait_ns)
+{
+    return grid_barrier(sc, st, wait_ns, [] {});
 }
 
 }  // namespace art

@@ -50,7 +50,6 @@ struct art_grid {
     size_t srcLn_cap = 0;
     std::vector<float> h_Ln_stage;
     PinnedVec<float> h_srcLn_pin;
-    bool buf_2bin[art::kNL] = {};
     std::vector<int> src_lmax;
 
     // device buffers owned by the grid
@@ -69,10 +68,13 @@ struct art_grid {
     bool dir_rotate = false;
     double dir_rot[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
 
+    // forward fronts (quads) of the levels beyond l0
+    art::QuadBuf quad[art::kNL] = {};
+    unsigned long long quad_cap[art::kNL] = {};      // allocated quads per level
+
+    // adjoint fronts
     art::RayBuf buf[art::kNL] = {};
     unsigned long long buf_cap[art::kNL] = {};      // allocated rays per level
-    unsigned long long buf_cap_req[art::kNL] = {};
-    bool buf_adj[art::kNL] = {};                     // adjoint arrays allocated
 
     // adjoint: source luminosities and a dL buffer for callers that pass none
     float* d_srcL = nullptr;

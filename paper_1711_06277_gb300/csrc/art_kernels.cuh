@@ -1,20 +1,37 @@
 // art_kernels.cuh -- forward trace kernels of the GB300 adaptive ray trace.
 //
-// Work decomposition. The rays of one HEALPix level form a "front" held structure-of-arrays
-// in a level buffer. A warp takes rays from the front in chunks (one ray per lane, lanes
-// refill from the chunk as their rays end), walks each ray from its start radius to its end
-// (Sec. 2.1: r_max(l), tau > tau_max or the grid boundary) and appends the four children of
-// every split ray to the next level's buffer with one warp-aggregated reservation.
+// Work decomposition. The rays of one HEALPix level form a "front" of quads, the four
+// children of a split ray, in the order their parents ended. A warp takes 64 neighbouring rays
+// at a time, two per lane, and walks them in lock step from their start radius to their ends
+// (Sec. 2.1: r_max(l), tau > tau_max or the grid boundary), then appends the children of its
+// split rays to the next front with one reservation. Small fronts are walked one ray per lane.
+//
+// What bounds it: the SM's reductions and its instruction issue, about equally. An SM issues a
+// 16-byte reduction at 1.36 clocks per lane when the lanes hit different sectors (44 clocks per
+// full warp, measured), and equal addresses within a warp are not combined: one reduction per
+// ray and step capped the trace at 2.2e11 crossings per second, whatever the instruction
+// count. Two siblings lie in the same cell in 44 % of their steps (m_ray = 4), and merging them
+// within a thread costs a compare and four predicated adds, where merging across lanes costs
+// shuffles. Lock step keeps siblings together and needs no refill of idle lanes: neighbouring
+// rays of a front take nearly the same number of steps (88-93 % lane use over a warp). Four rays
+// per lane merge more (0.51 against 0.68 sectors per crossing) but leave 12 instead of 20 warps
+// per SM (16.7 against 14.3 ms on 256^3 / 16 sources, before the step was trimmed further).
+// Against one ray per lane with refills (and floating-point pairs for the distances):
+// 84.9 -> 49.0 ms on 256^3 / 64 sources, 620 -> 425 ms on 512^3 / 64 sources, 3.55 -> 0.30 ms on
+// 128^3 / 64 sources cut at 19 cells, where rays of 7 steps had waited for refills every 64.
 //
 // Two schedules share that routine:
 //   * plain: one launch per (source, level), fronts kept whole;
 //   * persistent: one cooperative launch for all sources. The launch loops over phases;
-//     each phase consumes the top part of the deepest non-empty level buffer, at most a
-//     quarter of the next buffer's capacity, so the children always fit. Deepest-first order
-//     keeps every buffer bounded, which is the memory role the paper's last-in-first-out ray
-//     stack plays (Sec. 2.2). A grid barrier with a bounded wait separates phases; the
-//     retired-ray weights 4^(l_max - l) are summed as the paper's destroy counter (Sec. 2.2).
+//     each phase consumes the top part of the deepest non-empty front, at most a quarter of
+//     the next front's capacity, so the children always fit. Deepest-first order keeps every
+//     buffer bounded, which is the memory role the paper's last-in-first-out ray stack plays
+//     (Sec. 2.2). A grid barrier with a bounded wait separates phases; the last block to
+//     arrive chooses the next phase. The retired-ray weights 4^(l_max - l) are summed as the
+//     paper's destroy counter (Sec. 2.2).
 #pragma once
+
+#include <type_traits>
 
 #include "art_device.cuh"
 
@@ -120,6 +137,10 @@ __global__ void k_opacity(int nx, int ny, int nz, const float* __restrict__ nH0,
     const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
     const unsigned step = gridDim.x * blockDim.x;
     bool bad = false;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        chi[npad] = kEnded;
+        if (chi2) chi2[npad] = make_float2(kEnded, 0.f);
+    }
     for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
         unsigned i;
         if (!unpad(q, nx, ny, nz, i)) {
@@ -138,194 +159,385 @@ __global__ void k_opacity(int nx, int ny, int nz, const float* __restrict__ nH0,
     if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicCAS(&st->error, 0, -1);
 }
 
-// Level-l0 rays of sources [s0, s0 + ns): pixel-major within each source.
-__global__ void k_inject(int s0, int nsrc, unsigned npix0, RayBuf B, unsigned long long* count)
-{
-    unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-    unsigned long long n = (unsigned long long)nsrc * npix0;
-    if (i == 0) *count = n;
-    if (i >= n) return;
-    unsigned s = (unsigned)(i / npix0);
-    unsigned p = (unsigned)(i - (unsigned long long)s * npix0);
-    B.src[i] = s0 + s;
-    B.pix[i] = p;
-    B.L[i] = 0.f;     // filled from the source table when the ray starts
-    B.tau[i] = 0.f;
-}
-
-// Processes the rays in slots [cursor .. end) of level l, whose phase starts at slot
-// `begin` (cursor advanced atomically by warps, `chunk` slots at a time). The children of
-// the ray in slot i go to slots 4 (i - begin) .. +3 of level l + 1, so the next front keeps
-// the pixel order of this one; parents that do not split mark their four slots empty. Idle
-// lanes are refilled once 16 of the 32 are idle, so the ray set-up runs with many lanes at
-// once. Warp-uniform: every lane of the warp must call it.
 // The per-cell records a trace gathers: opacities (one bin) or opacity pairs (two bins).
 template <class Cell> __device__ __forceinline__ const Cell* cells_of(const TraceArgs& A);
 template <> __device__ __forceinline__ const float* cells_of<float>(const TraceArgs& A) { return A.chi; }
 template <> __device__ __forceinline__ const float2* cells_of<float2>(const TraceArgs& A) { return A.chi2; }
 
-// Idle lanes of a warp before it refills them from its chunk, and steps between refill
-// checks (measured: 16 lanes > 18, 14 > 12 > 10; 64 steps > 32 > 16 > 8).
-#ifndef ART_FWD_IDLE
-#define ART_FWD_IDLE 16
-#endif
-#ifndef ART_FWD_STEPS
-#define ART_FWD_STEPS 64
-#endif
+// Threads per block of the forward kernels at most, and blocks per SM that the register
+// budget must leave room for (65536 / (128 * 5) = 102 registers a thread: two walks).
+constexpr int kTraceMaxThreads = 128;
+constexpr int kTraceMinBlocks = 5;
+// Steps between checks whether a warp still has rays.
+constexpr int kCheckSteps = 4;
 
-template <class Cell, bool kCut>
-__device__ void run_rays(const TraceArgs& A, const Cell* cells, int l,
-                         unsigned long long* cursor, unsigned long long begin,
-                         unsigned long long end, Tally& T)
+__device__ __forceinline__ void load_pair(const float* p, float& a, float& b) { a = __ldg(p); b = 0.f; }
+__device__ __forceinline__ void load_pair(const float2* p, float& a, float& b)
+{
+    const float2 v = __ldg(p);
+    a = v.x;
+    b = v.y;
+}
+
+// Tallies of a block: photon sums per thread (no atomics while rays end), counters per warp
+// or per level. Reduced once, when the kernel ends.
+struct BlockTally {
+    double escaped[kTraceMaxThreads], dropped[kTraceMaxThreads];
+    double escaped_n[kTraceMaxThreads], dropped_n[kTraceMaxThreads];
+    unsigned long long crossings, destroy;
+    unsigned long long rays[kNL];
+};
+
+__device__ __forceinline__ BlockTally& block_tally()
+{
+    __shared__ BlockTally t;
+    return t;
+}
+
+__device__ __forceinline__ void block_tally_init()
+{
+    BlockTally& T = block_tally();
+    const int i = threadIdx.x;
+    T.escaped[i] = T.dropped[i] = T.escaped_n[i] = T.dropped_n[i] = 0.0;
+    if (i < kNL) T.rays[i] = 0ull;
+    if (i == 0) T.crossings = T.destroy = 0ull;
+    __syncthreads();
+}
+
+__device__ __forceinline__ void block_tally_flush(DevStats* st)
+{
+    BlockTally& T = block_tally();
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) {
+        v[0] += T.escaped[i];
+        v[1] += T.dropped[i];
+        v[2] += T.escaped_n[i];
+        v[3] += T.dropped_n[i];
+    }
+    double* out[4] = {&st->escaped, &st->dropped, &st->escaped_n, &st->dropped_n};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(kFull, v[k], off);
+        if (threadIdx.x == 0 && v[k] != 0.0) atomicAdd(out[k], v[k]);
+    }
+    if (threadIdx.x == 0) {
+        if (T.crossings) atomicAdd(&st->crossings, T.crossings);
+        if (T.destroy) atomicAdd(&st->destroy, T.destroy);
+    }
+    if (threadIdx.x < kNL && T.rays[threadIdx.x]) {
+        atomicAdd(&st->rays_per_level[threadIdx.x], T.rays[threadIdx.x]);
+        atomicAdd(&st->rays_total, T.rays[threadIdx.x]);
+        atomicMax(&st->level_reached, (int)threadIdx.x);
+    }
+}
+
+// Sum of a few floats in two floats, for the tallies.
+__device__ __forceinline__ void df_accumulate(df& s, float v)
+{
+    const df r = df_two_sum(s.hi, v);
+    s.hi = r.hi;
+    s.lo += r.lo;
+}
+
+// Photons of the rays of a lane, side by side (V: float or float2).
+template <class V>
+struct Photons {
+    V L, tau;
+    V Lc;        // photon ledger: the rounding error of this walk's L updates; tallied with
+                 // the ray, never used for deposits
+    V n[3];      // directions (hi parts) for momentum deposits
+    V Ln, taun, Lnc;  // non-ionizing bin (two-bin traces only)
+};
+
+// L - dL, and its rounding error (Fast2Sum, dL <= L) for the photon ledger: where a cell is
+// nearly transparent dL falls below half an ulp of L, so the deposited dL never leaves L. The
+// deposits keep using L itself, whose relative accuracy survives strong attenuation (L + Lc
+// carries the absolute error of all deposits instead); only the tallies of retired rays take
+// L + Lc.
+template <class V>
+__device__ __forceinline__ void lose(V& L, V& Lc, V dL)
+{
+    const V Lnew = vsub(L, dL);
+    Lc = vadd(Lc, vsub(vsub(L, Lnew), dL));
+    L = Lnew;
+}
+
+// Walks kWidth (1 or 2) rays per lane: the rays of quads [begin, end) of level l, taken 32
+// lanes at a time from `cursor`, which counts items of kWidth rays. Base-level quads are
+// implied by their index (src0 is the first source), deeper ones are records; strided says
+// that a lane takes two base rays 32 apart instead of neighbours. Warp-uniform.
+template <class Cell, bool kCut, int kWidth>
+__device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, int l,
+                           unsigned long long* cursor, unsigned long long end, unsigned src0,
+                           bool strided)
 {
     constexpr bool two = TwoBin<Cell>::value;
+    using V = typename std::conditional<kWidth == 1, float, float2>::type;
+    constexpr unsigned kPerQuad = 4u / kWidth;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt = (1u << lane) - 1u;
     const LevelInfo& LV = A.levels[l];
-    const RayBuf& B = A.buf[l];
-    const RayBuf& C = A.buf[l + 1];
-    const bool has_next = l < A.lmax_glob;
-
-    // slot indices fit in 32 bits (level buffers hold fewer than 2^31 slots)
-    const unsigned b32 = (unsigned)begin, e32 = (unsigned)end;
-    unsigned wnext = 0, wend = 0;
-    bool more = true;
-    bool active = false;
-    WalkT<Cell> W;
-    unsigned s = 0, p = 0;
-    unsigned slot = 0;
-    float L0 = 0.f;
-    bool splits = false;
-    bool first = false;  // next step is the first segment of a base-level ray
-    const bool base = l == A.level0;
-    unsigned ncross = 0, nrays = 0;
+    const bool base = kWidth == 2 && l == A.level0;  // base rays are walked two per lane
+    BlockTally& T = block_tally();
+    __shared__ float4 s_second[kTraceMaxThreads];
+    const unsigned items = (unsigned)end * kPerQuad;  // front ends below 2^29 quads
+    unsigned ncross = 0;
 
     for (;;) {
-        // refill idle lanes from the warp's chunk, fetching chunks as needed
-        unsigned need = __ballot_sync(kFull, !active);
-        if (__popc(need) >= ART_FWD_IDLE || need == kFull) {
-            while (need && more) {
-                if (wnext >= wend) {
-                    unsigned long long b = 0;
-                    if (lane == 0) b = atomicAdd(cursor, (unsigned long long)A.chunk);
-                    b = __shfl_sync(kFull, b, 0);
-                    if (b >= end) { more = false; break; }
-                    wnext = (unsigned)b;
-                    wend = min(wnext + (unsigned)A.chunk, e32);
-                }
-                const unsigned avail = min(wend - wnext, 32u);
-                const unsigned rank = __popc(need & lt);
-                if (!active && rank < avail) {
-                    slot = wnext + rank;
-                    const int st = ray_begin<kCut>(A, LV, B, l, slot, W, cells, s, p, L0, splits);
-                    if (st > 0) {
-                        active = true;
-                        first = base;
-                        ++nrays;
-                    } else {
-                        if (st == 0) {  // starts outside the grid: escapes with its full L
-                            atomicAdd(&T.escaped, (double)L0);
-                            if constexpr (two) atomicAdd(&T.escaped_n, (double)W.Ln + (double)W.Lnc);
-                            atomicAdd(&T.destroy, LV.destroy_w);
-                            ++nrays;
-                        }
-                        if (has_next) write_holes(C, 4ull * (slot - b32));
-                    }
-                }
-                wnext += min(avail, (unsigned)__popc(need));
-                need = __ballot_sync(kFull, !active);
+        unsigned b = 0;
+        if (lane == 0) b = (unsigned)min(atomicAdd(cursor, 32ull), (unsigned long long)items);
+        b = __shfl_sync(kFull, b, 0);
+        if (b >= items) break;
+
+        // ---- set-up: a part of a quad per lane
+        const unsigned item = b + lane;
+        const bool valid = item < items;
+        Path W[kWidth];
+        Photons<V> P;
+        float cell[kWidth], celln[kWidth];
+        unsigned s = 0, pix = 0;
+        const unsigned apart = strided ? 32u : 1u;  // between the pixels of a lane's rays
+        fix rend = kNoEnd;
+        bool splits = false;
+        P.L = P.tau = P.Lc = P.Ln = P.taun = P.Lnc = vset<V>(0.f);
+        if (valid) {
+            unsigned quad = item / kPerQuad, part = item % kPerQuad * kWidth;
+            if (strided) {
+                quad = (2u * b + lane) / 4u;
+                part = lane % 4u;
             }
-        }
-        if (!__any_sync(kFull, active)) {
-            if (!more) break;
-            continue;
+            float L0 = 0.f, tau0 = 0.f, Ln0 = 0.f, taun0 = 0.f;
+            if (base) {
+                s = src0 + quad / A.base_quads;
+                pix = 4u * (quad % A.base_quads);
+            } else {
+                const uint4 r = __ldcg(A.quad[l].rec + quad);
+                s = r.x;
+                pix = r.y;
+                L0 = __uint_as_float(r.z);
+                tau0 = __uint_as_float(r.w);
+                if constexpr (two) {
+                    const float2 rn = __ldcg(A.quad[l].recn + quad);
+                    Ln0 = rn.x;
+                    taun0 = rn.y;
+                }
+            }
+            pix += part;
+            const float4 sh = __ldg(&A.src[s].hi);
+            const float4 sl = __ldg(&A.src[s].lo);
+            const longlong2 xy = __ldg(&A.src[s].xy);
+            const longlong2 z_ = __ldg(&A.src[s].z_);
+            const df u[3] = {{sh.x, sl.x}, {sh.y, sl.y}, {sh.z, sl.z}};
+            const fix ux[3] = {xy.x, xy.y, z_.x};
+            splits = l < __float_as_int(sl.w);
+            rend = end_radius<kCut>(splits, LV.rmaxx, A.dmax);
+            if (base) {
+                L0 = sh.w;
+                if constexpr (two) Ln0 = __ldg(A.srcLn + s);
+            }
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j) {
+                df n[3];
+                fix code[3];
+                load_direction(LV.dir + 3ull * (pix + j * apart), n, code);
+                const bool inside = path_start(W[j], A.nx, A.ny, A.nz, A.fbits, u, ux, n, code,
+                                               LV.r0, LV.r0x);
+                // padded cell 0 is a sentinel: a ray that starts outside exits at once
+                load_pair(cells + (inside ? W[j].idx : 0), cell[j], celln[j]);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) vget(P.n[a], j) = n[a].hi;
+            }
+            P.L = vset<V>(L0);
+            P.tau = vset<V>(tau0);
+            P.Ln = vset<V>(Ln0);
+            P.taun = vset<V>(taun0);
+        } else {
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j) {
+                W[j] = Path{};
+                W[j].t[1] = 1ll << 40;
+                W[j].t[2] = 1ll << 41;
+                cell[j] = kSentinel;
+                celln[j] = 0.f;
+            }
+            P.n[0] = P.n[1] = P.n[2] = vset<V>(0.f);
         }
 
+        // ---- walk: a ray that has ended sits in a cell of negative opacity (the sentinel
+        // ring where it left the grid, the end marker where it reached its end radius) or has
+        // passed tau_max, and does nothing more. In two-bin traces the packet is used up once
+        // its dust-only depth (never the larger one) passes tau_max.
+        int second_key = -1;
+        auto step = [&](auto first) {
+            int key[kWidth];
+            V ds, x, xn = vset<V>(0.f);
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j) {
+                const float depth = vget(two ? P.taun : P.tau, j);
+                bool alive = false;
+                if constexpr (two) alive = !(cell[j] < 0.f) & !(depth > A.tau_max);
+                walk_move_load(W[j], rend, A.unit, cell[j], depth, A.tau_max, -1 - j,
+                               (int)A.npad, cells, vget(ds, j), vget(x, j), key[j], ncross);
+                if constexpr (two) {
+                    vget(xn, j) = celln[j] * vget(ds, j);
+                    if (alive) celln[j] = __ldg(&cells[W[j].idx].y);
+                }
+            }
+            // deposit and loss
+            P.tau = vadd(P.tau, x);
+            const V ph = phi_of(x);
+            const V G = vmul(vmul(P.L, ds), ph);
+            const V dL = vmul(vmul(P.L, x), ph);
+            lose(P.L, P.Lc, dL);
+            V dm = dL;  // momentum of both bins
+            if constexpr (two) {
+                P.taun = vadd(P.taun, xn);
+                const V dLn = vmul(vmul(P.Ln, xn), phi_of(xn));
+                lose(P.Ln, P.Lnc, dLn);
+                dm = vadd(dm, dLn);
+            }
+            const V f0 = vmul(dm, P.n[0]), f1 = vmul(dm, P.n[1]), f2 = vmul(dm, P.n[2]);
+            float4 v[kWidth];
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j)
+                v[j] = make_float4(vget(G, j), vget(f0, j), vget(f1, j), vget(f2, j));
+            if constexpr (kWidth == 2 && decltype(first)::value) {
+                if (!strided) merge_pair(key[0], v[0], key[1], v[1], -2);
+                merge_lanes(key[0], v[0]);
+                merge_lanes(key[1], v[1]);
+                red_v4_if(A.acc, key[0], v[0]);
+                second_key = key[1];
+                s_second[threadIdx.x] = v[1];
+            } else {
+                if constexpr (kWidth == 2) merge_pair(key[0], v[0], key[1], v[1], -2);
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j) red_v4_if(A.acc, key[j], v[j]);
+            }
+        };
+        // The first segments of base rays all lie in their source's cell: a warp deposits those
+        // of each of its two groups of 32 as one sum, the second when the walk is done, so that
+        // the additions to that one cell are spread over the phase.
+        if (base) step(std::true_type{});
+        for (;;) {
+            bool any = false;
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j)
+                any |= !(cell[j] < 0.f) & !(vget(two ? P.taun : P.tau, j) > A.tau_max);
+            if (!__any_sync(kFull, any)) break;
 #pragma unroll 1
-        for (int k = 0; k < ART_FWD_STEPS; ++k) {
-            bool dep = false;
-            int cell = 0;
-            float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (active) {
-                const StepOut o = walk_step<false>(W, A.fbits, cells, A.tau_max);
-                dep = o.seg;  // segments without length deposit nothing
-                cell = o.cell;
-                const float dm = two ? o.dL + o.dLn : o.dL;  // momentum of both bins
-                dv = make_float4(o.G, dm * W.n[0], dm * W.n[1], dm * W.n[2]);
-                ncross += o.seg ? 1u : 0u;
-                if (o.end) {
-                    active = false;
-                    const unsigned long long c4 = 4ull * (slot - b32);
-                    if (o.ev == EV_SPLIT && splits_at_end<kCut>(splits, LV.rmaxx, A.dmax)) {
-                        if (c4 + 4 <= C.cap) {
-                            const float Lc = 0.25f * W.L;
-                            *reinterpret_cast<uint4*>(C.src + c4) = make_uint4(s, s, s, s);
-                            *reinterpret_cast<uint4*>(C.pix + c4) =
-                                make_uint4(4 * p, 4 * p + 1, 4 * p + 2, 4 * p + 3);
-                            *reinterpret_cast<float4*>(C.L + c4) = make_float4(Lc, Lc, Lc, Lc);
-                            *reinterpret_cast<float4*>(C.tau + c4) =
-                                make_float4(W.tau, W.tau, W.tau, W.tau);
-                            if constexpr (two) {
-                                const float Ln = 0.25f * W.Ln;
-                                *reinterpret_cast<float4*>(C.Ln + c4) = make_float4(Ln, Ln, Ln, Ln);
-                                *reinterpret_cast<float4*>(C.taun + c4) =
-                                    make_float4(W.taun, W.taun, W.taun, W.taun);
-                            }
-                        } else {
-                            atomicCAS(&A.stats->error, 0, -3);  // ART_EQUEUE_OVERFLOW
-                        }
-                        // the split ray's ledger residual: its children start from L itself
-                        if (W.Lc != 0.f) atomicAdd(&T.escaped, (double)W.Lc);
-                        if constexpr (two) {
-                            if (W.Lnc != 0.f) atomicAdd(&T.escaped_n, (double)W.Lnc);
-                        }
-                    } else {
-                        // leaving the box or cut at d_max: escaped; tau > tau_max: dropped
-                        const double Lend = (double)W.L + (double)W.Lc;
-                        if (o.ev != EV_DROP) atomicAdd(&T.escaped, Lend);
-                        else atomicAdd(&T.dropped, Lend);
-                        if constexpr (two) {
-                            const double Lnend = (double)W.Ln + (double)W.Lnc;
-                            if (o.ev != EV_DROP) atomicAdd(&T.escaped_n, Lnend);
-                            else atomicAdd(&T.dropped_n, Lnend);
-                        }
-                        atomicAdd(&T.destroy, LV.destroy_w);
-                        if (has_next) write_holes(C, c4);
+            for (int k = 0; k < kCheckSteps; ++k) step(std::false_type{});
+        }
+        if (base) red_v4_if(A.acc, second_key, s_second[threadIdx.x]);
+
+        // ---- ends: tallies, and the children of split rays
+        bool child[kWidth];
+        unsigned nchild = 0, mine = 0, at[kWidth];
+        df esc = {0.f, 0.f}, dropped = {0.f, 0.f}, escn = {0.f, 0.f}, droppedn = {0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j) {
+            const bool drop = vget(two ? P.taun : P.tau, j) > A.tau_max;
+            child[j] = valid && cell[j] == kEnded && !drop &&
+                       splits_at_end<kCut>(splits, LV.rmaxx, A.dmax);
+            const unsigned m = __ballot_sync(kFull, child[j]);
+            // children in pixel order: group after group, or lane after lane
+            at[j] = __popc(m & lt) + (strided ? nchild : mine);
+            if (!strided && j > 0) {
+                at[j] += at[0];
+                at[0] += __popc(m & lt);
+            }
+            nchild += __popc(m);
+            mine += child[j] ? 1u : 0u;
+            // leaving the box or cut at d_max: escaped; tau > tau_max: dropped. A split ray
+            // leaves its ledger residual: its children start from L itself.
+            if (valid) {
+                df& to = drop ? dropped : esc;
+                df_accumulate(to, child[j] ? 0.f : vget(P.L, j));
+                df_accumulate(to, vget(P.Lc, j));
+                if constexpr (two) {
+                    df& ton = drop ? droppedn : escn;
+                    df_accumulate(ton, child[j] ? 0.f : vget(P.Ln, j));
+                    df_accumulate(ton, vget(P.Lnc, j));
+                }
+            }
+        }
+        T.escaped[threadIdx.x] += (double)esc.hi + (double)esc.lo;
+        if (dropped.hi != 0.f) T.dropped[threadIdx.x] += (double)dropped.hi + (double)dropped.lo;
+        if constexpr (two) {
+            T.escaped_n[threadIdx.x] += (double)escn.hi + (double)escn.lo;
+            T.dropped_n[threadIdx.x] += (double)droppedn.hi + (double)droppedn.lo;
+        }
+        const unsigned nray = kWidth * min(items - b, 32u);
+        unsigned slot = 0;
+        if (lane == 0) {
+            atomicAdd(&T.rays[l], (unsigned long long)nray);
+            atomicAdd(&T.destroy, (unsigned long long)(nray - nchild) * LV.destroy_w);
+            if (nchild) slot = (unsigned)atomicAdd(&A.sched->count[l + 1], (unsigned long long)nchild);
+        }
+        if (nchild) {
+            const QuadBuf& C = A.quad[l + 1];
+            slot = __shfl_sync(kFull, slot, 0);
+            if (slot + nchild > C.cap) {
+                atomicCAS(&A.stats->error, 0, -3);  // ART_EQUEUE_OVERFLOW
+            } else if (mine) {
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j) {
+                    if (child[j]) {
+                        __stcg(C.rec + slot + at[j],
+                               make_uint4(s, 4u * (pix + j * apart),
+                                          __float_as_uint(0.25f * vget(P.L, j)),
+                                          __float_as_uint(vget(P.tau, j))));
+                        if constexpr (two)
+                            __stcg(C.recn + slot + at[j],
+                                   make_float2(0.25f * vget(P.Ln, j), vget(P.taun, j)));
                     }
                 }
             }
-            if (base && __any_sync(kFull, first)) deposit_merged(A.acc, dep ? cell : -1, dv);
-            else deposit_if(A.acc, dep, cell, dv);
-            first = false;
         }
     }
-    tally_crossings(T, ncross);
-    count_rays(A.stats, l, nrays);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) ncross += __shfl_down_sync(kFull, ncross, off);
+    if (lane == 0 && ncross) atomicAdd(&T.crossings, (unsigned long long)ncross);
 }
 
-// Plain schedule: all slots of level l (one source's front).
-// Launch bounds of the trace kernels: at most ART_TRACE_MAX_THREADS threads per block and
-// ART_TRACE_MIN_BLOCKS resident blocks per SM, which caps the registers per thread at
-// 65536 / (threads x blocks).
-#ifndef ART_TRACE_MAX_THREADS
-#define ART_TRACE_MAX_THREADS 512
-#endif
-#ifndef ART_TRACE_MIN_BLOCKS
-#define ART_TRACE_MIN_BLOCKS 2
-#endif
-constexpr int kTraceMaxThreads = ART_TRACE_MAX_THREADS;
+// Rays per lane for a front of `quads` quads: one while that fits the chip's warps in one
+// round (latency counts there, and a step of one ray is shorter), else two; two at the base
+// level.
+__device__ __forceinline__ int front_width(bool base, unsigned long long quads)
+{
+    return !base && 4 * quads <= (unsigned long long)gridDim.x * blockDim.x ? 1 : 2;
+}
+
+// Base rays are taken 32 apart where the front's quads [begin, end) are whole groups of 64 rays
+// of one source.
+__device__ __forceinline__ bool front_strided(const TraceArgs& A, bool base,
+                                              unsigned long long begin, unsigned long long end)
+{
+    return base && A.base_quads % 16u == 0u && begin % 16u == 0u && end % 16u == 0u;
+}
 
 template <class Cell, bool kCut>
-__global__ void __launch_bounds__(ART_TRACE_MAX_THREADS, ART_TRACE_MIN_BLOCKS) k_trace_level(const __grid_constant__ TraceArgs A, int l)
+__device__ __forceinline__ void run_front(const TraceArgs& A, int l, int width,
+                                          unsigned long long* cursor, unsigned long long end,
+                                          unsigned src0, bool strided)
 {
-    tally_init();
-    Tally& T = tally_slots()[threadIdx.x >> 5];
+    if (width == 2) walk_front<Cell, kCut, 2>(A, cells_of<Cell>(A), l, cursor, end, src0, strided);
+    else walk_front<Cell, kCut, 1>(A, cells_of<Cell>(A), l, cursor, end, src0, false);
+}
+
+// Plain schedule: the whole front of level l of source s.
+template <class Cell, bool kCut>
+__global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_level(const __grid_constant__ TraceArgs A, int l, unsigned s)
+{
+    block_tally_init();
     // a front that overflowed (status set by the writer) is cut at the buffer capacity
     const unsigned long long end =
-        min(*((volatile unsigned long long*)&A.sched->count[l]), A.buf[l].cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && l < A.lmax_glob) A.sched->count[l + 1] = 4 * end;
-    run_rays<Cell, kCut>(A, cells_of<Cell>(A), l, &A.sched->cursor[l], 0, end, T);
-    tally_flush(A.stats);
+        l == A.level0 ? (unsigned long long)A.base_quads
+                      : min(*((volatile unsigned long long*)&A.sched->count[l]), A.quad[l].cap);
+    run_front<Cell, kCut>(A, l, front_width(l == A.level0, end), &A.sched->cursor[l], end, s,
+                          front_strided(A, l == A.level0, 0, end));
+    block_tally_flush(A.stats);
 }
 
 // Resets the per-level counters of the plain schedule before the next source.
@@ -335,54 +547,62 @@ __global__ void k_reset_counts(Sched* sc)
     if (t < kNL) { sc->count[t] = 0; sc->cursor[t] = 0; }
 }
 
+// Chooses the next phase of the persistent schedule (run by one thread, all others waiting).
+__device__ __forceinline__ void next_phase(const TraceArgs& A)
+{
+    volatile Sched* sc = A.sched;
+    if (!sc->started) {
+        sc->started = 1;
+        sc->count[A.level0] = (unsigned long long)A.base_quads * A.nsrc;
+    }
+    int l = -1;
+    for (int k = A.lmax_glob; k >= A.level0; --k)
+        if (sc->count[k] > 0) { l = k; break; }
+    if (l < 0) {
+        sc->done = 1;
+        return;
+    }
+    const unsigned long long have = sc->count[l];
+    unsigned long long take = have;
+    if (l < A.lmax_glob) take = min(have, A.quad[l + 1].cap / 4);
+    if (take == 0) {  // a phase must consume rays, or the schedule never ends
+        atomicCAS(&A.stats->error, 0, -8);  // ART_EINTERNAL
+        take = have;
+    }
+    const bool base = l == A.level0;
+    if (base && take > 16) take -= (have - take) % 16u ? 16u - (have - take) % 16u : 0u;
+    const int width = front_width(base, take);
+    sc->phase_strided = front_strided(A, base, have - take, have);
+    sc->phase_level = l;
+    sc->phase_width = width;
+    sc->phase_end = have;
+    sc->cursor[l] = (have - take) * (unsigned long long)(4 / width);
+    sc->count[l] = have - take;
+}
+
 // Persistent schedule: all sources, all levels, one cooperative launch.
 template <class Cell, bool kCut>
-__global__ void __launch_bounds__(ART_TRACE_MAX_THREADS, ART_TRACE_MIN_BLOCKS) k_trace_persistent(const __grid_constant__ TraceArgs A)
+__global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_persistent(const __grid_constant__ TraceArgs A)
 {
-    tally_init();
-    Tally& T = tally_slots()[threadIdx.x >> 5];
+    block_tally_init();
     Sched* sc = A.sched;
-    __shared__ int s_level;
-    __shared__ unsigned long long s_begin, s_end;
+    __shared__ int s_level, s_width, s_strided;
+    __shared__ unsigned long long s_end;
     for (;;) {
-        if (!grid_barrier(sc, A.stats, A.wait_ns)) break;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            volatile unsigned long long* cnt = sc->count;
-            int l = -1;
-            for (int k = A.lmax_glob; k >= A.level0; --k)
-                if (cnt[k] > 0) { l = k; break; }
-            if (l < 0) {
-                sc->done = 1;
-            } else {
-                unsigned long long have = min(cnt[l], A.buf[l].cap);
-                unsigned long long take = have;
-                if (l < A.lmax_glob) take = min(have, A.buf[l + 1].cap / 4);
-                if (take == 0) {  // a phase must consume rays, or the schedule never ends
-                    atomicCAS(&A.stats->error, 0, -8);  // ART_EINTERNAL
-                    take = have;
-                }
-                sc->phase_level = l;
-                sc->phase_begin = have - take;
-                sc->phase_end = have;
-                sc->cursor[l] = have - take;
-                cnt[l] = have - take;
-                if (l < A.lmax_glob) cnt[l + 1] = 4 * take;  // the children's slots
-            }
-            __threadfence();
-        }
-        if (!grid_barrier(sc, A.stats, A.wait_ns)) break;
+        if (!grid_barrier(sc, A.stats, A.wait_ns, [&] { next_phase(A); })) break;
         if (threadIdx.x == 0) {
             volatile Sched* v = sc;
             s_level = v->done ? -1 : v->phase_level;
-            s_begin = v->phase_begin;
+            s_width = v->phase_width;
+            s_strided = v->phase_strided;
             s_end = v->phase_end;
         }
         __syncthreads();
         const int l = s_level;
         if (l < 0) break;
-        run_rays<Cell, kCut>(A, cells_of<Cell>(A), l, &sc->cursor[l], s_begin, s_end, T);
+        run_front<Cell, kCut>(A, l, s_width, &sc->cursor[l], s_end, 0u, s_strided != 0);
     }
-    tally_flush(A.stats);
+    block_tally_flush(A.stats);
 }
 
 // Gamma, force and energy from the accumulator (padded layout) into the caller's SoA

@@ -32,7 +32,7 @@ namespace {
 // ends within nx + ny + nz + 2 steps.
 __global__ void k_reach(int nx, int ny, int nz, const float* __restrict__ chi,
                         const SrcDev* __restrict__ src, int nsrc, const float4* __restrict__ dir,
-                        unsigned npix, float tau_max, fix dmax, int fbits,
+                        unsigned npix, float tau_max, fix dmax, int fbits, int npad,
                         float* __restrict__ reach)
 {
     const unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
@@ -40,31 +40,29 @@ __global__ void k_reach(int nx, int ny, int nz, const float* __restrict__ chi,
     const unsigned s = (unsigned)(i / npix), p = (unsigned)(i - (unsigned long long)s * npix);
     const float4 sh = __ldg(&src[s].hi), sl = __ldg(&src[s].lo);
     const longlong2 xy = __ldg(&src[s].xy), z_ = __ldg(&src[s].z_);
-    const float4 e0 = __ldg(dir + 3ull * p), e1 = __ldg(dir + 3ull * p + 1);
-    const longlong2 e2 = __ldg(reinterpret_cast<const longlong2*>(dir + 3ull * p + 2));
     const df u[3] = {{sh.x, sl.x}, {sh.y, sl.y}, {sh.z, sl.z}};
     const fix ux[3] = {xy.x, xy.y, z_.x};
-    const df n[3] = {{e0.x, e0.w}, {e0.y, e1.x}, {e0.z, e1.y}};
-    const fix code[3] = {(fix)(((unsigned long long)__float_as_uint(e1.w) << 32) | __float_as_uint(e1.z)),
-                         e2.x, e2.y};
+    df n[3];
+    fix code[3];
+    load_direction(dir + 3ull * p, n, code);
     WalkT<float> W;
-    if (!walk_start(W, nx, ny, nz, fbits, u, ux, n, code, df{0.f, 0.f}, 0)) {
+    if (!path_start(W, nx, ny, nz, fbits, u, ux, n, code, df{0.f, 0.f}, 0)) {
         reach[i] = 0.f;
         return;
     }
-    W.rend = dmax;
     W.L = 0.f;
-    W.Lc = 0.f;
     W.tau = 0.f;
     W.cell = __ldg(chi + W.idx);
     float r = 0.f;
+    unsigned count = 0;
+    const float unit = exp2f((float)-fbits);
     const int bound = nx + ny + nz + 2;
     for (int k = 0; k < bound; ++k) {
         const fix before = W.tc;
-        const StepOut o = walk_step<true>(W, fbits, chi, tau_max);
+        const StepOut o = walk_step(W, dmax, unit, npad, chi, tau_max, count);
         if (o.ev == EV_NONE) continue;
         // an exit is seen one step late, in the sentinel cell: the ray left at `before`
-        r = (float)(o.ev == EV_EXIT ? before : W.tc) * exp2f((float)-fbits);
+        r = (float)(o.ev == EV_EXIT ? before : W.tc) * unit;
         break;
     }
     reach[i] = r;
@@ -105,7 +103,7 @@ int art_estimate_work(art_grid* g, const art_params* p, double* h_work)
         const fix dmax = p->d_max > 0.0 ? to_fix(p->d_max / g->dx, g->fbits) : kNoEnd;
         k_reach<<<(unsigned)((nray + 255) / 256), 256, 0, g->stream>>>(
             g->n[0], g->n[1], g->n[2], g->d_chi, d_src, ns, g->dir[le], npix, (float)p->tau_max,
-            dmax, g->fbits, d_reach);
+            dmax, g->fbits, (int)g->npad, d_reach);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
