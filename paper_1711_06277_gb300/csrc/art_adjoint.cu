@@ -12,19 +12,26 @@
 // points and tau_max retirement are held fixed.
 //
 // Nothing is stored per segment. Rays are traced with unit source luminosity (the loss is
-// linear in each L_s; gradients are scaled by L_s when deposited) in the deepest-first phases
-// of the persistent schedule, and every ray is walked twice:
-//   pass 1 sums the ray's own weighted G; a ray that splits stores that sum, a count of 4
-//     pending children and its children (with a back-pointer to it);
-//   pass 2 (S = own sum + the children's totals) deposits the gradients and adds the ray's
-//     total to its parent's. A ray that ends without splitting runs pass 2 at once; the lane
-//     whose child brings a parent's pending count to zero runs the parent's pass 2, and so on
-//     towards the base level.
-// Children always finish before their parent's pass 2 because the count only reaches zero
-// after all four of them have added their totals.
+// linear in each L_s; gradients are scaled by L_s when deposited) and every ray is walked twice:
+//   pass 1 sums the ray's own weighted segments; a ray that splits stores that sum and its
+//     children (a quad with a back-pointer to it);
+//   pass 2 (S = own sum + the children's totals) deposits the gradients. The total of a quad's
+//     four rays is the parent's sum over its descendants: one writer, no atomics.
+// The fronts and the lock-step walks are those of the forward trace (two rays per lane, one in
+// small fronts). The persistent schedule takes the deepest unfinished work first: "expand" a
+// part of a front (pass 1), then everything below it, then "collapse" that part (pass 2). A warp
+// whose 64 rays all end without splitting runs pass 2 at once; such parts (all of the deepest
+// fronts, and every part without children) need no collapse.
+//
+// Before, each lane ran its own state machine of both passes with refills, atomic count-downs of
+// the parents and completions in between, with 21 of 32 lanes active. Against that: 9.28 ->
+// 4.73 ms on 128^3 / 16 sources with a force term, 1.69 -> 0.81 ms on an odd box with force and
+// dust. What bounds it now is the issue of its instructions (69 % of cycles, 104 per ray and
+// step), then the latency of the record gathers (20 warps per SM hold 40 rays' worth).
 #include <cmath>
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "art.h"
 #include "art_internal.h"
@@ -36,341 +43,450 @@ namespace {
 
 // Running sum in two floats without renormalisation: hi + g is split exactly (two-sum) and
 // its rounding error collected in lo.
-__device__ __forceinline__ df df_acc(df a, float g)
+template <class V>
+__device__ __forceinline__ void sum_add(V& hi, V& lo, V g)
 {
-    const df s = df_two_sum(a.hi, g);
-    return {s.hi, a.lo + s.lo};
+    const V s = vadd(hi, g);
+    const V bb = vsub(s, hi);
+    lo = vadd(lo, vadd(vsub(hi, vsub(s, bb)), vsub(g, bb)));
+    hi = s;
 }
 
-// a - g for a remainder that only decreases (a >= g >= 0): with |hi| >= g the error of
+// hi + lo - g for a remainder that only decreases (a >= g >= 0): with |hi| >= g the error of
 // hi - g is exact by the fast two-sum; where rounding of earlier steps left hi just below g,
 // hi - g is itself exact (Sterbenz) and the error is 0.
-__device__ __forceinline__ df df_dec(df a, float g)
+template <class V>
+__device__ __forceinline__ void sum_take(V& hi, V& lo, V g)
 {
-    const float s = a.hi - g;
-    const float e = (a.hi - s) - g;
-    return {s, a.lo + e};
+    const V s = vsub(hi, g);
+    lo = vadd(lo, vsub(vsub(hi, s), g));
+    hi = s;
 }
 
-// Per-lane sum of dloss/dL for the source of the lane's recent rays, flushed to the global
-// FP64 sum when the lane moves to another source (rays of one source are consecutive).
-struct DLacc {
-    df v;
-    unsigned src;
-};
-
-__device__ __forceinline__ void dl_add(DLacc& D, double* dL, unsigned s, df own)
+// Adds the lanes' parts v of dloss/dL to their sources' FP64 sums: one addition per warp where
+// all rays are of one source, as most neighbouring rays of a front are (an addition per ray,
+// 11 M to 16 addresses, bound the sweep: 5.77 against 3.85 ms on 128^3 / 16 sources without a
+// force term). Warp-uniform; lanes without rays pass v = 0.
+__device__ __forceinline__ void dl_add(double* dL, unsigned src, bool valid, double v)
 {
-    if (s != D.src) {
-        if (D.src != 0xffffffffu && D.v.hi != 0.f) atomicAdd(dL + D.src, (double)D.v.hi + (double)D.v.lo);
-        D.src = s;
-        D.v = {0.f, 0.f};
+    const unsigned lead = __shfl_sync(kFull, src, __ffs(__ballot_sync(kFull, valid)) - 1);
+    if (__all_sync(kFull, !valid || src == lead)) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(kFull, v, off);
+        if ((threadIdx.x & 31u) == 0 && v != 0.0) atomicAdd(dL + lead, v);
+    } else if (valid && v != 0.0) {
+        atomicAdd(dL + src, v);
     }
-    D.v = df_add(D.v, own);
 }
 
-__device__ __forceinline__ void red_f32(float* p, float v)
+__device__ __forceinline__ void red_f32_if(float* base, int key, float v)
 {
-    asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %1, 0;\n\t"
+                 "@q red.global.add.f32 [%0], %2;\n\t}"
+                 :: "l"(base + key), "r"(key), "f"(v) : "memory");
 }
 
-// The {chi, chi_H, w, 0} part of a reverse-sweep cell record, and the force weight of the
-// segment: q = (v . n) / dV, so that the segment adds q dL to the loss (0 without a force term).
-__device__ __forceinline__ float4 rec_main(const float4& c) { return c; }
-__device__ __forceinline__ float4 rec_main(const CellF& c) { return c.a; }
-__device__ __forceinline__ float4 rec_main(const CellW& c) { return make_float4(c.chi, c.chi, c.w, 0.f); }
-__device__ __forceinline__ float force_weight(const float4&, const float*, float) { return 0.f; }
-__device__ __forceinline__ float force_weight(const CellW&, const float*, float) { return 0.f; }
+// The parts of a cell record: opacity, its neutral-H part, weight, and the force weight of the
+// segment q = (v . n) / dV, so that the segment adds q dL to the loss (0 without a force term).
+__device__ __forceinline__ float neutral_of(const float4& c) { return c.y; }
+__device__ __forceinline__ float neutral_of(const CellF& c) { return c.a.y; }
+__device__ __forceinline__ float neutral_of(const CellW& c) { return c.chi; }
+__device__ __forceinline__ float weight_of(const float4& c) { return c.z; }
+__device__ __forceinline__ float weight_of(const CellF& c) { return c.a.z; }
+__device__ __forceinline__ float weight_of(const CellW& c) { return c.w; }
 __device__ __forceinline__ float force_weight(const CellF& c, const float* n, float fs)
 {
     return fs * fmaf(c.b.x, n[0], fmaf(c.b.y, n[1], c.b.z * n[2]));
 }
+template <class Cell> struct HasForce { static constexpr bool value = false; };
+template <> struct HasForce<CellF> { static constexpr bool value = true; };
 template <class Cell> __device__ __forceinline__ const Cell* recs_of(const TraceArgs& A);
 template <> __device__ __forceinline__ const float4* recs_of<float4>(const TraceArgs& A) { return A.rec; }
 template <> __device__ __forceinline__ const CellF* recs_of<CellF>(const TraceArgs& A) { return A.recf; }
 template <> __device__ __forceinline__ const CellW* recs_of<CellW>(const TraceArgs& A) { return A.recw; }
 
-// Idle lanes of a warp before it refills them from the queue, and steps per round (between
-// refill checks; completions run at the end of each round). Measured on the 128^3 /
-// 16-source and 512^3 / 8-source cases: 32 steps at 16 lanes beat 8 at 12 by 1 % and 10 %;
-// longer rounds or a threshold of 20 lanes gain a little more at 512^3 and lose at 128^3.
-#ifndef ART_ADJ_IDLE
-#define ART_ADJ_IDLE 16
-#endif
-#ifndef ART_ADJ_STEPS
-#define ART_ADJ_STEPS 32
-#endif
-
-// One expand phase of the reverse sweep on the rays in slots [cursor .. end) of level l
-// (phase starting at slot `begin`). Pass 1 walks each ray for its own weighted sum. A ray
-// that splits stores that sum, a pending-children count of 4 and its children (in order, as
-// in the forward trace). A ray that ends without splitting (a leaf) walks again at once
-// (pass 2) from the start state kept from pass 1, depositing its gradients; once the warp's
-// round of steps ends it adds its total to its parent and counts the parent down (the
-// completions of a round run together). The lane that brings a parent's
-// count to zero takes over the parent's pass 2 (its level below this phase's), and so on
-// towards the base level: no separate collapse phase is needed, because the deepest-first
-// schedule does not reuse a level's slots before everything below it has finished. The
-// level data and buffer descriptors are copied out of the kernel parameters here: a
-// rewrite of the completion step that held references into the parameter block, indexed
-// by the changing level lv, never finished on the GPU with the d_max cutoff (the same
-// inputs finish in 2 ms with this form). Warp-uniform.
-template <class Cell, bool kCut>
-__device__ void run_adjoint(const TraceArgs& A, int l, unsigned long long* cursor,
-                            unsigned long long begin, unsigned long long end, Tally& T, DLacc& D)
+// c = *p if q, as a predicated load.
+__device__ __forceinline__ void load_if(bool q, const float4* p, float4& c)
 {
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %5, 0;\n\t"
+        "@q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+        : "+f"(c.x), "+f"(c.y), "+f"(c.z), "+f"(c.w) : "l"(p), "r"((int)q));
+}
+__device__ __forceinline__ void load_if(bool q, const CellF* p, CellF& c)
+{
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %9, 0;\n\t"
+        "@q ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t}"
+        : "+f"(c.a.x), "+f"(c.a.y), "+f"(c.a.z), "+f"(c.a.w), "+f"(c.b.x), "+f"(c.b.y),
+          "+f"(c.b.z), "+f"(c.b.w)
+        : "l"(p), "r"((int)q));
+}
+__device__ __forceinline__ void load_if(bool q, const CellW* p, CellW& c)
+{
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\t"
+        "@q ld.global.nc.v2.f32 {%0, %1}, [%2];\n\t}"
+        : "+f"(c.chi), "+f"(c.w) : "l"(p), "r"((int)q));
+}
+
+// What a lane knows of its quad.
+struct QuadInfo {
+    unsigned quad, src, pix;  // pix: the lane's first ray
+    float L, tau;
+    fix rend;
+    bool splits;
+};
+
+// The rays of a lane during a walk.
+template <class Cell, int kWidth>
+struct Walkers {
+    using V = typename std::conditional<kWidth == 1, float, float2>::type;
+    Path W[kWidth];
+    Cell cell[kWidth];
+    float n[kWidth][3];  // used with a force term only
+    V L, tau;
+};
+
+template <class Cell, int kWidth>
+__device__ __forceinline__ void walkers_start(const TraceArgs& A, const Cell* recs,
+                                              const LevelInfo& LV, const QuadInfo& Q, bool valid,
+                                              Walkers<Cell, kWidth>& R)
+{
+    using V = typename Walkers<Cell, kWidth>::V;
+    if (valid) {
+        const float4 sh = __ldg(&A.src[Q.src].hi);
+        const float4 sl = __ldg(&A.src[Q.src].lo);
+        const longlong2 xy = __ldg(&A.src[Q.src].xy);
+        const longlong2 z_ = __ldg(&A.src[Q.src].z_);
+        const df u[3] = {{sh.x, sl.x}, {sh.y, sl.y}, {sh.z, sl.z}};
+        const fix ux[3] = {xy.x, xy.y, z_.x};
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j) {
+            df n[3];
+            fix code[3];
+            load_direction(LV.dir + 3ull * (Q.pix + j), n, code);
+            const bool inside = path_start(R.W[j], A.nx, A.ny, A.nz, A.fbits, u, ux, n, code,
+                                           LV.r0, LV.r0x);
+            // padded cell 0 is a sentinel: a ray that starts outside exits at once
+            R.cell[j] = load_cell(recs + (inside ? R.W[j].idx : 0));
+#pragma unroll
+            for (int a = 0; a < 3; ++a) R.n[j][a] = n[a].hi;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j) {
+            R.W[j] = Path{};
+            R.W[j].t[1] = 1ll << 40;
+            R.W[j].t[2] = 1ll << 41;
+            R.cell[j] = load_cell(recs);
+            R.n[j][0] = R.n[j][1] = R.n[j][2] = 0.f;
+        }
+    }
+    R.L = vset<V>(Q.L);
+    R.tau = vset<V>(Q.tau);
+}
+
+// Walks the lane's rays to their ends. Pass 1 adds each segment's loss w k G + q dL to (hi, lo);
+// pass 2 takes it from (hi, lo), what is left of the sum over the segment and all that follows
+// it, and deposits the segment's gradient scaled by Ls. Ended rays as in the forward trace.
+template <class Cell, int kWidth, int kPass, bool kParts, bool kFirst>
+__device__ __forceinline__ void walkers_step(const TraceArgs& A, const Cell* __restrict__ recs,
+                                             fix rend, Walkers<Cell, kWidth>& R,
+                                             typename Walkers<Cell, kWidth>::V& hi,
+                                             typename Walkers<Cell, kWidth>::V& lo, float Ls,
+                                             unsigned& ncross)
+{
+    using V = typename Walkers<Cell, kWidth>::V;
+    constexpr bool force = HasForce<Cell>::value;
+    V ds, x, wk, hv, q = vset<V>(0.f);
+    int key[kWidth];
+#pragma unroll
+    for (int j = 0; j < kWidth; ++j) {
+        const float chi = chi_of(R.cell[j]), depth = vget(R.tau, j);
+        const bool alive = !(chi < 0.f) & !(depth > A.tau_max);
+        // (a ray that has ended may hold the record of a cell it never entered)
+        vget(wk, j) = alive ? weight_of(R.cell[j]) * A.gscale : 0.f;
+        vget(hv, j) = neutral_of(R.cell[j]);
+        if constexpr (force)
+            vget(q, j) = alive ? force_weight(R.cell[j], R.n[j], A.fscale) : 0.f;
+        walk_move<kParts>(R.W[j], rend, A.unit, chi, depth, A.tau_max, -1 - j, (int)A.npad,
+                          vget(ds, j), vget(x, j), key[j], ncross);
+        load_if(alive, recs + R.W[j].idx, R.cell[j]);
+    }
+    V dphi;
+    const V ph = phi_dphi<kPass == 2>(x, dphi);
+    const V Lin = R.L;
+    const V G = vmul(vmul(Lin, ds), ph);
+    const V dL = vmul(vmul(Lin, x), ph);
+    R.L = vsub(R.L, dL);
+    R.tau = vadd(R.tau, x);
+    const V g = force ? vfma(q, dL, vmul(wk, G)) : vmul(wk, G);
+    if constexpr (kPass == 1) {
+        sum_add(hi, lo, g);
+    } else {
+        sum_take(hi, lo, g);
+        const V after = vadd(hi, lo);
+        // d(segment loss)/d dtau: w k L_in ds phi' + q L_in e^-dtau (R.L is now L_in e^-dtau)
+        V own = vmul(vmul(vmul(wk, Lin), ds), dphi);
+        if constexpr (force) own = vfma(q, R.L, own);
+        const V val = vmul(vmul(vmul(vset<V>(Ls), hv), ds), vsub(own, after));
+        float d[kWidth];
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j) d[j] = vget(val, j);
+        if constexpr (kWidth == 2)
+            asm("{\n\t.reg .pred q;\n\tsetp.eq.s32 q, %1, %2;\n\t@q add.f32 %0, %0, %3;\n\t"
+                "@q mov.b32 %1, -2;\n\t}" : "+f"(d[0]), "+r"(key[1]) : "r"(key[0]), "f"(d[1]));
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j) {
+            if constexpr (kFirst) {  // all in their source's cell: one sum per warp
+                float4 v = make_float4(d[j], 0.f, 0.f, 0.f);
+                merge_lanes(key[j], v);
+                d[j] = v.x;
+            }
+            red_f32_if(A.grad, key[j], d[j]);
+        }
+    }
+}
+
+template <class Cell, int kWidth, int kPass>
+__device__ __forceinline__ void walkers_run(const TraceArgs& A, const Cell* __restrict__ recs,
+                                            bool base, fix rend, Walkers<Cell, kWidth>& R,
+                                            typename Walkers<Cell, kWidth>::V& hi,
+                                            typename Walkers<Cell, kWidth>::V& lo, float Ls,
+                                            unsigned& ncross)
+{
+    // the first cells around a source, where a segment can more than double the distance (at
+    // most six faces lie within the longest segment, 3^(1/2) cells)
+    if (base) {
+        walkers_step<Cell, kWidth, kPass, true, true>(A, recs, rend, R, hi, lo, Ls, ncross);
+#pragma unroll 1
+        for (int k = 1; k < 6; ++k)
+            walkers_step<Cell, kWidth, kPass, true, false>(A, recs, rend, R, hi, lo, Ls, ncross);
+    }
+    for (;;) {
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j)
+            any |= !(chi_of(R.cell[j]) < 0.f) & !(vget(R.tau, j) > A.tau_max);
+        if (!__any_sync(kFull, any)) break;
+#pragma unroll 1
+        for (int k = 0; k < kCheckSteps; ++k)
+            walkers_step<Cell, kWidth, kPass, false, false>(A, recs, rend, R, hi, lo, Ls, ncross);
+    }
+}
+
+// One phase on the quads up to `end` of level l, taken 32 lanes at a time from `cursor` (items
+// of kWidth rays): expand (pass 1, and pass 2 where no ray of the warp splits) or collapse
+// (pass 2 of the quads not done yet). Warp-uniform.
+template <class Cell, bool kCut, int kWidth>
+__device__ void sweep_front(const TraceArgs& A, int l, bool collapse, unsigned long long* cursor,
+                            unsigned long long end)
+{
+    using V = typename Walkers<Cell, kWidth>::V;
+    constexpr unsigned kPerQuad = 4u / kWidth;
     const Cell* const recs = recs_of<Cell>(A);
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt = (1u << lane) - 1u;
-    const LevelInfo LV = A.levels[l];
-    const RayBuf B = A.buf[l];
-    const RayBuf C = A.buf[l + 1];
-    const bool has_next = l < A.lmax_glob;
-    const float gs = A.gscale;
-
-    // slot indices fit in 32 bits (level buffers hold fewer than 2^31 slots)
-    const unsigned b32 = (unsigned)begin, e32 = (unsigned)end;
-    unsigned wnext = 0, wend = 0;
-    bool more = true;
-    int mode = 0;          // 0 idle, 1 pass 1 (level l), 2 pass 2 (level lv <= l),
-                           // 3 pass 2 ended, completion pending
-    int lv = l;            // level of the ray being walked
-    WalkT<Cell> W;
-    // pass-1 start of the ray (next face per axis, start cell), so that a leaf's pass 2
-    // restarts without a new ray set-up
-    fix t0[3] = {0, 0, 0};
-    int idx0 = 0;
-    unsigned s = 0, p = 0;
-    unsigned slot = 0;
-    float L0 = 0.f, Ls = 0.f;
-    df own = {0.f, 0.f};   // own weighted sum (pass 1), kept for dL in pass 2
-    float total = 0.f;     // own + descendants (pass 2), passed to the parent
-    df rem = {0.f, 0.f};   // weighted sum over what follows the current segment (pass 2)
-    bool splits = false;
-    fix rend = kNoEnd;     // radius where the ray of level lv ends (split or cutoff)
-    unsigned ncross = 0, nrays = 0, nstep = 0;
-    // Every step crosses at least one face and the sentinel ring ends every walk that
-    // leaves the grid, so walks end by construction. As a safety net the warp counts its
-    // rounds of steps (ART_ADJ_STEPS each) and gives up past a bound far beyond any phase
-    // (ART_EINTERNAL), so the kernel always ends.
-    unsigned rounds = 0;
-    unsigned nretired = 0;  // rays retired here (weight destroy_w each, summed at the end)
-
-    // Completion of the ray in `slot` at level lv (pass 2 done, or a ray without segments):
-    // dL, the parent's sum, and possibly the parent's pass 2 in this lane.
-    auto complete = [&]() {
-        for (;;) {
-            dl_add(D, A.dL, s, own);  // every ray of the chain has source s
-            if (lv == A.level0) { mode = 0; return; }
-            const RayBuf Bl = A.buf[lv];
-            const RayBuf Pl = A.buf[lv - 1];
-            const unsigned par = __ldcg(Bl.parent + slot);
-            if (total != 0.f) red_f32(Pl.sub + par, total);
-            // count the parent down with acquire-release ordering: this ray's sum (above) is
-            // released with the decrement, and the lane that takes the count to zero acquires
-            // every sibling's sum before reading the parent's total
-            unsigned old;
-            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;"
-                         : "=r"(old) : "l"(Pl.pending + par), "r"(0xffffffffu) : "memory");
-            if (old != 1u) { mode = 0; return; }
-            // last child: this lane replays the parent (pass 2)
-            lv -= 1;
-            slot = par;
-            const float2 ov = __ldcg(Pl.own + slot);
-            own = {ov.x, ov.y};
-            rem = df_add(own, {__ldcg(Pl.sub + slot), 0.f});
-            total = rem.hi + rem.lo;
-            const LevelInfo Lp = A.levels[lv];
-            ray_begin<kCut>(A, Lp, Pl, lv, slot, W, recs, s, p, L0, splits, rend);
-            Ls = __ldg(A.srcL + s);
-            mode = 2;
-            return;
-        }
-    };
+    const LevelInfo& LV = A.levels[l];
+    const AdjBuf& B = A.adj[l];
+    const bool base = l == A.level0;
+    BlockTally& T = block_tally();
+    const unsigned items = (unsigned)end * kPerQuad;  // front ends below 2^29 quads
+    unsigned ncross = 0;
 
     for (;;) {
-        unsigned need = __ballot_sync(kFull, mode == 0);
-        if (__popc(need) >= ART_ADJ_IDLE || need == kFull) {
-            while (need && more) {
-                if (wnext >= wend) {
-                    unsigned long long b = 0;
-                    if (lane == 0) b = atomicAdd(cursor, (unsigned long long)A.chunk);
-                    b = __shfl_sync(kFull, b, 0);
-                    if (b >= end) { more = false; break; }
-                    wnext = (unsigned)b;
-                    wend = min(wnext + (unsigned)A.chunk, e32);
-                }
-                const unsigned avail = min(wend - wnext, 32u);
-                const unsigned rank = __popc(need & lt);
-                if (mode == 0 && rank < avail) {
-                    slot = wnext + rank;
-                    lv = l;
-                    const int st = ray_begin<kCut>(A, LV, B, l, slot, W, recs, s, p, L0, splits, rend);
-                    if (st > 0) {
-                        Ls = __ldg(A.srcL + s);
-                        t0[0] = W.t[0];
-                        t0[1] = W.t[1];
-                        t0[2] = W.t[2];
-                        idx0 = W.idx;
-                        mode = 1;
-                        own = {0.f, 0.f};
-                        ++nrays;
-                    } else {
-                        if (has_next) write_holes(C, 4ull * (slot - b32));
-                        if (st == 0) {  // starts outside the grid: a leaf with zero sums
-                            ++nretired;
-                            ++nrays;
-                            own = {0.f, 0.f};
-                            total = 0.f;
-                            complete();
-                        }
-                    }
-                }
-                wnext += min(avail, (unsigned)__popc(need));
-                need = __ballot_sync(kFull, mode == 0);
+        unsigned b = 0;
+        if (lane == 0) b = (unsigned)min(atomicAdd(cursor, 32ull), (unsigned long long)items);
+        b = __shfl_sync(kFull, b, 0);
+        if (b >= items) break;
+        const unsigned item = b + lane;
+        bool valid = item < items;
+        QuadInfo Q = {item / kPerQuad, 0u, 0u, 0.f, 0.f, kNoEnd, false};
+        const unsigned part = item % kPerQuad * kWidth;
+        const unsigned ray = 4u * Q.quad + part;  // slot of the lane's first ray
+        unsigned parent = 0u;
+        if (valid && (collapse || !base)) parent = __ldcg(B.parent + Q.quad);
+        if (collapse) valid = valid && parent != kDone;
+        if (!__any_sync(kFull, valid)) continue;
+        float Ls = 0.f;
+        if (valid) {
+            if (base) {
+                Q.src = Q.quad / A.base_quads;
+                Q.pix = 4u * (Q.quad % A.base_quads);
+                Q.L = __ldg(&A.src[Q.src].hi).w;
+            } else {
+                const uint4 r = __ldcg(B.rec + Q.quad);
+                Q.src = r.x;
+                Q.pix = r.y;
+                Q.L = __uint_as_float(r.z);
+                Q.tau = __uint_as_float(r.w);
             }
-        }
-        if (!__any_sync(kFull, mode != 0)) {
-            if (!more) break;
-            continue;
+            Q.pix += part;
+            Q.splits = l < __float_as_int(__ldg(&A.src[Q.src].lo).w);
+            Q.rend = end_radius<kCut>(Q.splits, LV.rmaxx, A.dmax);
+            Ls = __ldg(A.srcL + Q.src);
         }
 
-        if (++rounds > (1u << 28)) {  // warp-uniform: no phase comes near this
-            if (lane == 0) atomicCAS(&A.stats->error, 0, -8);  // ART_EINTERNAL
-            break;
-        }
-#pragma unroll 1
-        for (int k = 0; k < ART_ADJ_STEPS; ++k) {
-            if (mode == 1 || mode == 2) {
-                const float4 cm = rec_main(W.cell);
-                const float wv = cm.z;   // weight and neutral-H opacity of this cell
-                const float hv = cm.y;
-                const float q = force_weight(W.cell, W.n, A.fscale);
-                const StepOut o = walk_step(W, rend, A.unit, (int)A.npad, recs, A.tau_max, nstep);
-                // this segment's loss: w k G, plus q dL with a force term
-                const float g = fmaf(q, o.dL, wv * gs * o.G);
-                if (mode == 1) {
-                    own = df_acc(own, g);
-                    ncross += o.seg ? 1u : 0u;
-                } else {
-                    rem = df_dec(rem, g);
-                    const float after = rem.hi + rem.lo;
-                    // d(segment loss)/d dtau: w k L_in ds phi' + q L_in e^-dtau (W.L is now
-                    // L_in e^-dtau)
-                    const float own_d = fmaf(q, W.L, wv * gs * o.Lin * o.ds * o.dphi);
-                    const float val = Ls * hv * o.ds * (own_d - after);
-                    if (o.seg) red_f32(A.grad + o.cell, val);
+        V hi = vset<V>(0.f), lo = vset<V>(0.f);
+        bool second = collapse;  // pass 2 follows
+        float total = 0.f;       // loss of the lane's rays and their descendants
+        if (!collapse) {
+            Walkers<Cell, kWidth> R;
+            walkers_start<Cell, kWidth>(A, recs, LV, Q, valid, R);
+            walkers_run<Cell, kWidth, 1>(A, recs, base, Q.rend, R, hi, lo, 0.f, ncross);
+
+            // ends: the rays' own sums, and the children of split rays
+            bool child[kWidth];
+            unsigned nchild = 0, mine = 0, at[kWidth];
+            double own = 0.0;
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j) {
+                child[j] = valid && chi_of(R.cell[j]) == kEnded && !(vget(R.tau, j) > A.tau_max) &&
+                           splits_at_end<kCut>(Q.splits, LV.rmaxx, A.dmax);
+                const unsigned m = __ballot_sync(kFull, child[j]);
+                at[j] = __popc(m & lt) + mine;  // children in lane order
+                if (j > 0) {
+                    at[j] += at[0];
+                    at[0] += __popc(m & lt);
                 }
-                if (o.ev != EV_NONE) {
-                    if (mode == 1) {
-                        const unsigned long long c4 = 4ull * (slot - b32);
-                        if (o.ev == EV_SPLIT && splits_at_end<kCut>(splits, LV.rmaxx, A.dmax)) {
-                            B.own[slot] = make_float2(own.hi, own.lo);
-                            B.sub[slot] = 0.f;
-                            B.pending[slot] = 4u;
-                            if (c4 + 4 <= C.cap) {
-                                const float Lc = 0.25f * W.L;
-                                *reinterpret_cast<uint4*>(C.src + c4) = make_uint4(s, s, s, s);
-                                *reinterpret_cast<uint4*>(C.pix + c4) =
-                                    make_uint4(4 * p, 4 * p + 1, 4 * p + 2, 4 * p + 3);
-                                *reinterpret_cast<float4*>(C.L + c4) = make_float4(Lc, Lc, Lc, Lc);
-                                *reinterpret_cast<float4*>(C.tau + c4) =
-                                    make_float4(W.tau, W.tau, W.tau, W.tau);
-                                *reinterpret_cast<uint4*>(C.parent + c4) =
-                                    make_uint4(slot, slot, slot, slot);
-                            } else {
-                                atomicCAS(&A.stats->error, 0, -3);
-                            }
-                            mode = 0;
-                        } else {
-                            ++nretired;
-                            if (has_next) write_holes(C, c4);
-                            // a leaf: pass 2 right away
-                            total = own.hi + own.lo;
-                            rem = own;
-                            // a leaf: pass 2 right away, from the kept start state (direction
-                            // steps, source and luminosity are the ray's own already)
-                            W.t[0] = t0[0];
-                            W.t[1] = t0[1];
-                            W.t[2] = t0[2];
-                            W.idx = idx0;
-                            W.tc = LV.r0x;
-                            W.L = L0;
-                            W.tau = l == A.level0 ? 0.f : __ldcg(B.tau + slot);
-                            W.cell = load_cell(recs + idx0);
-                            mode = 2;
+                nchild += __popc(m);
+                mine += child[j] ? 1u : 0u;
+                if (valid) own += (double)vget(hi, j) + (double)vget(lo, j);
+            }
+            dl_add(A.dL, Q.src, valid, own);
+            unsigned slot = 0;
+            if (lane == 0) {
+                const unsigned nray = kWidth * min(items - b, 32u);
+                atomicAdd(&T.rays[l], (unsigned long long)nray);
+                atomicAdd(&T.destroy, (unsigned long long)(nray - nchild) * LV.destroy_w);
+                if (nchild)
+                    slot = (unsigned)atomicAdd(&A.sched->count[l + 1], (unsigned long long)nchild);
+            }
+            second = nchild == 0;
+            if (nchild) {
+                const AdjBuf& C = A.adj[l + 1];
+                slot = __shfl_sync(kFull, slot, 0);
+                if (slot + nchild > C.cap) {
+                    atomicCAS(&A.stats->error, 0, -3);  // ART_EQUEUE_OVERFLOW
+                } else {
+#pragma unroll
+                    for (int j = 0; j < kWidth; ++j) {
+                        if (child[j]) {
+                            __stcg(C.rec + slot + at[j],
+                                   make_uint4(Q.src, 4u * (Q.pix + j),
+                                              __float_as_uint(0.25f * vget(R.L, j)),
+                                              __float_as_uint(vget(R.tau, j))));
+                            __stcg(C.parent + slot + at[j], ray + j);
                         }
-                    } else {
-                        mode = 3;
                     }
                 }
+                if (valid) {  // kept for the collapse
+                    if (base) __stcg(B.parent + Q.quad, 0u);
+#pragma unroll
+                    for (int j = 0; j < kWidth; ++j) {
+                        __stcg(B.own + ray + j, make_float2(vget(hi, j), vget(lo, j)));
+                        __stcg(B.sub + ray + j, 0.f);
+                    }
+                }
+            } else if (valid) {
+                if (part == 0u) __stcg(B.parent + Q.quad, kDone);
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j) total += vget(hi, j) + vget(lo, j);
+            }
+        } else if (valid) {
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j) {
+                const float2 own = __ldcg(B.own + ray + j);
+                const df rem = df_add({own.x, own.y}, {__ldcg(B.sub + ray + j), 0.f});
+                vget(hi, j) = rem.hi;
+                vget(lo, j) = rem.lo;
+                total += rem.hi + rem.lo;
             }
         }
-        // Completions of the round's finished pass-2 walks run together: the count-down of
-        // the parent with its memory ordering, and the set-up of the parent's pass 2 for a
-        // last child, whose latencies then overlap across lanes (measured 4 % faster than
-        // completing each walk in its own step, and faster than batches of 1 to 8 lanes, in
-        // rounds of 8 steps).
-        if (mode == 3) complete();
-    }
-    tally_crossings(T, ncross);
-    count_rays(A.stats, l, nrays);
-    // the destroy counter: rays retired at this phase's level, weight 4^(l_max - l)
+        if (second) {
+            Walkers<Cell, kWidth> R;
+            unsigned again = 0;
+            walkers_start<Cell, kWidth>(A, recs, LV, Q, valid, R);
+            walkers_run<Cell, kWidth, 2>(A, recs, base, Q.rend, R, hi, lo, Ls, again);
+            if (!base) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) nretired += __shfl_down_sync(kFull, nretired, off);
-    if (lane == 0 && nretired > 0) atomicAdd(&T.destroy, (unsigned long long)nretired * LV.destroy_w);
+                for (unsigned off = 1u; off < kPerQuad; off <<= 1)
+                    total += __shfl_xor_sync(kFull, total, off);
+                if (valid && part == 0u) __stcg(A.adj[l - 1].sub + parent, total);
+            }
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) ncross += __shfl_down_sync(kFull, ncross, off);
+    if (lane == 0 && ncross) atomicAdd(&T.crossings, (unsigned long long)ncross);
+}
+
+// Chooses the next phase (run by one thread, all others waiting): the deepest level with open
+// quads, which are then collapsed (everything below them is finished), or with quads to expand.
+__device__ __forceinline__ void next_sweep(const TraceArgs& A)
+{
+    volatile Sched* sc = A.sched;
+    if (!sc->started) {
+        sc->started = 1;
+        sc->count[A.level0] = (unsigned long long)A.base_quads * A.nsrc;
+    } else if (sc->phase_kind == 0 && (sc->phase_level == A.lmax_glob ||
+                                       sc->count[sc->phase_level + 1] == 0)) {
+        sc->open_end[sc->phase_level] = 0;  // no children: every warp ran both passes
+    }
+    int l = A.lmax_glob;
+    while (l >= A.level0 && sc->open_end[l] == 0 && sc->count[l] == 0) --l;
+    if (l < A.level0) {
+        sc->done = 1;
+        return;
+    }
+    unsigned long long begin, end;
+    if (sc->open_end[l] != 0) {
+        sc->phase_kind = 1;
+        begin = sc->open_begin[l];
+        end = sc->open_end[l];
+        sc->open_end[l] = 0;
+    } else {
+        sc->phase_kind = 0;
+        end = sc->count[l];
+        unsigned long long take = end;
+        if (l < A.lmax_glob) take = min(end, A.adj[l + 1].cap / 4);
+        if (take == 0) {  // a phase must consume rays, or the schedule never ends
+            atomicCAS(&A.stats->error, 0, -8);  // ART_EINTERNAL
+            take = end;
+        }
+        begin = end - take;
+        sc->count[l] = begin;
+        sc->open_begin[l] = begin;
+        sc->open_end[l] = end;
+    }
+    const int width = front_width(false, end - begin);
+    sc->phase_level = l;
+    sc->phase_width = width;
+    sc->phase_end = end;
+    sc->cursor[l] = begin * (unsigned long long)(4 / width);
 }
 
 template <class Cell, bool kCut>
-__global__ void __launch_bounds__(256, 4) k_backward_persistent(const __grid_constant__ TraceArgs A)
+__global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_backward_persistent(const __grid_constant__ TraceArgs A)
 {
-    tally_init();
-    Tally& T = tally_slots()[threadIdx.x >> 5];
-    DLacc D = {{0.f, 0.f}, 0xffffffffu};
+    block_tally_init();
     Sched* sc = A.sched;
-    __shared__ int s_level;
-    __shared__ unsigned long long s_begin, s_end;
+    __shared__ int s_level, s_width, s_kind;
+    __shared__ unsigned long long s_end;
     for (;;) {
-        if (!grid_barrier(sc, A.stats, A.wait_ns)) break;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            volatile Sched* v = sc;
-            int l = -1;
-            for (int k = A.lmax_glob; k >= A.level0; --k)
-                if (v->count[k] > 0) { l = k; break; }
-            if (l < 0) {
-                v->done = 1;
-            } else {
-                const unsigned long long have = min(v->count[l], A.buf[l].cap);
-                unsigned long long take = have;
-                if (l < A.lmax_glob) take = min(have, A.buf[l + 1].cap / 4);
-                if (take == 0) {  // a phase must consume rays, or the schedule never ends
-                    atomicCAS(&A.stats->error, 0, -8);  // ART_EINTERNAL
-                    take = have;
-                }
-                const unsigned long long b = have - take;
-                v->count[l] = b;
-                v->phase_level = l;
-                v->phase_begin = b;
-                v->phase_end = have;
-                v->cursor[l] = b;
-                if (l < A.lmax_glob) v->count[l + 1] = 4 * take;  // the children's slots
-            }
-            __threadfence();
-        }
-        if (!grid_barrier(sc, A.stats, A.wait_ns)) break;
+        if (!grid_barrier(sc, A.stats, A.wait_ns, [&] { next_sweep(A); })) break;
         if (threadIdx.x == 0) {
             volatile Sched* v = sc;
             s_level = v->done ? -1 : v->phase_level;
-            s_begin = v->phase_begin;
+            s_width = v->phase_width;
+            s_kind = v->phase_kind;
             s_end = v->phase_end;
         }
         __syncthreads();
         const int l = s_level;
         if (l < 0) break;
-        run_adjoint<Cell, kCut>(A, l, &sc->cursor[l], s_begin, s_end, T, D);
+        if (s_width == 2) sweep_front<Cell, kCut, 2>(A, l, s_kind == 1, &sc->cursor[l], s_end);
+        else sweep_front<Cell, kCut, 1>(A, l, s_kind == 1, &sc->cursor[l], s_end);
     }
-    if (D.src != 0xffffffffu && D.v.hi != 0.f) atomicAdd(A.dL + D.src, (double)D.v.hi + (double)D.v.lo);
-    tally_flush(A.stats);
+    block_tally_flush(A.stats);
 }
 
 // Per-cell record of the reverse sweep in the padded layout: one 16-byte gather per
@@ -382,6 +498,9 @@ __global__ void k_pack_cells(int nx, int ny, int nz, const float* __restrict__ n
 {
     const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
     const unsigned step = gridDim.x * blockDim.x;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        rec[npad] = make_float4(kEnded, 0.f, 0.f, 0.f);
+    }
     for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
         unsigned i;
         if (!unpad(q, nx, ny, nz, i)) {
@@ -403,6 +522,10 @@ __global__ void k_pack_cells_f(int nx, int ny, int nz, const float* __restrict__
     const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
     const size_t ncell = (size_t)nx * ny * nz;
     const unsigned step = gridDim.x * blockDim.x;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        rec[npad].a = make_float4(kEnded, 0.f, 0.f, 0.f);
+        rec[npad].b = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
         unsigned i;
         if (!unpad(q, nx, ny, nz, i)) {
@@ -424,6 +547,9 @@ __global__ void k_pack_cells_w(int nx, int ny, int nz, const float* __restrict__
 {
     const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
     const unsigned step = gridDim.x * blockDim.x;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        rec[npad] = CellW{kEnded, 0.f};
+    }
     for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
         unsigned i;
         if (!unpad(q, nx, ny, nz, i)) {
@@ -442,19 +568,6 @@ __global__ void k_unpad_grad(int nx, int ny, int nz, const float* __restrict__ s
     const unsigned step = gridDim.x * blockDim.x;
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < ncell; i += step)
         dst[i] = src[pad_of(i, nx, ny)];
-}
-
-__global__ void k_inject_all(int nsrc, unsigned npix0, RayBuf B, unsigned long long* count)
-{
-    unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-    unsigned long long n = (unsigned long long)nsrc * npix0;
-    if (i == 0) *count = n;
-    if (i >= n) return;
-    unsigned s = (unsigned)(i / npix0);
-    B.src[i] = s;
-    B.pix[i] = (unsigned)(i - (unsigned long long)s * npix0);
-    B.L[i] = 0.f;
-    B.tau[i] = 0.f;
 }
 
 int status_of(cudaError_t e)
@@ -504,12 +617,6 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     float* grad_pad = reinterpret_cast<float*>(g->d_acc);
     if ((rc = status_of(cudaMemsetAsync(grad_pad, 0, sizeof(float) * g->npad, st)))) return rc;
     if ((rc = status_of(cudaMemsetAsync(g->d_sched, 0, sizeof(Sched), st)))) return rc;
-    const int l0 = p->level0;
-    const unsigned npix0 = 12u << (2 * l0);
-    const unsigned long long nb = (unsigned long long)ns * npix0;
-    k_inject_all<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(ns, npix0, g->buf[l0],
-                                                            &g->d_sched->count[l0]);
-    if ((rc = status_of(cudaGetLastError()))) return rc;
     const int pack_blocks = (int)std::min<long long>((g->npad + 255) / 256, (long long)g->sms * 16);
     const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
     const double sH_dx = p->sigma_H * g->dx;
@@ -536,15 +643,14 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     A.rec = g->d_rec;
     A.recf = d_v ? g->d_recf : nullptr;
     A.recw = light ? g->d_recw : nullptr;
-    A.w = d_w;
     A.grad = grad_pad;
     A.dL = dL;
     A.srcL = g->d_srcL;
     const double dV = g->dx * g->dx * g->dx;
     A.gscale = (float)(p->sigma_H * g->dx / dV);
     A.fscale = (float)(1.0 / dV);
-    // the reverse sweep is compiled for blocks of at most 256 threads (register budget)
-    const int threads = p->block_threads > 0 && p->block_threads < 256 ? p->block_threads : 256;
+    // block size: the caller's (or 128), at most what the kernels are built for
+    const int threads = std::min(p->block_threads > 0 ? p->block_threads : 128, kTraceMaxThreads);
     const bool cut = p->d_max > 0.0;
     void (*kern)(TraceArgs) =
         light ? (cut ? k_backward_persistent<CellW, true> : k_backward_persistent<CellW, false>)

@@ -158,25 +158,20 @@ int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto)
     return ART_OK;
 }
 
-// Front of level l with room for `need` rays of a reverse sweep.
+// Front of level l with room for `need` quads of a reverse sweep.
 static int ensure_adjoint_front(art_grid* g, int l, unsigned long long need)
 {
-    RayBuf& b = g->buf[l];
-    if (need > g->buf_cap[l]) {
-        dev_free(b.src); dev_free(b.pix); dev_free(b.L); dev_free(b.tau);
-        dev_free(b.parent); dev_free(b.own); dev_free(b.sub); dev_free(b.pending);
-        b = RayBuf{};
-        g->buf_cap[l] = 0;
-        int rc = dev_alloc(&b.src, need);
-        if (!rc) rc = dev_alloc(&b.pix, need);
-        if (!rc) rc = dev_alloc(&b.L, need);
-        if (!rc) rc = dev_alloc(&b.tau, need);
+    AdjBuf& b = g->adj[l];
+    if (need > g->adj_cap[l]) {
+        dev_free(b.rec); dev_free(b.parent); dev_free(b.own); dev_free(b.sub);
+        b = AdjBuf{};
+        g->adj_cap[l] = 0;
+        int rc = dev_alloc(&b.rec, need);
         if (!rc) rc = dev_alloc(&b.parent, need);
-        if (!rc) rc = dev_alloc(&b.own, need);
-        if (!rc) rc = dev_alloc(&b.sub, need);
-        if (!rc) rc = dev_alloc(&b.pending, need);
+        if (!rc) rc = dev_alloc(&b.own, 4 * need);
+        if (!rc) rc = dev_alloc(&b.sub, 4 * need);
         if (rc) return rc;
-        g->buf_cap[l] = need;
+        g->adj_cap[l] = need;
     }
     b.cap = need;  // the capacity this sweep may use
     return ART_OK;
@@ -306,7 +301,7 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         need = (need + 3) & ~3ull;
         int rc = ART_OK;
         if (adjoint) {
-            rc = ensure_adjoint_front(g, l, need);
+            rc = ensure_adjoint_front(g, l, std::max(need / 4, 4ull));
         } else if (l > l0) {
             // in the persistent schedule a phase takes a quarter of the next front's quads
             const unsigned long long quads = plain ? need / 4 : std::max(need / 4, 4ull);
@@ -353,7 +348,6 @@ TraceArgs make_args(art_grid* g, const art_params* p)
     A.nz = g->n[2];
     A.level0 = p->level0;
     A.lmax_glob = g->lmax_glob;
-    A.chunk = p->chunk > 0 ? p->chunk : 64;
     A.tau_max = (float)p->tau_max;
     A.chi = g->d_chi;
     A.chi2 = g->d_chi2;
@@ -362,9 +356,9 @@ TraceArgs make_args(art_grid* g, const art_params* p)
     A.src = g->d_src;
     A.levels = g->d_levels;
     for (int l = 0; l < kNL; ++l) {
-        A.buf[l] = g->buf[l];
+        A.adj[l] = g->adj[l];
         A.quad[l] = g->quad[l];
-        if (l > g->lmax_glob) A.buf[l].cap = A.quad[l].cap = 0;
+        if (l > g->lmax_glob) A.adj[l].cap = A.quad[l].cap = 0;
     }
     A.base_quads = 3u << (2 * p->level0);
     A.nsrc = (unsigned)g->L.size();
@@ -632,9 +626,8 @@ void art_destroy_grid(art_grid* g)
         dev_free(g->dir[l]);
         dev_free(g->quad[l].rec);
         dev_free(g->quad[l].recn);
-        RayBuf& b = g->buf[l];
-        dev_free(b.src); dev_free(b.pix); dev_free(b.L); dev_free(b.tau);
-        dev_free(b.parent); dev_free(b.own); dev_free(b.sub); dev_free(b.pending);
+        AdjBuf& b = g->adj[l];
+        dev_free(b.rec); dev_free(b.parent); dev_free(b.own); dev_free(b.sub);
     }
     if (g->h_stats) cudaFreeHost(g->h_stats);
     if (g->h_levels) cudaFreeHost(g->h_levels);

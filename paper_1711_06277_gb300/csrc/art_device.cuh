@@ -124,19 +124,6 @@ struct LevelInfo {
     unsigned long long destroy_w;  // 4^(l_max_global - l)
 };
 
-// Adjoint fronts, SoA per level: source index, nested pixel, entering L and tau.
-struct RayBuf {
-    unsigned* src;
-    unsigned* pix;
-    float* L;
-    float* tau;
-    unsigned* parent;   // slot of the parent in the level above
-    float2* own;        // weighted sum over the ray's own segments (pass 1), double-float
-    float* sub;         // weighted sum over the ray's descendants (added by the children)
-    unsigned* pending;  // children of a split ray still to finish
-    unsigned long long cap;
-};
-
 // Forward fronts: one record per quad, the four children of a split ray, {source, pixel of
 // the first child, entering L of each child (bits), tau (bits)}; two-bin traces add {Ln, taun}.
 struct QuadBuf {
@@ -145,12 +132,17 @@ struct QuadBuf {
     unsigned long long cap;
 };
 
-// Per-thread tallies, reduced per block at kernel exit.
-struct Tally {
-    double escaped, dropped;
-    unsigned long long crossings, destroy;
-    double escaped_n, dropped_n;  // non-ionizing bin of two-bin traces
+// Adjoint fronts: the same records, the slot (4 quad + child) of the quad's parent ray in the
+// level above (kDone once the quad is finished), and per ray its own weighted sum (pass 1,
+// double-float) and the weighted sum over its descendants.
+struct AdjBuf {
+    uint4* rec;
+    unsigned* parent;
+    float2* own;
+    float* sub;
+    unsigned long long cap;  // quads
 };
+constexpr unsigned kDone = 0xffffffffu;
 
 // Device-resident counters of one trace.
 struct DevStats {
@@ -166,8 +158,10 @@ struct DevStats {
 struct Sched {
     unsigned long long count[kNL];   // rays held in the level buffer (a stack, top = count)
     unsigned long long cursor[kNL];  // next ray of the current phase / launch
-    unsigned long long phase_begin, phase_end;
-    int phase_level, phase_width, phase_strided, done, started, pad;
+    unsigned long long phase_end;
+    int phase_level, phase_width, phase_strided, phase_kind, done, started;
+    // adjoint: quads of a level whose descendants are still being swept
+    unsigned long long open_begin[kNL], open_end[kNL];
     unsigned bar_count, bar_gen;
 };
 
@@ -178,19 +172,17 @@ struct CellW;
 struct TraceArgs {
     int nx, ny, nz;
     int level0, lmax_glob;
-    int chunk;
     float tau_max;
     const float* chi;        // opacity per cell times dx (per cell length), padded layout
     const float2* chi2;      // two-bin traces: {chi_i, chi_n} per cell length, padded
     const float* srcLn;      // two-bin traces: base-ray non-ionizing luminosity per source
     const float4* rec;       // adjoint: per cell {chi, chi_H, w, 0}
-    const float* w;          // adjoint weights per cell
     float* grad;             // adjoint gradient per cell (padded scratch)
     double* dL;              // adjoint output per source
     float4* acc;             // per-cell accumulator (sum L ds phi, sum dL n), padded
     const SrcDev* src;
     const LevelInfo* levels;
-    RayBuf buf[kNL];         // adjoint fronts
+    AdjBuf adj[kNL];         // adjoint fronts
     QuadBuf quad[kNL];       // forward fronts (levels beyond l0)
     unsigned base_quads;     // quads of level l0 per source (3 * 4^l0)
     unsigned nsrc;
@@ -207,8 +199,6 @@ struct TraceArgs {
     int fbits;               // fraction bits of the fixed-point distances
     float unit;              // 2^-fbits, their unit in cells
 };
-
-enum : int { EV_NONE = 0, EV_EXIT = 1, EV_DROP = 2, EV_SPLIT = 3 };
 
 // ---------------------------------------------------------------------------------------
 // ray walk
@@ -260,13 +250,6 @@ struct Path {
     int idx;      // index of the current cell in the padded layout (sentinel ring around
                   // the grid, see pad_index)
     int ss[3];    // signed index step of a crossing on each axis
-};
-
-template <class Cell>
-struct WalkT : Path {
-    float n[3];   // direction (hi parts) for momentum deposits
-    float L, tau;
-    Cell cell;    // record of the current cell (prefetched)
 };
 
 // Cell records are stored with a ring of sentinel cells around the nx*ny*nz grid (opacity
@@ -332,18 +315,6 @@ __device__ __forceinline__ bool path_start(Path& W, int nx, int ny, int nz, int 
     return inside;
 }
 
-// Outcome of one crossing step: the deposit to make (in cell, when seg) and the event.
-struct StepOut {
-    int cell;     // the cell the segment lies in (padded layout), negative without a segment
-    bool seg;     // the segment has positive length: deposit and count it
-    float ds;     // segment length (cell units), > 0 when seg
-    float Lin;
-    float G;      // L_in ds phi(dtau)
-    float dL;     // L_in (1 - e^-dtau)
-    float dphi;   // d phi / d dtau
-    int ev;
-};
-
 __device__ __forceinline__ float ex2_ftz(float v)
 {
     float r;
@@ -383,6 +354,12 @@ __device__ __forceinline__ float2 vrcp_max1(float2 v)
 }
 __device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ float2 vmax(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
+// a where x < 1, else b
+__device__ __forceinline__ float vbelow1(float x, float a, float b) { return x < 1.f ? a : b; }
+__device__ __forceinline__ float2 vbelow1(float2 x, float2 a, float2 b)
+{
+    return make_float2(x.x < 1.f ? a.x : b.x, x.y < 1.f ? a.y : b.y);
+}
 __device__ __forceinline__ float& vget(float& v, int) { return v; }
 __device__ __forceinline__ float& vget(float2& v, int j) { return j ? v.y : v.x; }
 __device__ __forceinline__ float vget(const float& v, int) { return v; }
@@ -406,28 +383,32 @@ __device__ __forceinline__ V phi_of(V x)
     return vmax(vmul(E, S), large);
 }
 
-// phi(x) and phi'(x) from the same exponential (the reverse sweep needs both). Below 1, with
-// y = x/2, E = e^{-y} and S = sinh(y)/y: phi = E S and phi' = E (S'(y) - S) / 2, S' to y^7
-// (S' - S stays near -1, so nothing cancels); above 1, phi' = (e^{-x} - phi)/x.
-__device__ __forceinline__ float phi_dphi(float x, float& dphi)
+// phi(x) and phi'(x) of a ray of the reverse sweep, which needs both. Below 1, with y = x/2,
+// E = e^{-y} and S = sinh(y)/y: phi = E S and phi' = E (S'(y) - S) / 2, S' to y^7 (S' - S stays
+// near -1, so nothing cancels); above 1, phi' = (e^{-x} - phi)/x. Chosen by x, not as the larger
+// of the two: near 1 they differ by rounding, and the larger would bias a sum of many.
+template <bool kDerivative, class V>
+__device__ __forceinline__ V phi_dphi(V x, V& dphi)
 {
-    const float y = 0.5f * x;
-    const float E = ex2_ftz(-kHalfLog2e * x);
-    const float y2 = y * y;
-    float S = fmaf(y2, 1.f / 362880.f, 1.f / 5040.f);
-    S = fmaf(S, y2, 1.f / 120.f);
-    S = fmaf(S, y2, 1.f / 6.f);
-    S = fmaf(S, y2, 1.f);
-    float Sp = fmaf(y2, 1.f / 45360.f, 1.f / 840.f);
-    Sp = fmaf(Sp, y2, 1.f / 30.f);
-    Sp = fmaf(Sp, y2, 1.f / 3.f);
-    Sp *= y;
-    const float r = rcp_ftz(fmaxf(x, 1.f));
-    const float E2 = E * E;
-    const float large = (1.f - E2) * r;
-    const bool sm = x < 1.f;
-    dphi = sm ? 0.5f * E * (Sp - S) : (E2 - large) * r;
-    return sm ? E * S : large;
+    const V E = vex2(vmul(x, vset<V>(-kHalfLog2e)));
+    const V y = vmul(x, vset<V>(0.5f));
+    const V y2 = vmul(y, y);
+    V S = vfma(y2, vset<V>(1.f / 362880.f), vset<V>(1.f / 5040.f));
+    S = vfma(S, y2, vset<V>(1.f / 120.f));
+    S = vfma(S, y2, vset<V>(1.f / 6.f));
+    S = vfma(S, y2, vset<V>(1.f));
+    const V r = vrcp_max1(x);
+    const V E2 = vmul(E, E);
+    const V large = vmul(vsub(vset<V>(1.f), E2), r);
+    const V phi = vbelow1(x, vmul(E, S), large);
+    if constexpr (kDerivative) {
+        V Sp = vfma(y2, vset<V>(1.f / 45360.f), vset<V>(1.f / 840.f));
+        Sp = vfma(Sp, y2, vset<V>(1.f / 30.f));
+        Sp = vfma(Sp, y2, vset<V>(1.f / 3.f));
+        Sp = vmul(Sp, y);
+        dphi = vbelow1(x, vmul(vmul(vset<V>(0.5f), E), vsub(Sp, S)), vmul(vsub(E2, large), r));
+    }
+    return phi;
 }
 
 // The geometric part of a step: the segment from tc to the next face or to the end radius
@@ -435,7 +416,7 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
 // the next cell is the end marker npad. ds is the length (cell units; unit = 2^-fbits) and key
 // the cell of the segment, 0 and `none` where there is nothing to deposit: the length is not
 // positive or the ray has ended (chi < 0, or depth > limit). Deposits are counted in ncross;
-// x is chi ds. walk_move_load also replaces chi by the opacity at the start of the next
+// x is chi ds, 0 with ds (also where chi is infinite). walk_move_load also replaces chi by the opacity at the start of the next
 // cell's record, unless the ray has ended.
 //
 // The earliest of the three faces and the end radius is decided on the high words (2^-19
@@ -454,13 +435,27 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
 // instructions (14.3 against 12.2 ms on 256^3 / 16 sources).
 //   operands: 0-2 t, 3 tc, 4 idx, 5 ncross, 6 ds, 7 key, 8 x, 9 chi, 10-12 d, 13-15 ss,
 //   16 rend, 17 unit, 18 none, 19 npad, 20 depth, 21 limit
-#define ART_MOVE_ADVANCE \
+#define ART_LENGTH "cvt.rn.f32.s64 fl, mv;\n\t"
+#define ART_LENGTH_PARTS \
+    "cvt.rn.f32.s64 fm, m;\n\t" \
+    "cvt.rn.f32.s64 fc, %3;\n\t" \
+    "cvt.rni.s64.f32 at, fm;\n\t" \
+    "sub.s64 at, m, at;\n\t" \
+    "cvt.rn.f32.s64 gm, at;\n\t" \
+    "cvt.rni.s64.f32 at, fc;\n\t" \
+    "sub.s64 at, %3, at;\n\t" \
+    "cvt.rn.f32.s64 gc, at;\n\t" \
+    "sub.rn.f32 fm, fm, fc;\n\t" \
+    "sub.rn.f32 gm, gm, gc;\n\t" \
+    "add.rn.f32 fl, fm, gm;\n\t"
+#define ART_MOVE_ADVANCE(LENGTH) \
     "sub.s64 mv, m, %3;\n\t" \
+    LENGTH \
     "mov.b64 %3, m;\n\t" \
-    "cvt.rn.f32.s64 %6, mv;\n\t" \
-    "mul.f32 %6, %6, %17;\n\t" \
-    "selp.f32 %6, %6, 0f00000000, pa;\n\t" \
-    "mul.f32 %8, %9, %6;\n\t" \
+    "mov.f32 %6, 0f00000000;\n\t" \
+    "mov.f32 %8, 0f00000000;\n\t" \
+    "@pa mul.f32 %6, fl, %17;\n\t" \
+    "@pa mul.f32 %8, %9, %6;\n\t" \
     "selp.b32 %7, %4, %18, pa;\n\t" \
     "@pa add.u32 %5, %5, 1;\n\t" \
     "@p0 add.s64 %0, %0, %10;\n\t" \
@@ -470,10 +465,11 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
     "@p1 add.s32 %4, %4, %14;\n\t" \
     "@p2 add.s32 %4, %4, %15;\n\t" \
     "@ps mov.b32 %4, %19;\n\t"
-#define ART_MOVE_PTX \
+#define ART_MOVE_PTX(LENGTH) \
     "{\n\t" \
     ".reg .pred p0, p1, p2, ps, ta, tb, tc, po, pa;\n\t" \
     ".reg .b32 l0, l1, l2, lr, h0, h1, h2, hr, hm, lm, cl, ch;\n\t" \
+    ".reg .f32 fl, fm, fc, gm, gc;\n\t" \
     ".reg .b64 m, tol, d, mv, at;\n\t" \
     "mov.b64 {l0, h0}, %0;\n\t" \
     "mov.b64 {l1, h1}, %1;\n\t" \
@@ -504,7 +500,7 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
     "selp.b32 lm, l0, lm, p0;\n\t" \
     "mov.b64 m, {lm, hm};\n\t" \
     "mov.pred pa, po;\n\t" \
-    ART_MOVE_ADVANCE \
+    ART_MOVE_ADVANCE(LENGTH) \
     "bra moved_%=;\n\t" \
     "tie_%=:\n\t" \
     "min.s64 m, %0, %1;\n\t" \
@@ -519,7 +515,7 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
     "setp.le.s64 ps, %16, m;\n\t" \
     "selp.b64 m, %16, m, ps;\n\t" \
     "setp.gt.and.s64 pa, m, %3, po;\n\t" \
-    ART_MOVE_ADVANCE \
+    ART_MOVE_ADVANCE(LENGTH) \
     "moved_%=:\n\t"
 #define ART_MOVE_OPERANDS                                                                      \
         : "+l"(W.t[0]), "+l"(W.t[1]), "+l"(W.t[2]), "+l"(W.tc), "+r"(W.idx), "+r"(ncross),     \
@@ -527,11 +523,16 @@ __device__ __forceinline__ float phi_dphi(float x, float& dphi)
         : "l"(W.d[0]), "l"(W.d[1]), "l"(W.d[2]), "r"(W.ss[0]), "r"(W.ss[1]), "r"(W.ss[2]),     \
           "l"(rend), "f"(unit), "r"(none), "r"(npad), "f"(depth), "f"(limit)
 
+// kParts: the length is the difference of the ends' leading 24 bits plus that of the rest. Both
+// forms round alike but for segments that more than double the distance from the source, the
+// first few of a ray.
+template <bool kParts>
 __device__ __forceinline__ void walk_move(Path& W, fix rend, float unit, float chi, float depth,
                                           float limit, int none, int npad, float& ds, float& x,
                                           int& key, unsigned& ncross)
 {
-    asm(ART_MOVE_PTX "}" ART_MOVE_OPERANDS);
+    if constexpr (kParts) asm(ART_MOVE_PTX(ART_LENGTH_PARTS) "}" ART_MOVE_OPERANDS);
+    else asm(ART_MOVE_PTX(ART_LENGTH) "}" ART_MOVE_OPERANDS);
 }
 
 template <class Cell>
@@ -540,42 +541,11 @@ __device__ __forceinline__ void walk_move_load(Path& W, fix rend, float unit, fl
                                                const Cell* cells, float& ds, float& x, int& key,
                                                unsigned& ncross)
 {
-    asm(ART_MOVE_PTX
+    asm(ART_MOVE_PTX(ART_LENGTH)
         "mad.wide.s32 at, %4, %22, %23;\n\t"
         "@po ld.global.nc.f32 %9, [at];\n\t"
         "}"
         ART_MOVE_OPERANDS, "n"((int)sizeof(Cell)), "l"(cells));
-}
-
-// One step of a walk of the reverse sweep (and of the work estimate, which passes L = 0): the
-// segment, its attenuation and the next cell's record. When the step ends the ray (event other
-// than EV_NONE) the walk state other than L and tau is left unspecified.
-template <class Cell>
-__device__ __forceinline__ StepOut walk_step(WalkT<Cell>& W, fix rend, float unit, int npad,
-                                             const Cell* __restrict__ cells, float tau_max,
-                                             unsigned& ncross)
-{
-    StepOut o;
-    // A step that starts in a sentinel cell ends the ray: it left the grid with the crossing
-    // of the previous step (whose segment was deposited then); nothing is deposited now.
-    const bool out = chi_of(W.cell) < 0.f;
-    float x;
-    walk_move(W, rend, unit, chi_of(W.cell), 0.f, 0.f, -1, npad, o.ds, x, o.cell, ncross);
-    const bool split = W.idx == npad;
-    o.seg = o.cell >= 0;
-    // prefetch of the next cell: from a cell inside the grid every crossing (also a diagonal
-    // one) lands inside the padded layout
-    const Cell ncell = out ? cell_zero<Cell>() : load_cell(cells + W.idx);
-    const float ph = phi_dphi(x, o.dphi);
-    o.Lin = W.L;
-    o.G = W.L * o.ds * ph;
-    o.dL = W.L * x * ph;
-    W.L -= o.dL;
-    W.tau += x;
-    const bool drop = o.seg && W.tau > tau_max;
-    o.ev = out ? EV_EXIT : (drop ? EV_DROP : (split ? EV_SPLIT : EV_NONE));
-    W.cell = ncell;
-    return o;
 }
 
 // Merges the deposits of lanes that hit the same cell (runs of equal cell index in lane
@@ -628,55 +598,82 @@ __device__ __forceinline__ void red_v4_if(float4* __restrict__ acc, int key, flo
 // ---------------------------------------------------------------------------------------
 // helpers shared by the forward and backward kernels
 // ---------------------------------------------------------------------------------------
-// Per-warp tallies live in shared memory (one Tally per warp, updated with shared atomics
-// when a ray ends), so they cost no registers in the walk loop.
-__device__ __forceinline__ Tally* tally_slots()
+// Threads per block of the trace kernels at most, and blocks per SM that the register budget
+// must leave room for (65536 / (128 * 5) = 102 registers a thread: two walks).
+constexpr int kTraceMaxThreads = 128;
+constexpr int kTraceMinBlocks = 5;
+// Steps between checks whether a warp still has rays.
+constexpr int kCheckSteps = 4;
+
+// Tallies of a block: photon sums per thread (no atomics while rays end), counters per warp
+// or per level. Reduced once, when the kernel ends.
+struct BlockTally {
+    double escaped[kTraceMaxThreads], dropped[kTraceMaxThreads];
+    double escaped_n[kTraceMaxThreads], dropped_n[kTraceMaxThreads];
+    unsigned long long crossings, destroy;
+    unsigned long long rays[kNL];
+};
+
+__device__ __forceinline__ BlockTally& block_tally()
 {
-    __shared__ Tally s_t[32];
-    return s_t;
+    __shared__ BlockTally t;
+    return t;
 }
 
-__device__ __forceinline__ void tally_init()
+__device__ __forceinline__ void block_tally_init()
 {
-    Tally* t = tally_slots();
-    if (threadIdx.x < 32) t[threadIdx.x] = Tally{0.0, 0.0, 0ull, 0ull, 0.0, 0.0};
+    BlockTally& T = block_tally();
+    const int i = threadIdx.x;
+    T.escaped[i] = T.dropped[i] = T.escaped_n[i] = T.dropped_n[i] = 0.0;
+    if (i < kNL) T.rays[i] = 0ull;
+    if (i == 0) T.crossings = T.destroy = 0ull;
     __syncthreads();
 }
 
-// Adds a lane count of crossings to its warp's tally.
-__device__ __forceinline__ void tally_crossings(Tally& T, unsigned n)
+__device__ __forceinline__ void block_tally_flush(DevStats* st)
 {
+    BlockTally& T = block_tally();
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) {
+        v[0] += T.escaped[i];
+        v[1] += T.dropped[i];
+        v[2] += T.escaped_n[i];
+        v[3] += T.dropped_n[i];
+    }
+    double* out[4] = {&st->escaped, &st->dropped, &st->escaped_n, &st->dropped_n};
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) n += __shfl_down_sync(kFull, n, off);
-    if ((threadIdx.x & 31u) == 0 && n > 0) atomicAdd(&T.crossings, (unsigned long long)n);
-}
-
-__device__ __forceinline__ void tally_flush(DevStats* st)
-{
-    __syncthreads();
+    for (int k = 0; k < 4; ++k) {
+        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(kFull, v[k], off);
+        if (threadIdx.x == 0 && v[k] != 0.0) atomicAdd(out[k], v[k]);
+    }
     if (threadIdx.x == 0) {
-        const Tally* t = tally_slots();
-        Tally s = {0.0, 0.0, 0ull, 0ull, 0.0, 0.0};
-        for (int w = 0; w < (int)((blockDim.x + 31) / 32); ++w) {
-            s.escaped += t[w].escaped;
-            s.dropped += t[w].dropped;
-            s.escaped_n += t[w].escaped_n;
-            s.dropped_n += t[w].dropped_n;
-            s.crossings += t[w].crossings;
-            s.destroy += t[w].destroy;
-        }
-        atomicAdd(&st->escaped, s.escaped);
-        atomicAdd(&st->dropped, s.dropped);
-        if (s.escaped_n != 0.0) atomicAdd(&st->escaped_n, s.escaped_n);
-        if (s.dropped_n != 0.0) atomicAdd(&st->dropped_n, s.dropped_n);
-        atomicAdd(&st->crossings, s.crossings);
-        atomicAdd(&st->destroy, s.destroy);
+        if (T.crossings) atomicAdd(&st->crossings, T.crossings);
+        if (T.destroy) atomicAdd(&st->destroy, T.destroy);
+    }
+    if (threadIdx.x < kNL && T.rays[threadIdx.x]) {
+        atomicAdd(&st->rays_per_level[threadIdx.x], T.rays[threadIdx.x]);
+        atomicAdd(&st->rays_total, T.rays[threadIdx.x]);
+        atomicMax(&st->level_reached, (int)threadIdx.x);
     }
 }
 
-// Slot value of a ray buffer entry that holds no ray: the children slots of a parent that
-// did not split (each parent owns four consecutive child slots, so fronts keep pixel order).
-constexpr unsigned kHole = 0xffffffffu;
+// Sum of a few floats in two floats, for the tallies.
+__device__ __forceinline__ void df_accumulate(df& s, float v)
+{
+    const df r = df_two_sum(s.hi, v);
+    s.hi = r.hi;
+    s.lo += r.lo;
+}
+
+// Rays per lane for a front of `quads` quads: one while that fits the chip's warps in one
+// round (latency counts there, and a step of one ray is shorter), else two; two at the base
+// level.
+__device__ __forceinline__ int front_width(bool base, unsigned long long quads)
+{
+    return !base && 4 * quads <= (unsigned long long)gridDim.x * blockDim.x ? 1 : 2;
+}
 
 // Where a ray of a level with split radius rmax ends: at rmax if it can split and (kCut) at
 // the d_max cutoff, whichever comes first; at equal radii the cut wins.
@@ -704,60 +701,6 @@ __device__ __forceinline__ void load_direction(const float4* e, df n[3], fix cod
     code[0] = (fix)(((unsigned long long)__float_as_uint(e1.w) << 32) | __float_as_uint(e1.z));
     code[1] = e2.x;
     code[2] = e2.y;
-}
-
-// Starts the walk of ray i of level l: loads its record, its source and its direction
-// entry. Returns 1 if the ray starts inside the grid, 0 if it starts outside (it escapes at
-// once), -1 if slot i holds no ray. L0 receives its entering L.
-template <bool kCut, class Cell>
-__device__ __forceinline__ int ray_begin(const TraceArgs& A, const LevelInfo& LV, const RayBuf& B,
-                                         int l, unsigned long long i, WalkT<Cell>& W,
-                                         const Cell* cells, unsigned& s, unsigned& p, float& L0,
-                                         bool& splits, fix& rend)
-{
-    s = __ldcg(B.src + i);
-    if (s == kHole) return -1;
-    p = __ldcg(B.pix + i);
-    const float4 sh = __ldg(&A.src[s].hi);
-    const float4 sl = __ldg(&A.src[s].lo);
-    const longlong2 xy = __ldg(&A.src[s].xy);
-    const longlong2 z_ = __ldg(&A.src[s].z_);
-    L0 = (l == A.level0) ? sh.w : __ldcg(B.L + i);
-    const float tau0 = (l == A.level0) ? 0.f : __ldcg(B.tau + i);
-    splits = l < __float_as_int(sl.w);
-    const float4* e = LV.dir + 3ull * p;
-    const df u[3] = {{sh.x, sl.x}, {sh.y, sl.y}, {sh.z, sl.z}};
-    const fix ux[3] = {xy.x, xy.y, z_.x};
-    df n[3];
-    fix code[3];
-    load_direction(e, n, code);
-    const bool inside = path_start(W, A.nx, A.ny, A.nz, A.fbits, u, ux, n, code, LV.r0, LV.r0x);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) W.n[a] = n[a].hi;
-    rend = end_radius<kCut>(splits, LV.rmaxx, A.dmax);
-    W.L = L0;
-    W.tau = tau0;
-    W.cell = inside ? load_cell(cells + W.idx) : cell_zero<Cell>();
-    return inside ? 1 : 0;
-}
-
-// Marks the four child slots of parent slot c4/4 as empty.
-__device__ __forceinline__ void write_holes(const RayBuf& C, unsigned long long c4)
-{
-    if (c4 + 4 <= C.cap)
-        *reinterpret_cast<uint4*>(C.src + c4) = make_uint4(kHole, kHole, kHole, kHole);
-}
-
-// Adds a warp's count of rays started at level l to the per-level counters.
-__device__ __forceinline__ void count_rays(DevStats* st, int l, unsigned n)
-{
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) n += __shfl_down_sync(kFull, n, off);
-    if ((threadIdx.x & 31u) == 0 && n > 0) {
-        atomicAdd(&st->rays_per_level[l], (unsigned long long)n);
-        atomicAdd(&st->rays_total, (unsigned long long)n);
-        atomicMax(&st->level_reached, l);
-    }
 }
 
 // Grid-wide barrier for a cooperative launch. Every wait is bounded by wait_ns of
@@ -805,9 +748,4 @@ __device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long 
     __syncthreads();
     return s_ok != 0;
 }
-__device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long wait_ns)
-{
-    return grid_barrier(sc, st, wait_ns, [] {});
-}
-
 }  // namespace art

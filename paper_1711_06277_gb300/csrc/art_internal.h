@@ -73,8 +73,8 @@ struct art_grid {
     unsigned long long quad_cap[art::kNL] = {};      // allocated quads per level
 
     // adjoint fronts
-    art::RayBuf buf[art::kNL] = {};
-    unsigned long long buf_cap[art::kNL] = {};      // allocated rays per level
+    art::AdjBuf adj[art::kNL] = {};
+    unsigned long long adj_cap[art::kNL] = {};       // allocated quads per level
 
     // adjoint: source luminosities and a dL buffer for callers that pass none
     float* d_srcL = nullptr;

@@ -164,81 +164,12 @@ template <class Cell> __device__ __forceinline__ const Cell* cells_of(const Trac
 template <> __device__ __forceinline__ const float* cells_of<float>(const TraceArgs& A) { return A.chi; }
 template <> __device__ __forceinline__ const float2* cells_of<float2>(const TraceArgs& A) { return A.chi2; }
 
-// Threads per block of the forward kernels at most, and blocks per SM that the register
-// budget must leave room for (65536 / (128 * 5) = 102 registers a thread: two walks).
-constexpr int kTraceMaxThreads = 128;
-constexpr int kTraceMinBlocks = 5;
-// Steps between checks whether a warp still has rays.
-constexpr int kCheckSteps = 4;
-
 __device__ __forceinline__ void load_pair(const float* p, float& a, float& b) { a = __ldg(p); b = 0.f; }
 __device__ __forceinline__ void load_pair(const float2* p, float& a, float& b)
 {
     const float2 v = __ldg(p);
     a = v.x;
     b = v.y;
-}
-
-// Tallies of a block: photon sums per thread (no atomics while rays end), counters per warp
-// or per level. Reduced once, when the kernel ends.
-struct BlockTally {
-    double escaped[kTraceMaxThreads], dropped[kTraceMaxThreads];
-    double escaped_n[kTraceMaxThreads], dropped_n[kTraceMaxThreads];
-    unsigned long long crossings, destroy;
-    unsigned long long rays[kNL];
-};
-
-__device__ __forceinline__ BlockTally& block_tally()
-{
-    __shared__ BlockTally t;
-    return t;
-}
-
-__device__ __forceinline__ void block_tally_init()
-{
-    BlockTally& T = block_tally();
-    const int i = threadIdx.x;
-    T.escaped[i] = T.dropped[i] = T.escaped_n[i] = T.dropped_n[i] = 0.0;
-    if (i < kNL) T.rays[i] = 0ull;
-    if (i == 0) T.crossings = T.destroy = 0ull;
-    __syncthreads();
-}
-
-__device__ __forceinline__ void block_tally_flush(DevStats* st)
-{
-    BlockTally& T = block_tally();
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) {
-        v[0] += T.escaped[i];
-        v[1] += T.dropped[i];
-        v[2] += T.escaped_n[i];
-        v[3] += T.dropped_n[i];
-    }
-    double* out[4] = {&st->escaped, &st->dropped, &st->escaped_n, &st->dropped_n};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(kFull, v[k], off);
-        if (threadIdx.x == 0 && v[k] != 0.0) atomicAdd(out[k], v[k]);
-    }
-    if (threadIdx.x == 0) {
-        if (T.crossings) atomicAdd(&st->crossings, T.crossings);
-        if (T.destroy) atomicAdd(&st->destroy, T.destroy);
-    }
-    if (threadIdx.x < kNL && T.rays[threadIdx.x]) {
-        atomicAdd(&st->rays_per_level[threadIdx.x], T.rays[threadIdx.x]);
-        atomicAdd(&st->rays_total, T.rays[threadIdx.x]);
-        atomicMax(&st->level_reached, (int)threadIdx.x);
-    }
-}
-
-// Sum of a few floats in two floats, for the tallies.
-__device__ __forceinline__ void df_accumulate(df& s, float v)
-{
-    const df r = df_two_sum(s.hi, v);
-    s.hi = r.hi;
-    s.lo += r.lo;
 }
 
 // Photons of the rays of a lane, side by side (V: float or float2).
@@ -376,8 +307,7 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
 #pragma unroll
             for (int j = 0; j < kWidth; ++j) {
                 const float depth = vget(two ? P.taun : P.tau, j);
-                bool alive = false;
-                if constexpr (two) alive = !(cell[j] < 0.f) & !(depth > A.tau_max);
+                [[maybe_unused]] const bool alive = !(cell[j] < 0.f) & !(depth > A.tau_max);
                 walk_move_load(W[j], rend, A.unit, cell[j], depth, A.tau_max, -1 - j,
                                (int)A.npad, cells, vget(ds, j), vget(x, j), key[j], ncross);
                 if constexpr (two) {
@@ -499,14 +429,6 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ncross += __shfl_down_sync(kFull, ncross, off);
     if (lane == 0 && ncross) atomicAdd(&T.crossings, (unsigned long long)ncross);
-}
-
-// Rays per lane for a front of `quads` quads: one while that fits the chip's warps in one
-// round (latency counts there, and a step of one ray is shorter), else two; two at the base
-// level.
-__device__ __forceinline__ int front_width(bool base, unsigned long long quads)
-{
-    return !base && 4 * quads <= (unsigned long long)gridDim.x * blockDim.x ? 1 : 2;
 }
 
 // Base rays are taken 32 apart where the front's quads [begin, end) are whole groups of 64 rays

@@ -45,26 +45,24 @@ __global__ void k_reach(int nx, int ny, int nz, const float* __restrict__ chi,
     df n[3];
     fix code[3];
     load_direction(dir + 3ull * p, n, code);
-    WalkT<float> W;
+    Path W;
     if (!path_start(W, nx, ny, nz, fbits, u, ux, n, code, df{0.f, 0.f}, 0)) {
         reach[i] = 0.f;
         return;
     }
-    W.L = 0.f;
-    W.tau = 0.f;
-    W.cell = __ldg(chi + W.idx);
-    float r = 0.f;
+    float tau = 0.f, cell = __ldg(chi + W.idx);
     unsigned count = 0;
-    const float unit = exp2f((float)-fbits);
+    const float unit = ldexpf(1.f, -fbits);
     const int bound = nx + ny + nz + 2;
     for (int k = 0; k < bound; ++k) {
-        const fix before = W.tc;
-        const StepOut o = walk_step(W, dmax, unit, npad, chi, tau_max, count);
-        if (o.ev == EV_NONE) continue;
-        // an exit is seen one step late, in the sentinel cell: the ray left at `before`
-        r = (float)(o.ev == EV_EXIT ? before : W.tc) * unit;
-        break;
+        float ds, x;
+        int key;
+        walk_move_load(W, dmax, unit, cell, tau, tau_max, -1, npad, chi, ds, x, key, count);
+        tau += x;
+        // left the grid or reached the cutoff, or used up
+        if (cell < 0.f || tau > tau_max) break;
     }
+    const float r = (float)W.tc * unit;
     reach[i] = r;
 }
 
