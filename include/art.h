@@ -71,9 +71,9 @@ typedef struct {
     unsigned flags;      /* ART_F_* */
     int schedule;        /* ART_SCHED_* */
     int block_threads;   /* threads per block of the trace kernels (0 = library choice; at most
-                            128 in the forward trace, 256 in the reverse sweep) */
-    int chunk;           /* rays a warp of the reverse sweep takes from the queue at a time
-                            (0 = library choice; the forward trace takes 32 lanes' worth) */
+                            640, one block per SM) */
+    int chunk;           /* accepted and checked as before (0 or a multiple of 32); the kernels
+                            take 32 lanes' worth of rays at a time */
     long long queue_capacity; /* rays per level buffer beyond l0 (0 = library choice; the
                             persistent trace holds at least 16) */
     double wait_limit_s; /* bound on any device-side wait (grid barrier); 0 = library default

@@ -278,7 +278,7 @@ __device__ __forceinline__ void walkers_run(const TraceArgs& A, const Cell* __re
 // (pass 2 of the quads not done yet). Warp-uniform.
 template <class Cell, bool kCut, int kWidth>
 __device__ void sweep_front(const TraceArgs& A, int l, bool collapse, unsigned long long* cursor,
-                            unsigned long long end)
+                            unsigned long long begin, unsigned long long end)
 {
     using V = typename Walkers<Cell, kWidth>::V;
     constexpr unsigned kPerQuad = 4u / kWidth;
@@ -290,12 +290,12 @@ __device__ void sweep_front(const TraceArgs& A, int l, bool collapse, unsigned l
     const bool base = l == A.level0;
     BlockTally& T = block_tally();
     const unsigned items = (unsigned)end * kPerQuad;  // front ends below 2^29 quads
+    const unsigned first = (unsigned)begin * kPerQuad;
+    Batches batches(cursor, first, items);
     unsigned ncross = 0;
 
     for (;;) {
-        unsigned b = 0;
-        if (lane == 0) b = (unsigned)min(atomicAdd(cursor, 32ull), (unsigned long long)items);
-        b = __shfl_sync(kFull, b, 0);
+        const unsigned b = batches.take(first);
         if (b >= items) break;
         const unsigned item = b + lane;
         bool valid = item < items;
@@ -423,29 +423,44 @@ __device__ void sweep_front(const TraceArgs& A, int l, bool collapse, unsigned l
 // quads, which are then collapsed (everything below them is finished), or with quads to expand.
 __device__ __forceinline__ void next_sweep(const TraceArgs& A)
 {
-    volatile Sched* sc = A.sched;
-    if (!sc->started) {
-        sc->started = 1;
-        sc->count[A.level0] = (unsigned long long)A.base_quads * A.nsrc;
-    } else if (sc->phase_kind == 0 && (sc->phase_level == A.lmax_glob ||
-                                       sc->count[sc->phase_level + 1] == 0)) {
-        sc->open_end[sc->phase_level] = 0;  // no children: every warp ran both passes
+    Sched* sc = A.sched;
+    const int started = __ldcg(&sc->started), kind = __ldcg(&sc->phase_kind);
+    const int was = __ldcg(&sc->phase_level);
+    int l = -1;
+    unsigned long long have = 0, opened = 0, below = 0;
+    // the levels are read side by side, from the deepest
+#pragma unroll
+    for (int k = kLevels - 1; k >= 0; --k) {
+        const unsigned long long c = __ldcg(&sc->count[k]);
+        unsigned long long open = __ldcg(&sc->open_end[k]);
+        // an expanded part without children: every warp ran both passes
+        if (started && kind == 0 && k == was && below == 0) open = 0;
+        below = c;
+        if (l < 0 && (c > 0 || open > 0)) {
+            l = k;
+            have = c;
+            opened = open;
+        }
     }
-    int l = A.lmax_glob;
-    while (l >= A.level0 && sc->open_end[l] == 0 && sc->count[l] == 0) --l;
-    if (l < A.level0) {
+    if (started && kind == 0 && l <= was) sc->open_end[was] = 0;
+    if (!started) {
+        l = A.level0;
+        have = (unsigned long long)A.base_quads * A.nsrc;
+    }
+    sc->started = 1;
+    if (l < 0) {
         sc->done = 1;
         return;
     }
     unsigned long long begin, end;
-    if (sc->open_end[l] != 0) {
+    if (opened != 0) {
         sc->phase_kind = 1;
-        begin = sc->open_begin[l];
-        end = sc->open_end[l];
+        begin = __ldcg(&sc->open_begin[l]);
+        end = opened;
         sc->open_end[l] = 0;
     } else {
         sc->phase_kind = 0;
-        end = sc->count[l];
+        end = have;
         unsigned long long take = end;
         if (l < A.lmax_glob) take = min(end, A.adj[l + 1].cap / 4);
         if (take == 0) {  // a phase must consume rays, or the schedule never ends
@@ -457,11 +472,12 @@ __device__ __forceinline__ void next_sweep(const TraceArgs& A)
         sc->open_begin[l] = begin;
         sc->open_end[l] = end;
     }
-    const int width = front_width(false, end - begin);
+    const int width = front_width(end - begin);
     sc->phase_level = l;
     sc->phase_width = width;
+    sc->phase_begin = begin;
     sc->phase_end = end;
-    sc->cursor[l] = begin * (unsigned long long)(4 / width);
+    sc->cursor[l] = begin * (unsigned long long)(4 / width) + 32ull * warps_in_grid();
 }
 
 template <class Cell, bool kCut>
@@ -470,104 +486,105 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_backward_
     block_tally_init();
     Sched* sc = A.sched;
     __shared__ int s_level, s_width, s_kind;
-    __shared__ unsigned long long s_end;
+    __shared__ unsigned long long s_begin, s_end;
     for (;;) {
         if (!grid_barrier(sc, A.stats, A.wait_ns, [&] { next_sweep(A); })) break;
         if (threadIdx.x == 0) {
-            volatile Sched* v = sc;
-            s_level = v->done ? -1 : v->phase_level;
-            s_width = v->phase_width;
-            s_kind = v->phase_kind;
-            s_end = v->phase_end;
+            s_level = __ldcg(&sc->done) ? -1 : __ldcg(&sc->phase_level);
+            s_width = __ldcg(&sc->phase_width);
+            s_kind = __ldcg(&sc->phase_kind);
+            s_begin = __ldcg(&sc->phase_begin);
+            s_end = __ldcg(&sc->phase_end);
         }
         __syncthreads();
         const int l = s_level;
         if (l < 0) break;
-        if (s_width == 2) sweep_front<Cell, kCut, 2>(A, l, s_kind == 1, &sc->cursor[l], s_end);
-        else sweep_front<Cell, kCut, 1>(A, l, s_kind == 1, &sc->cursor[l], s_end);
+        if (s_width == 2) sweep_front<Cell, kCut, 2>(A, l, s_kind == 1, &sc->cursor[l], s_begin, s_end);
+        else sweep_front<Cell, kCut, 1>(A, l, s_kind == 1, &sc->cursor[l], s_begin, s_end);
     }
     block_tally_flush(A.stats);
 }
 
-// Per-cell record of the reverse sweep in the padded layout: one 16-byte gather per
-// crossing, {chi, chi_H, w, 0} with chi and its neutral-H part formed exactly as k_opacity
-// forms the forward trace's opacity; the sentinel ring holds {-1, 0, 0, 0}.
-__global__ void k_pack_cells(int nx, int ny, int nz, const float* __restrict__ nH0,
-                             const float* __restrict__ nH, double sH_dx, double sd_dx,
-                             const float* __restrict__ w, float4* __restrict__ rec)
+// Per-cell records of the reverse sweep in the padded layout, one gather per crossing, with
+// the opacity and its neutral-H part formed exactly as k_opacity forms the forward trace's
+// opacity; the sentinel ring and the end marker hold zero weights. The same pass clears the
+// gradient and flags bad densities.
+struct CellIn {
+    float a, b, w, v0, v1, v2;
+};
+__device__ __forceinline__ void make_record(float4& r, float chi, float h, const CellIn& c)
 {
-    const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
-    const unsigned step = gridDim.x * blockDim.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        rec[npad] = make_float4(kEnded, 0.f, 0.f, 0.f);
-    }
-    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
-        unsigned i;
-        if (!unpad(q, nx, ny, nz, i)) {
-            rec[q] = make_float4(kSentinel, 0.f, 0.f, 0.f);
-            continue;
-        }
-        const double h = (double)nH0[i] * sH_dx;
-        const double dust = nH ? (double)nH[i] * sd_dx : 0.0;
-        rec[q] = make_float4(__double2float_rn(h + dust), __double2float_rn(h), w ? w[i] : 0.f, 0.f);
-    }
+    r = make_float4(chi, h, c.w, 0.f);
+}
+// with the force weight v
+__device__ __forceinline__ void make_record(CellF& r, float chi, float h, const CellIn& c)
+{
+    r.a = make_float4(chi, h, c.w, 0.f);
+    r.b = make_float4(c.v0, c.v1, c.v2, 0.f);
+}
+// without dust and force term: the neutral-H part is the opacity
+__device__ __forceinline__ void make_record(CellW& r, float, float h, const CellIn& c)
+{
+    r = CellW{h, c.w};
 }
 
-// The same with the force weight v (3 blocks of nx*ny*nz floats: x, y, z).
-__global__ void k_pack_cells_f(int nx, int ny, int nz, const float* __restrict__ nH0,
-                               const float* __restrict__ nH, double sH_dx, double sd_dx,
-                               const float* __restrict__ w, const float* __restrict__ v,
-                               CellF* __restrict__ rec)
+template <class Cell>
+__global__ void __launch_bounds__(256) k_pack_cells(int nx, int ny, int nz,
+                                                    const float* __restrict__ nH0,
+                                                    const float* __restrict__ nH, Coef sH, Coef sd,
+                                                    const float* __restrict__ w,
+                                                    const float* __restrict__ v,
+                                                    Cell* __restrict__ rec,
+                                                    float* __restrict__ grad,
+                                                    DevStats* __restrict__ st)
 {
-    const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
     const size_t ncell = (size_t)nx * ny * nz;
-    const unsigned step = gridDim.x * blockDim.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        rec[npad].a = make_float4(kEnded, 0.f, 0.f, 0.f);
-        rec[npad].b = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
-        unsigned i;
-        if (!unpad(q, nx, ny, nz, i)) {
-            rec[q].a = make_float4(kSentinel, 0.f, 0.f, 0.f);
-            rec[q].b = make_float4(0.f, 0.f, 0.f, 0.f);
-            continue;
-        }
-        const double h = (double)nH0[i] * sH_dx;
-        const double dust = nH ? (double)nH[i] * sd_dx : 0.0;
-        rec[q].a = make_float4(__double2float_rn(h + dust), __double2float_rn(h), w ? w[i] : 0.f, 0.f);
-        rec[q].b = make_float4(v[i], v[ncell + i], v[2 * ncell + i], 0.f);
-    }
-}
-
-// The 8-byte record {chi, w} of a sweep without dust and force term (sentinel {-1, 0}).
-__global__ void k_pack_cells_w(int nx, int ny, int nz, const float* __restrict__ nH0,
-                               double sH_dx, const float* __restrict__ w,
-                               CellW* __restrict__ rec)
-{
-    const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
-    const unsigned step = gridDim.x * blockDim.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        rec[npad] = CellW{kEnded, 0.f};
-    }
-    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
-        unsigned i;
-        if (!unpad(q, nx, ny, nz, i)) {
-            rec[q] = CellW{kSentinel, 0.f};
-            continue;
-        }
-        rec[q] = CellW{__double2float_rn((double)nH0[i] * sH_dx), w ? w[i] : 0.f};
-    }
+    bool bad = false;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        make_record(rec[(size_t)(nx + 2) * (ny + 2) * (nz + 2)], kEnded, kEnded, CellIn{});
+    each_padded_cell(
+        nx, ny, nz,
+        [&](unsigned i) {
+            CellIn c = {nH0[i], nH ? nH[i] : 0.f, w ? w[i] : 0.f, 0.f, 0.f, 0.f};
+            if constexpr (HasForce<Cell>::value) {
+                c.v0 = v[i];
+                c.v1 = v[ncell + i];
+                c.v2 = v[2 * ncell + i];
+            }
+            return c;
+        },
+        [&](unsigned q, bool inside, const CellIn& c) {
+            float chi = kSentinel, h = kSentinel, dust;
+            if (inside) {
+                bad = bad || bad_density(c.a) || bad_density(c.b);
+                opacities(sH, sd, c.a, c.b, chi, h, dust);
+            }
+            make_record(rec[q], chi, h, c);
+            grad[q] = 0.f;
+        });
+    if (bad) atomicCAS(&st->error, 0, -1);
 }
 
 // Gradient per cell from the padded scratch it was summed in, into the caller's layout.
-__global__ void k_unpad_grad(int nx, int ny, int nz, const float* __restrict__ src,
-                             float* __restrict__ dst)
+__global__ void __launch_bounds__(256) k_unpad_grad(int nx, int ny, int nz,
+                                                    const float* __restrict__ src,
+                                                    float* __restrict__ dst)
 {
     const unsigned ncell = (unsigned)nx * (unsigned)ny * (unsigned)nz;
-    const unsigned step = gridDim.x * blockDim.x;
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < ncell; i += step)
-        dst[i] = src[pad_of(i, nx, ny)];
+    const unsigned long long step = 4ull * gridDim.x * blockDim.x;
+    for (unsigned long long base = 4ull * blockIdx.x * blockDim.x + threadIdx.x; base < ncell; base += step) {
+        float a[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long i = base + (unsigned)k * blockDim.x;
+            if (i < ncell) a[k] = __ldcs(src + pad_of((unsigned)i, nx, ny));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long i = base + (unsigned)k * blockDim.x;
+            if (i < ncell) dst[i] = a[k];
+        }
+    }
 }
 
 int status_of(cudaError_t e)
@@ -593,7 +610,7 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     if (ns == 0) return ART_ESTATE;
     if (g->two_bin) return ART_EINVAL;  // the reverse sweep covers one-bin traces
     cudaStream_t st = g->stream;
-    if ((rc = status_of(cudaMemsetAsync(g->d_stats, 0, sizeof(DevStats), st)))) return rc;
+    if ((rc = status_of(cudaMemsetAsync(g->d_state, 0, sizeof(DevState), st)))) return rc;
     rc = prepare_trace(g, p, true);
     if (rc) return rc;
     if ((size_t)ns > g->srcL_cap) {
@@ -615,28 +632,28 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     if ((rc = status_of(cudaMemsetAsync(dL, 0, sizeof(double) * ns, st)))) return rc;
     // the gradient is summed in the padded layout, in the (otherwise idle) accumulator
     float* grad_pad = reinterpret_cast<float*>(g->d_acc);
-    if ((rc = status_of(cudaMemsetAsync(grad_pad, 0, sizeof(float) * g->npad, st)))) return rc;
-    if ((rc = status_of(cudaMemsetAsync(g->d_sched, 0, sizeof(Sched), st)))) return rc;
-    const int pack_blocks = (int)std::min<long long>((g->npad + 255) / 256, (long long)g->sms * 16);
+    const int pack_blocks = cell_blocks(g->npad);
     const int nx = g->n[0], ny = g->n[1], nz = g->n[2];
-    const double sH_dx = p->sigma_H * g->dx;
-    const double sd_dx = g->nH ? p->sigma_d * g->dx : 0.0;
+    const Coef sH = coef_of(p->sigma_H * g->dx);
+    const Coef sd = coef_of(g->nH ? p->sigma_d * g->dx : 0.0);
     // without dust the neutral-H opacity is the opacity: an 8-byte record serves
-    const bool light = !d_v && sd_dx == 0.0;
+    const bool light = !d_v && sd.full == 0.0;
     if (light) {
         if (!g->d_recw && (rc = status_of(cudaMalloc((void**)&g->d_recw, sizeof(CellW) * (g->npad + 1)))))
             return rc;
-        k_pack_cells_w<<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, sH_dx, d_w, g->d_recw);
+        k_pack_cells<CellW><<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH, sd, d_w,
+                                                         nullptr, g->d_recw, grad_pad, g->d_stats);
     } else if (d_v) {
         if (!g->d_recf && (rc = status_of(cudaMalloc((void**)&g->d_recf, sizeof(CellF) * (g->npad + 1)))))
             return rc;
-        k_pack_cells_f<<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH_dx, sd_dx, d_w,
-                                                    d_v, g->d_recf);
+        k_pack_cells<CellF><<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH, sd, d_w,
+                                                         d_v, g->d_recf, grad_pad, g->d_stats);
     } else {
         if (!g->d_rec && (rc = status_of(cudaMalloc((void**)&g->d_rec, sizeof(float4) * (g->npad + 1)))))
             return rc;
-        k_pack_cells<<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH_dx, sd_dx, d_w,
-                                                  g->d_rec);
+        k_pack_cells<float4><<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH, sd, d_w,
+                                                          nullptr, g->d_rec, grad_pad,
+                                                          g->d_stats);
     }
     if ((rc = status_of(cudaGetLastError()))) return rc;
     TraceArgs A = make_args(g, p);
@@ -649,8 +666,7 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     const double dV = g->dx * g->dx * g->dx;
     A.gscale = (float)(p->sigma_H * g->dx / dV);
     A.fscale = (float)(1.0 / dV);
-    // block size: the caller's (or 128), at most what the kernels are built for
-    const int threads = std::min(p->block_threads > 0 ? p->block_threads : 128, kTraceMaxThreads);
+    const int threads = trace_threads(p);
     const bool cut = p->d_max > 0.0;
     void (*kern)(TraceArgs) =
         light ? (cut ? k_backward_persistent<CellW, true> : k_backward_persistent<CellW, false>)
@@ -671,8 +687,7 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if ((rc = status_of(cudaLaunchKernelEx(&cfg, kern, A)))) return rc;
-    const int unpad_blocks = (int)std::min<long long>((g->ncell + 255) / 256, (long long)g->sms * 16);
-    k_unpad_grad<<<unpad_blocks, 256, 0, st>>>(nx, ny, nz, grad_pad, d_dlog_nH0);
+    k_unpad_grad<<<cell_blocks(g->ncell), 256, 0, st>>>(nx, ny, nz, grad_pad, d_dlog_nH0);
     if ((rc = status_of(cudaGetLastError()))) return rc;
     if ((rc = status_of(cudaMemcpyAsync(g->h_stats, g->d_stats, sizeof(DevStats),
                                         cudaMemcpyDeviceToHost, st))))

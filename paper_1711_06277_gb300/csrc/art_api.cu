@@ -111,6 +111,17 @@ fix to_fix(double cells, int fbits)
     return v < (double)kFar ? (fix)std::llrint(v) : kFar - 1;
 }
 
+// An opacity coefficient for the device: two floats where products with densities below 1e18
+// stay in their range, parts included.
+Coef coef_of(double v)
+{
+    Coef c;
+    split_df(v, c.hi, c.lo);
+    c.full = v;
+    c.wide = v != 0.0 && !(v > 1e-18 && v < 1e18);
+    return c;
+}
+
 // Device record of a source at u (cell units).
 SrcDev source_record(const art_grid* g, const double u[3], double base_L, int lmax)
 {
@@ -318,19 +329,28 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
     g->prep_schedule = p->schedule;
     g->prep_qcap = p->queue_capacity;
     g->prep_two_bin = g->two_bin;
-    // --- opacity per cell length
-    return run_opacity(g, p, g->two_bin && !adjoint);
+    return ART_OK;
 }
 
-// Opacity per cell length (padded layout) into d_chi, and the two-bin pairs into d_chi2.
-int run_opacity(art_grid* g, const art_params* p, bool two_bin)
+// Block size of the trace kernels: the caller's, at most (and by default) what they are built
+// for.
+int trace_threads(const art_params* p)
 {
-    const double sH_dx = p->sigma_H * g->dx;
-    const double sd_dx = g->nH ? p->sigma_d * g->dx : 0.0;
-    int blocks = (int)std::min<long long>((g->npad + 255) / 256, (long long)g->sms * 16);
-    k_opacity<<<blocks, 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2], g->nH0, g->nH, sH_dx,
-                                             sd_dx, g->d_chi, two_bin ? g->d_chi2 : nullptr,
-                                             g->d_stats);
+    return p->block_threads > 0 ? std::min(p->block_threads, kTraceMaxThreads) : kTraceMaxThreads;
+}
+
+// Blocks of 256 threads for a pass over n cells, four cells per thread.
+int cell_blocks(long long n) { return (int)((n + 1023) / 1024); }
+
+// Opacity per cell length (padded layout) into d_chi, and the two-bin pairs into d_chi2; clears
+// acc if given.
+int run_opacity(art_grid* g, const art_params* p, bool two_bin, float4* acc)
+{
+    const Coef sH = coef_of(p->sigma_H * g->dx);
+    const Coef sd = coef_of(g->nH ? p->sigma_d * g->dx : 0.0);
+    k_opacity<<<cell_blocks(g->npad), 256, 0, g->stream>>>(
+        g->n[0], g->n[1], g->n[2], g->nH0, g->nH, sH, sd, g->d_chi,
+        two_bin ? g->d_chi2 : nullptr, acc, g->d_stats);
     ART_TRY(cudaGetLastError());
     return ART_OK;
 }
@@ -453,8 +473,11 @@ int art_create_grid(art_grid** out, int nx, int ny, int nz, const double box_lo[
     if (!rc) rc = dev_alloc(&g->d_chi, npad + 1);
     if (!rc) rc = dev_alloc(&g->d_acc, npad);
     if (!rc) rc = dev_alloc(&g->d_levels, kNL);
-    if (!rc) rc = dev_alloc(&g->d_sched, 1);
-    if (!rc) rc = dev_alloc(&g->d_stats, 1);
+    if (!rc) rc = dev_alloc(&g->d_state, 1);
+    if (!rc) {
+        g->d_sched = &g->d_state->sched;
+        g->d_stats = &g->d_state->stats;
+    }
     if (!rc) rc = cuda_status(cudaMallocHost((void**)&g->h_stats, sizeof(DevStats)));
     if (!rc) rc = cuda_status(cudaMallocHost((void**)&g->h_levels, sizeof(LevelInfo) * kNL));
     if (rc) {
@@ -529,15 +552,14 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     int rc = check_params(p);
     if (rc) return rc;
     if (g->L.empty()) return ART_ESTATE;
-    ART_TRY(cudaMemsetAsync(g->d_stats, 0, sizeof(DevStats), g->stream));
+    ART_TRY(cudaMemsetAsync(g->d_state, 0, sizeof(DevState), g->stream));
     rc = prepare_trace(g, p, false);
     if (rc) return rc;
-    ART_TRY(cudaMemsetAsync(g->d_acc, 0, sizeof(float4) * (size_t)g->npad, g->stream));
-    ART_TRY(cudaMemsetAsync(g->d_sched, 0, sizeof(Sched), g->stream));
+    rc = run_opacity(g, p, g->two_bin, g->d_acc);
+    if (rc) return rc;
     const int ns = (int)g->L.size();
     const int l0 = p->level0;
-    // block size: the caller's (or 128), at most what the trace kernels are built for
-    const int threads = std::min(p->block_threads > 0 ? p->block_threads : 128, kTraceMaxThreads);
+    const int threads = trace_threads(p);
     TraceArgs A = make_args(g, p);
     if (p->schedule == ART_SCHED_PLAIN) {
         int per_sm = 0;
@@ -548,7 +570,7 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
         if (per_sm < 1) return ART_EINVAL;
         const int grid = per_sm * g->sms;
         for (int s = 0; s < ns; ++s) {
-            k_reset_counts<<<1, 32, 0, g->stream>>>(g->d_sched);
+            k_reset_counts<<<1, 32, 0, g->stream>>>(g->d_sched, (unsigned)(grid * (threads / 32)));
             for (int l = l0; l <= g->src_lmax[s]; ++l)
                 kern<<<grid, threads, 0, g->stream>>>(A, l, (unsigned)s);
         }
@@ -578,9 +600,9 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     const float gscale = (float)(p->sigma_H * g->dx / dV);
     const float fscale = (float)(1.0 / dV);
     const float escale = (float)(g->dx / dV);
-    int blocks = (int)std::min<long long>((g->ncell + 255) / 256, (long long)g->sms * 16);
-    k_finalize<<<blocks, 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2], g->d_acc, gscale,
-                                              fscale, escale, d_gamma, d_force, d_energy);
+    k_finalize<<<cell_blocks(g->ncell), 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2], g->d_acc,
+                                                             gscale, fscale, escale, d_gamma,
+                                                             d_force, d_energy);
     ART_TRY(cudaGetLastError());
     ART_TRY(cudaMemcpyAsync(g->h_stats, g->d_stats, sizeof(DevStats), cudaMemcpyDeviceToHost,
                             g->stream));
@@ -613,8 +635,7 @@ void art_destroy_grid(art_grid* g)
     dev_free(g->d_acc);
     dev_free(g->d_src);
     dev_free(g->d_levels);
-    dev_free(g->d_sched);
-    dev_free(g->d_stats);
+    dev_free(g->d_state);
     dev_free(g->d_srcL);
     dev_free(g->d_rec);
     dev_free(g->d_recf);

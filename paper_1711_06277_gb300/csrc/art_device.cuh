@@ -21,7 +21,8 @@
 
 namespace art {
 
-constexpr int kNL = 20;                 // level slots (levels 0..13 used)
+constexpr int kNL = 20;                 // level slots
+constexpr int kLevels = 14;             // levels 0..13 are used
 constexpr unsigned kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------------------------------
@@ -158,11 +159,16 @@ struct DevStats {
 struct Sched {
     unsigned long long count[kNL];   // rays held in the level buffer (a stack, top = count)
     unsigned long long cursor[kNL];  // next ray of the current phase / launch
-    unsigned long long phase_end;
+    unsigned long long phase_begin, phase_end;
     int phase_level, phase_width, phase_strided, phase_kind, done, started;
     // adjoint: quads of a level whose descendants are still being swept
     unsigned long long open_begin[kNL], open_end[kNL];
     unsigned bar_count, bar_gen;
+};
+
+struct DevState {
+    Sched sched;
+    DevStats stats;
 };
 
 // Everything the trace kernels read.
@@ -252,6 +258,42 @@ struct Path {
     int ss[3];    // signed index step of a crossing on each axis
 };
 
+// An opacity coefficient (cross section times cell length) in two floats; wide marks one whose
+// parts do not fit (the opacity is then formed in FP64).
+struct Coef {
+    float hi, lo;
+    double full;
+    int wide;
+};
+
+// c n to float: the product in two floats, rounded once (in FP64, at 1/64 of the FP32 rate, the
+// conversions alone bounded the opacity pass: 24 us for 128^3 cells).
+__device__ __forceinline__ df coef_times(const Coef& c, float n)
+{
+    const float p = c.hi * n;
+    return {p, fmaf(c.lo, n, fmaf(c.hi, n, -p))};
+}
+
+__device__ __forceinline__ bool bad_density(float v) { return !(v >= 0.f) || isinf(v); }
+
+// Opacity per cell length of a cell with neutral density a and total density b (0 without dust):
+// neutral-H part, dust part and their sum, each rounded once from the exact value.
+__device__ __forceinline__ void opacities(const Coef& sH, const Coef& sd, float a, float b,
+                                          float& chi, float& chiH, float& dust)
+{
+    if (sH.wide | sd.wide | !(a < 1e18f) | !(b < 1e18f)) {
+        const double h = (double)a * sH.full, d = (double)b * sd.full;
+        chi = __double2float_rn(h + d);
+        chiH = __double2float_rn(h);
+        dust = __double2float_rn(d);
+        return;
+    }
+    const df h = coef_times(sH, a), d = coef_times(sd, b);
+    chiH = h.hi + h.lo;
+    dust = d.hi + d.lo;
+    chi = df_add(h, d).hi;
+}
+
 // Cell records are stored with a ring of sentinel cells around the nx*ny*nz grid (opacity
 // < 0): cell (i, j, k) sits at (i + 1) + (nx + 2) ((j + 1) + (ny + 2) (k + 1)). A ray leaves
 // the grid when the cell it steps into is a sentinel, so the walk keeps no per-axis count of
@@ -275,6 +317,32 @@ __device__ __forceinline__ bool unpad(unsigned q, int nx, int ny, int nz, unsign
     const int Z = (int)(r / py) - 1;
     i = (unsigned)X + (unsigned)nx * ((unsigned)Y + (unsigned)ny * (unsigned)Z);
     return X >= 0 && X < nx && Y >= 0 && Y < ny && Z >= 0 && Z < nz;
+}
+
+// Runs store(q, inside, load(i)) for every padded cell q, i its index in the caller's layout
+// (load runs for cells of the grid only). Four cells per thread and round keep four loads in
+// flight; one at a time in a grid-stride loop had taken 17 us for 128^3 cells.
+template <class Load, class Store>
+__device__ __forceinline__ void each_padded_cell(int nx, int ny, int nz, Load load, Store store)
+{
+    const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
+    const unsigned long long step = 4ull * gridDim.x * blockDim.x;
+    for (unsigned long long base = 4ull * blockIdx.x * blockDim.x + threadIdx.x; base < npad; base += step) {
+        decltype(load(0u)) v[4] = {};
+        bool in[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long q = base + (unsigned)k * blockDim.x;
+            unsigned i = 0;
+            in[k] = q < npad && unpad((unsigned)q, nx, ny, nz, i);
+            if (in[k]) v[k] = load(i);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long q = base + (unsigned)k * blockDim.x;
+            if (q < npad) store((unsigned)q, in[k], v[k]);
+        }
+    }
 }
 
 // Padded index of cell i of the caller's nx*ny*nz layout.
@@ -598,10 +666,10 @@ __device__ __forceinline__ void red_v4_if(float4* __restrict__ acc, int key, flo
 // ---------------------------------------------------------------------------------------
 // helpers shared by the forward and backward kernels
 // ---------------------------------------------------------------------------------------
-// Threads per block of the trace kernels at most, and blocks per SM that the register budget
-// must leave room for (65536 / (128 * 5) = 102 registers a thread: two walks).
-constexpr int kTraceMaxThreads = 128;
-constexpr int kTraceMinBlocks = 5;
+// Threads per block of the trace kernels at most: one block of 20 warps per SM (65536 / 640 =
+// 102 registers a thread: two walks), so that a grid barrier has 152 arrivals and not 760.
+constexpr int kTraceMaxThreads = 640;
+constexpr int kTraceMinBlocks = 1;
 // Steps between checks whether a warp still has rays.
 constexpr int kCheckSteps = 4;
 
@@ -667,12 +735,39 @@ __device__ __forceinline__ void df_accumulate(df& s, float v)
     s.lo += r.lo;
 }
 
+// Items of a front are taken 32 at a time, the first by the warp's place in the grid (the warps of
+// an SM far apart, so that a small front spreads over the chip), further ones from a cursor
+// that starts behind those: a front of one round costs no atomics, where one per warp on one
+// address had taken microseconds.
+__device__ __forceinline__ unsigned warps_in_grid() { return gridDim.x * (blockDim.x >> 5); }
+
+struct Batches {
+    unsigned long long* cursor;
+    unsigned next, items;
+    bool first;
+    __device__ __forceinline__ Batches(unsigned long long* c, unsigned begin, unsigned n)
+        : cursor(c), next(begin + 32u * ((threadIdx.x >> 5) * gridDim.x + blockIdx.x)), items(n),
+          first(true) {}
+    // First item of the warp's next batch, or a value >= items when there is none. Warp-uniform.
+    __device__ __forceinline__ unsigned take(unsigned begin)
+    {
+        if (first) {
+            first = false;
+            return next;
+        }
+        if (begin + 32u * warps_in_grid() >= items) return items;
+        unsigned b = 0;
+        if ((threadIdx.x & 31u) == 0)
+            b = (unsigned)min(atomicAdd(cursor, 32ull), (unsigned long long)items);
+        return __shfl_sync(kFull, b, 0);
+    }
+};
+
 // Rays per lane for a front of `quads` quads: one while that fits the chip's warps in one
-// round (latency counts there, and a step of one ray is shorter), else two; two at the base
-// level.
-__device__ __forceinline__ int front_width(bool base, unsigned long long quads)
+// round (latency counts there, and a step of one ray is shorter), else two.
+__device__ __forceinline__ int front_width(unsigned long long quads)
 {
-    return !base && 4 * quads <= (unsigned long long)gridDim.x * blockDim.x ? 1 : 2;
+    return 4 * quads <= (unsigned long long)gridDim.x * blockDim.x ? 1 : 2;
 }
 
 // Where a ray of a level with split radius rmax ends: at rmax if it can split and (kCut) at
@@ -720,32 +815,33 @@ __device__ __forceinline__ bool grid_barrier(Sched* sc, DevStats* st, long long 
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        volatile unsigned* gen = &sc->bar_gen;
-        const unsigned g = *gen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(&sc->bar_count, 1u) + 1u;
-        if (arrived == gridDim.x) {
-            __threadfence();
+        unsigned g, arrived;
+        asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(g) : "l"(&sc->bar_gen) : "memory");
+        // release this block's writes, acquire those of the blocks before it
+        asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;"
+                     : "=r"(arrived) : "l"(&sc->bar_count) : "memory");
+        if (arrived + 1u == gridDim.x) {
             last();
-            atomicExch(&sc->bar_count, 0u);
-            __threadfence();
-            atomicAdd(&sc->bar_gen, 1u);
+            sc->bar_count = 0u;
+            asm volatile("st.release.gpu.u32 [%0], %1;" :: "l"(&sc->bar_gen), "r"(g + 1u) : "memory");
         } else {
             const unsigned long long t0 = global_ns();
-            while (*gen == g) {
+            for (;;) {
+                unsigned now;
+                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(now) : "l"(&sc->bar_gen) : "memory");
+                if (now != g) break;
                 if (wait_ns < 0 || (long long)(global_ns() - t0) > wait_ns) {
                     atomicCAS(&st->error, 0, -4);  // ART_ETIMEOUT
                     ok = 0;
                     break;
                 }
-                __nanosleep(40);
             }
         }
-        __threadfence();
         if (*((volatile int*)&st->error) != 0) ok = 0;
         s_ok = ok;
     }
     __syncthreads();
     return s_ok != 0;
 }
+
 }  // namespace art

@@ -59,8 +59,9 @@ struct art_grid {
     art::SrcDev* d_src = nullptr;
     size_t src_cap = 0;
     art::LevelInfo* d_levels = nullptr;
-    art::Sched* d_sched = nullptr;
-    art::DevStats* d_stats = nullptr;
+    art::DevState* d_state = nullptr;  // scheduler and counters, cleared together
+    art::Sched* d_sched = nullptr;     // in d_state
+    art::DevStats* d_stats = nullptr;  // in d_state
     art::DevStats* h_stats = nullptr;  // pinned
 
     float4* dir[art::kNL] = {};     // per level: 3 float4 per pixel (n and 1/n as df)
@@ -108,9 +109,12 @@ struct art_grid {
 namespace art {
 int check_params(const art_params* p);
 int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto);
-int run_opacity(art_grid* g, const art_params* p, bool two_bin);
+int run_opacity(art_grid* g, const art_params* p, bool two_bin, float4* acc);
+int trace_threads(const art_params* p);
+int cell_blocks(long long n);
 double rmax_cells(double m_ray, int level);
 fix to_fix(double cells, int fbits);
+Coef coef_of(double v);
 SrcDev source_record(const art_grid* g, const double u[3], double base_L, int lmax);
 int prepare_trace(art_grid* g, const art_params* p, bool adjoint);
 TraceArgs make_args(art_grid* g, const art_params* p);

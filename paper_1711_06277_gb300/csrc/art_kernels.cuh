@@ -128,35 +128,34 @@ __global__ void k_directions(int level, unsigned long long npix, double r0, doub
 }
 
 // chi per cell length (dx) in FP32 from the density fields, in the padded layout with the
-// sentinel ring; flags bad densities.
-__global__ void k_opacity(int nx, int ny, int nz, const float* __restrict__ nH0,
-                          const float* __restrict__ nH, double sH_dx, double sd_dx,
-                          float* __restrict__ chi, float2* __restrict__ chi2,
-                          DevStats* __restrict__ st)
+// sentinel ring; flags bad densities and clears the accumulator (if given).
+__global__ void __launch_bounds__(256) k_opacity(int nx, int ny, int nz,
+                                                 const float* __restrict__ nH0,
+                                                 const float* __restrict__ nH, Coef sH, Coef sd,
+                                                 float* __restrict__ chi,
+                                                 float2* __restrict__ chi2,
+                                                 float4* __restrict__ acc,
+                                                 DevStats* __restrict__ st)
 {
-    const unsigned npad = (unsigned)(nx + 2) * (unsigned)(ny + 2) * (unsigned)(nz + 2);
-    const unsigned step = gridDim.x * blockDim.x;
     bool bad = false;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const size_t npad = (size_t)(nx + 2) * (ny + 2) * (nz + 2);
         chi[npad] = kEnded;
         if (chi2) chi2[npad] = make_float2(kEnded, 0.f);
     }
-    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < npad; q += step) {
-        unsigned i;
-        if (!unpad(q, nx, ny, nz, i)) {
-            chi[q] = kSentinel;
-            if (chi2) chi2[q] = make_float2(kSentinel, 0.f);
-            continue;
-        }
-        float a = nH0[i];
-        float b = nH ? nH[i] : 0.f;
-        bad = bad || !(a >= 0.f) || !(b >= 0.f) || isinf(a) || isinf(b);
-        double h = (double)a * sH_dx;
-        const double dust = (double)b * sd_dx;
-        chi[q] = __double2float_rn(h + dust);
-        if (chi2) chi2[q] = make_float2(__double2float_rn(h + dust), __double2float_rn(dust));
-    }
-    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicCAS(&st->error, 0, -1);
+    each_padded_cell(
+        nx, ny, nz, [&](unsigned i) { return make_float2(nH0[i], nH ? nH[i] : 0.f); },
+        [&](unsigned q, bool inside, float2 v) {
+            float c = kSentinel, h, dust = 0.f;
+            if (inside) {
+                bad = bad || bad_density(v.x) || bad_density(v.y);
+                opacities(sH, sd, v.x, v.y, c, h, dust);
+            }
+            chi[q] = c;
+            if (chi2) chi2[q] = make_float2(c, dust);
+            if (acc) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        });
+    if (bad) atomicCAS(&st->error, 0, -1);
 }
 
 // The per-cell records a trace gathers: opacities (one bin) or opacity pairs (two bins).
@@ -195,14 +194,22 @@ __device__ __forceinline__ void lose(V& L, V& Lc, V dL)
     L = Lnew;
 }
 
+// Deposits of the first segments of second groups, one slot per thread.
+__device__ __forceinline__ float4* second_slots()
+{
+    __shared__ float4 s[kTraceMaxThreads];
+    return s;
+}
+
 // Walks kWidth (1 or 2) rays per lane: the rays of quads [begin, end) of level l, taken 32
 // lanes at a time from `cursor`, which counts items of kWidth rays. Base-level quads are
-// implied by their index (src0 is the first source), deeper ones are records; strided says
-// that a lane takes two base rays 32 apart instead of neighbours. Warp-uniform.
+// implied by their index (src0 is the first source), deeper ones are records. strided says that
+// base rays come in whole groups of 64: a lane takes two rays 32 apart instead of neighbours,
+// or two batches make a group. Warp-uniform.
 template <class Cell, bool kCut, int kWidth>
 __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, int l,
-                           unsigned long long* cursor, unsigned long long end, unsigned src0,
-                           bool strided)
+                           unsigned long long* cursor, unsigned long long begin,
+                           unsigned long long end, unsigned src0, bool strided)
 {
     constexpr bool two = TwoBin<Cell>::value;
     using V = typename std::conditional<kWidth == 1, float, float2>::type;
@@ -210,16 +217,16 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt = (1u << lane) - 1u;
     const LevelInfo& LV = A.levels[l];
-    const bool base = kWidth == 2 && l == A.level0;  // base rays are walked two per lane
+    const bool base = l == A.level0;
     BlockTally& T = block_tally();
-    __shared__ float4 s_second[kTraceMaxThreads];
+    float4* const s_second = second_slots();
     const unsigned items = (unsigned)end * kPerQuad;  // front ends below 2^29 quads
+    const unsigned first = (unsigned)begin * kPerQuad;
+    Batches batches(cursor, first, items);
     unsigned ncross = 0;
 
     for (;;) {
-        unsigned b = 0;
-        if (lane == 0) b = (unsigned)min(atomicAdd(cursor, 32ull), (unsigned long long)items);
-        b = __shfl_sync(kFull, b, 0);
+        const unsigned b = batches.take(first);
         if (b >= items) break;
 
         // ---- set-up: a part of a quad per lane
@@ -229,13 +236,13 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
         Photons<V> P;
         float cell[kWidth], celln[kWidth];
         unsigned s = 0, pix = 0;
-        const unsigned apart = strided ? 32u : 1u;  // between the pixels of a lane's rays
+        const unsigned apart = kWidth == 2 && strided ? 32u : 1u;  // between a lane's pixels
         fix rend = kNoEnd;
         bool splits = false;
         P.L = P.tau = P.Lc = P.Ln = P.taun = P.Lnc = vset<V>(0.f);
         if (valid) {
             unsigned quad = item / kPerQuad, part = item % kPerQuad * kWidth;
-            if (strided) {
+            if (kWidth == 2 && strided) {
                 quad = (2u * b + lane) / 4u;
                 part = lane % 4u;
             }
@@ -333,22 +340,25 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
 #pragma unroll
             for (int j = 0; j < kWidth; ++j)
                 v[j] = make_float4(vget(G, j), vget(f0, j), vget(f1, j), vget(f2, j));
-            if constexpr (kWidth == 2 && decltype(first)::value) {
-                if (!strided) merge_pair(key[0], v[0], key[1], v[1], -2);
-                merge_lanes(key[0], v[0]);
-                merge_lanes(key[1], v[1]);
-                red_v4_if(A.acc, key[0], v[0]);
-                second_key = key[1];
-                s_second[threadIdx.x] = v[1];
+            if constexpr (decltype(first)::value) {
+                // the second of two groups of 32 waits until the walk is done
+                const bool later = kWidth == 1 && strided && (b / 32u) % 2u == 1u;
+                if constexpr (kWidth == 2)
+                    if (!strided) merge_pair(key[0], v[0], key[1], v[1], -2);
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j) merge_lanes(key[j], v[j]);
+                if (!later) red_v4_if(A.acc, key[0], v[0]);
+                second_key = kWidth == 2 ? key[kWidth - 1] : (later ? key[0] : -1);
+                s_second[threadIdx.x] = v[kWidth - 1];
             } else {
                 if constexpr (kWidth == 2) merge_pair(key[0], v[0], key[1], v[1], -2);
 #pragma unroll
                 for (int j = 0; j < kWidth; ++j) red_v4_if(A.acc, key[j], v[j]);
             }
         };
-        // The first segments of base rays all lie in their source's cell: a warp deposits those
-        // of each of its two groups of 32 as one sum, the second when the walk is done, so that
-        // the additions to that one cell are spread over the phase.
+        // The first segments of base rays all lie in their source's cell: those of 32 rays are
+        // deposited as one sum, in every second such group when the walk is done, so that the
+        // additions to that one cell are spread over the phase.
         if (base) step(std::true_type{});
         for (;;) {
             bool any = false;
@@ -361,32 +371,39 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
         }
         if (base) red_v4_if(A.acc, second_key, s_second[threadIdx.x]);
 
-        // ---- ends: tallies, and the children of split rays
-        bool child[kWidth];
+        // ---- ends: the children of split rays, and tallies (while the reservation of the
+        // children's slots is on its way)
+        bool child[kWidth], drop[kWidth];
         unsigned nchild = 0, mine = 0, at[kWidth];
-        df esc = {0.f, 0.f}, dropped = {0.f, 0.f}, escn = {0.f, 0.f}, droppedn = {0.f, 0.f};
 #pragma unroll
         for (int j = 0; j < kWidth; ++j) {
-            const bool drop = vget(two ? P.taun : P.tau, j) > A.tau_max;
-            child[j] = valid && cell[j] == kEnded && !drop &&
+            drop[j] = vget(two ? P.taun : P.tau, j) > A.tau_max;
+            child[j] = valid && cell[j] == kEnded && !drop[j] &&
                        splits_at_end<kCut>(splits, LV.rmaxx, A.dmax);
             const unsigned m = __ballot_sync(kFull, child[j]);
             // children in pixel order: group after group, or lane after lane
-            at[j] = __popc(m & lt) + (strided ? nchild : mine);
-            if (!strided && j > 0) {
+            at[j] = __popc(m & lt) + (apart > 1u ? nchild : mine);
+            if (apart == 1u && j > 0) {
                 at[j] += at[0];
                 at[0] += __popc(m & lt);
             }
             nchild += __popc(m);
             mine += child[j] ? 1u : 0u;
+        }
+        unsigned slot = 0;
+        if (lane == 0 && nchild)
+            slot = (unsigned)atomicAdd(&A.sched->count[l + 1], (unsigned long long)nchild);
+        df esc = {0.f, 0.f}, dropped = {0.f, 0.f}, escn = {0.f, 0.f}, droppedn = {0.f, 0.f};
+        if (valid) {
             // leaving the box or cut at d_max: escaped; tau > tau_max: dropped. A split ray
             // leaves its ledger residual: its children start from L itself.
-            if (valid) {
-                df& to = drop ? dropped : esc;
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j) {
+                df& to = drop[j] ? dropped : esc;
                 df_accumulate(to, child[j] ? 0.f : vget(P.L, j));
                 df_accumulate(to, vget(P.Lc, j));
                 if constexpr (two) {
-                    df& ton = drop ? droppedn : escn;
+                    df& ton = drop[j] ? droppedn : escn;
                     df_accumulate(ton, child[j] ? 0.f : vget(P.Ln, j));
                     df_accumulate(ton, vget(P.Lnc, j));
                 }
@@ -398,12 +415,10 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
             T.escaped_n[threadIdx.x] += (double)escn.hi + (double)escn.lo;
             T.dropped_n[threadIdx.x] += (double)droppedn.hi + (double)droppedn.lo;
         }
-        const unsigned nray = kWidth * min(items - b, 32u);
-        unsigned slot = 0;
         if (lane == 0) {
+            const unsigned nray = kWidth * min(items - b, 32u);
             atomicAdd(&T.rays[l], (unsigned long long)nray);
             atomicAdd(&T.destroy, (unsigned long long)(nray - nchild) * LV.destroy_w);
-            if (nchild) slot = (unsigned)atomicAdd(&A.sched->count[l + 1], (unsigned long long)nchild);
         }
         if (nchild) {
             const QuadBuf& C = A.quad[l + 1];
@@ -441,11 +456,11 @@ __device__ __forceinline__ bool front_strided(const TraceArgs& A, bool base,
 
 template <class Cell, bool kCut>
 __device__ __forceinline__ void run_front(const TraceArgs& A, int l, int width,
-                                          unsigned long long* cursor, unsigned long long end,
-                                          unsigned src0, bool strided)
+                                          unsigned long long* cursor, unsigned long long begin,
+                                          unsigned long long end, unsigned src0, bool strided)
 {
-    if (width == 2) walk_front<Cell, kCut, 2>(A, cells_of<Cell>(A), l, cursor, end, src0, strided);
-    else walk_front<Cell, kCut, 1>(A, cells_of<Cell>(A), l, cursor, end, src0, false);
+    if (width == 2) walk_front<Cell, kCut, 2>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, strided);
+    else walk_front<Cell, kCut, 1>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, false);
 }
 
 // Plain schedule: the whole front of level l of source s.
@@ -457,34 +472,44 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_lev
     const unsigned long long end =
         l == A.level0 ? (unsigned long long)A.base_quads
                       : min(*((volatile unsigned long long*)&A.sched->count[l]), A.quad[l].cap);
-    run_front<Cell, kCut>(A, l, front_width(l == A.level0, end), &A.sched->cursor[l], end, s,
+    run_front<Cell, kCut>(A, l, front_width(end), &A.sched->cursor[l], 0, end, s,
                           front_strided(A, l == A.level0, 0, end));
     block_tally_flush(A.stats);
 }
 
-// Resets the per-level counters of the plain schedule before the next source.
-__global__ void k_reset_counts(Sched* sc)
+// Resets the per-level counters of the plain schedule before the next source, whose launches
+// have `warps` warps.
+__global__ void k_reset_counts(Sched* sc, unsigned warps)
 {
     int t = threadIdx.x;
-    if (t < kNL) { sc->count[t] = 0; sc->cursor[t] = 0; }
+    if (t < kNL) { sc->count[t] = 0; sc->cursor[t] = 32ull * warps; }
 }
 
 // Chooses the next phase of the persistent schedule (run by one thread, all others waiting).
 __device__ __forceinline__ void next_phase(const TraceArgs& A)
 {
-    volatile Sched* sc = A.sched;
-    if (!sc->started) {
-        sc->started = 1;
-        sc->count[A.level0] = (unsigned long long)A.base_quads * A.nsrc;
-    }
+    Sched* sc = A.sched;
+    const int started = __ldcg(&sc->started);
     int l = -1;
-    for (int k = A.lmax_glob; k >= A.level0; --k)
-        if (sc->count[k] > 0) { l = k; break; }
+    unsigned long long have = 0;
+    // the counts of all levels are read side by side (one after the other they took 2 us)
+#pragma unroll
+    for (int k = 0; k < kLevels; ++k) {
+        const unsigned long long c = __ldcg(&sc->count[k]);
+        if (c > 0) {
+            l = k;
+            have = c;
+        }
+    }
+    if (!started) {
+        l = A.level0;
+        have = (unsigned long long)A.base_quads * A.nsrc;
+    }
+    sc->started = 1;
     if (l < 0) {
         sc->done = 1;
         return;
     }
-    const unsigned long long have = sc->count[l];
     unsigned long long take = have;
     if (l < A.lmax_glob) take = min(have, A.quad[l + 1].cap / 4);
     if (take == 0) {  // a phase must consume rays, or the schedule never ends
@@ -493,12 +518,13 @@ __device__ __forceinline__ void next_phase(const TraceArgs& A)
     }
     const bool base = l == A.level0;
     if (base && take > 16) take -= (have - take) % 16u ? 16u - (have - take) % 16u : 0u;
-    const int width = front_width(base, take);
+    const int width = front_width(take);
     sc->phase_strided = front_strided(A, base, have - take, have);
     sc->phase_level = l;
     sc->phase_width = width;
     sc->phase_end = have;
-    sc->cursor[l] = (have - take) * (unsigned long long)(4 / width);
+    sc->phase_begin = have - take;
+    sc->cursor[l] = (have - take) * (unsigned long long)(4 / width) + 32ull * warps_in_grid();
     sc->count[l] = have - take;
 }
 
@@ -509,41 +535,54 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_per
     block_tally_init();
     Sched* sc = A.sched;
     __shared__ int s_level, s_width, s_strided;
-    __shared__ unsigned long long s_end;
+    __shared__ unsigned long long s_begin, s_end;
     for (;;) {
         if (!grid_barrier(sc, A.stats, A.wait_ns, [&] { next_phase(A); })) break;
         if (threadIdx.x == 0) {
-            volatile Sched* v = sc;
-            s_level = v->done ? -1 : v->phase_level;
-            s_width = v->phase_width;
-            s_strided = v->phase_strided;
-            s_end = v->phase_end;
+            s_level = __ldcg(&sc->done) ? -1 : __ldcg(&sc->phase_level);
+            s_width = __ldcg(&sc->phase_width);
+            s_strided = __ldcg(&sc->phase_strided);
+            s_begin = __ldcg(&sc->phase_begin);
+            s_end = __ldcg(&sc->phase_end);
         }
         __syncthreads();
         const int l = s_level;
         if (l < 0) break;
-        run_front<Cell, kCut>(A, l, s_width, &sc->cursor[l], s_end, 0u, s_strided != 0);
+        run_front<Cell, kCut>(A, l, s_width, &sc->cursor[l], s_begin, s_end, 0u, s_strided != 0);
     }
     block_tally_flush(A.stats);
 }
 
 // Gamma, force and energy from the accumulator (padded layout) into the caller's SoA
-// outputs (nx*ny*nz layout).
-__global__ void k_finalize(int nx, int ny, int nz, const float4* __restrict__ acc, float gscale,
-                           float fscale, float escale, float* __restrict__ gamma,
-                           float* __restrict__ force, float* __restrict__ energy)
+// outputs (nx*ny*nz layout), four cells per thread and round.
+__global__ void __launch_bounds__(256) k_finalize(int nx, int ny, int nz,
+                                                  const float4* __restrict__ acc, float gscale,
+                                                  float fscale, float escale,
+                                                  float* __restrict__ gamma,
+                                                  float* __restrict__ force,
+                                                  float* __restrict__ energy)
 {
     const unsigned ncell = (unsigned)nx * (unsigned)ny * (unsigned)nz;
-    const unsigned step = gridDim.x * blockDim.x;
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < ncell; i += step) {
-        const float4 a = __ldcs(acc + pad_of(i, nx, ny));
-        gamma[i] = gscale * a.x;
-        if (force) {
-            force[i] = fscale * a.y;
-            force[(size_t)ncell + i] = fscale * a.z;
-            force[2 * (size_t)ncell + i] = fscale * a.w;
+    const unsigned long long step = 4ull * gridDim.x * blockDim.x;
+    for (unsigned long long base = 4ull * blockIdx.x * blockDim.x + threadIdx.x; base < ncell; base += step) {
+        float4 a[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long i = base + (unsigned)k * blockDim.x;
+            if (i < ncell) a[k] = __ldcs(acc + pad_of((unsigned)i, nx, ny));
         }
-        if (energy) energy[i] = escale * a.x;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long i = base + (unsigned)k * blockDim.x;
+            if (i >= ncell) break;
+            gamma[i] = gscale * a[k].x;
+            if (force) {
+                force[i] = fscale * a[k].y;
+                force[(size_t)ncell + i] = fscale * a[k].z;
+                force[2 * (size_t)ncell + i] = fscale * a[k].w;
+            }
+            if (energy) energy[i] = escale * a[k].x;
+        }
     }
 }
 
