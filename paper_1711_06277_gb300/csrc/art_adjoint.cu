@@ -79,13 +79,6 @@ __device__ __forceinline__ void dl_add(double* dL, unsigned src, bool valid, dou
     }
 }
 
-__device__ __forceinline__ void red_f32_if(float* base, int key, float v)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %1, 0;\n\t"
-                 "@q red.global.add.f32 [%0], %2;\n\t}"
-                 :: "l"(base + key), "r"(key), "f"(v) : "memory");
-}
-
 // The parts of a cell record: opacity, its neutral-H part, weight, and the force weight of the
 // segment q = (v . n) / dV, so that the segment adds q dL to the loss (0 without a force term).
 __device__ __forceinline__ float neutral_of(const float4& c) { return c.y; }
@@ -198,19 +191,33 @@ __device__ __forceinline__ void walkers_step(const TraceArgs& A, const Cell* __r
     constexpr bool force = HasForce<Cell>::value;
     V ds, x, wk, hv, q = vset<V>(0.f);
     int key[kWidth];
+    bool alive[kWidth], exact = false;
+    int high[kWidth];
 #pragma unroll
     for (int j = 0; j < kWidth; ++j) {
-        const float chi = chi_of(R.cell[j]), depth = vget(R.tau, j);
-        const bool alive = !(chi < 0.f) & !(depth > A.tau_max);
+        bool e;
+        alive[j] = !(chi_of(R.cell[j]) < 0.f) & !(vget(R.tau, j) > A.tau_max);
+        high[j] = earliest(R.W[j], rend, alive[j], e);
+        exact |= e;
         // (a ray that has ended may hold the record of a cell it never entered)
-        vget(wk, j) = alive ? weight_of(R.cell[j]) * A.gscale : 0.f;
+        vget(wk, j) = alive[j] ? weight_of(R.cell[j]) * A.gscale : 0.f;
         vget(hv, j) = neutral_of(R.cell[j]);
         if constexpr (force)
-            vget(q, j) = alive ? force_weight(R.cell[j], R.n[j], A.fscale) : 0.f;
-        walk_move<kParts>(R.W[j], rend, A.unit, chi, depth, A.tau_max, -1 - j, (int)A.npad,
-                          vget(ds, j), vget(x, j), key[j], ncross);
-        load_if(alive, recs + R.W[j].idx, R.cell[j]);
+            vget(q, j) = alive[j] ? force_weight(R.cell[j], R.n[j], A.fscale) : 0.f;
     }
+    if (exact) {
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j)
+            walk_move<true, kParts>(R.W[j], rend, A.unit, chi_of(R.cell[j]), alive[j], high[j],
+                                    -1 - j, (int)A.npad, vget(ds, j), vget(x, j), key[j], ncross);
+    } else {
+#pragma unroll
+        for (int j = 0; j < kWidth; ++j)
+            walk_move<false, kParts>(R.W[j], rend, A.unit, chi_of(R.cell[j]), alive[j], high[j],
+                                     -1 - j, (int)A.npad, vget(ds, j), vget(x, j), key[j], ncross);
+    }
+#pragma unroll
+    for (int j = 0; j < kWidth; ++j) load_if(alive[j], recs + R.W[j].idx, R.cell[j]);
     V dphi;
     const V ph = phi_dphi<kPass == 2>(x, dphi);
     const V Lin = R.L;
@@ -232,16 +239,12 @@ __device__ __forceinline__ void walkers_step(const TraceArgs& A, const Cell* __r
 #pragma unroll
         for (int j = 0; j < kWidth; ++j) d[j] = vget(val, j);
         if constexpr (kWidth == 2)
-            asm("{\n\t.reg .pred q;\n\tsetp.eq.s32 q, %1, %2;\n\t@q add.f32 %0, %0, %3;\n\t"
-                "@q mov.b32 %1, -2;\n\t}" : "+f"(d[0]), "+r"(key[1]) : "r"(key[0]), "f"(d[1]));
+            merge_pair(key[0], d[0], key[1], d[1], -2);
 #pragma unroll
         for (int j = 0; j < kWidth; ++j) {
-            if constexpr (kFirst) {  // all in their source's cell: one sum per warp
-                float4 v = make_float4(d[j], 0.f, 0.f, 0.f);
-                merge_lanes(key[j], v);
-                d[j] = v.x;
-            }
-            red_f32_if(A.grad, key[j], d[j]);
+            // the first segments are all in their source's cell: one sum per warp
+            if constexpr (kFirst) merge_lanes(key[j], d[j]);
+            red_if(A.grad, key[j], d[j]);
         }
     }
 }
@@ -568,8 +571,10 @@ __global__ void __launch_bounds__(256) k_pack_cells(int nx, int ny, int nz,
 // Gradient per cell from the padded scratch it was summed in, into the caller's layout.
 __global__ void __launch_bounds__(256) k_unpad_grad(int nx, int ny, int nz,
                                                     const float* __restrict__ src,
-                                                    float* __restrict__ dst)
+                                                    float* __restrict__ dst,
+                                                    const DevStats* stats, DevStats* host)
 {
+    publish_stats(stats, host);
     const unsigned ncell = (unsigned)nx * (unsigned)ny * (unsigned)nz;
     const unsigned long long step = 4ull * gridDim.x * blockDim.x;
     for (unsigned long long base = 4ull * blockIdx.x * blockDim.x + threadIdx.x; base < ncell; base += step) {
@@ -687,11 +692,9 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if ((rc = status_of(cudaLaunchKernelEx(&cfg, kern, A)))) return rc;
-    k_unpad_grad<<<cell_blocks(g->ncell), 256, 0, st>>>(nx, ny, nz, grad_pad, d_dlog_nH0);
+    k_unpad_grad<<<cell_blocks(g->ncell), 256, 0, st>>>(nx, ny, nz, grad_pad, d_dlog_nH0,
+                                                       g->d_stats, g->h_stats);
     if ((rc = status_of(cudaGetLastError()))) return rc;
-    if ((rc = status_of(cudaMemcpyAsync(g->h_stats, g->d_stats, sizeof(DevStats),
-                                        cudaMemcpyDeviceToHost, st))))
-        return rc;
     g->last_L_in = 0.0;
     for (double v : g->L) g->last_L_in += v;
     g->last_lmax = g->lmax_glob;

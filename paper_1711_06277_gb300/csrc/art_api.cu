@@ -54,6 +54,31 @@ void split_df(double v, float& hi, float& lo)
     lo = (float)(v - (double)hi);
 }
 
+using LevelKernel = void (*)(TraceArgs, int, unsigned);
+using PersistentKernel = void (*)(TraceArgs);
+
+// The kernels for one or two bins, with or without a cutoff and a force.
+template <class Cell>
+LevelKernel level_kernel_of(bool cut, bool force)
+{
+    return cut ? (force ? k_trace_level<Cell, true, true> : k_trace_level<Cell, true, false>)
+               : (force ? k_trace_level<Cell, false, true> : k_trace_level<Cell, false, false>);
+}
+LevelKernel level_kernel(bool two_bin, bool cut, bool force)
+{
+    return two_bin ? level_kernel_of<float2>(cut, force) : level_kernel_of<float>(cut, force);
+}
+template <class Cell>
+PersistentKernel persistent_kernel_of(bool cut, bool force)
+{
+    return cut ? (force ? k_trace_persistent<Cell, true, true> : k_trace_persistent<Cell, true, false>)
+               : (force ? k_trace_persistent<Cell, false, true> : k_trace_persistent<Cell, false, false>);
+}
+PersistentKernel persistent_kernel(bool two_bin, bool cut, bool force)
+{
+    return two_bin ? persistent_kernel_of<float2>(cut, force) : persistent_kernel_of<float>(cut, force);
+}
+
 template <class T>
 int dev_alloc(T** p, size_t count)
 {
@@ -343,14 +368,15 @@ int trace_threads(const art_params* p)
 int cell_blocks(long long n) { return (int)((n + 1023) / 1024); }
 
 // Opacity per cell length (padded layout) into d_chi, and the two-bin pairs into d_chi2; clears
-// acc if given.
-int run_opacity(art_grid* g, const art_params* p, bool two_bin, float4* acc)
+// the accumulator of a trace with a force (clear4) or without (clear1).
+int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, bool clear1)
 {
     const Coef sH = coef_of(p->sigma_H * g->dx);
     const Coef sd = coef_of(g->nH ? p->sigma_d * g->dx : 0.0);
     k_opacity<<<cell_blocks(g->npad), 256, 0, g->stream>>>(
         g->n[0], g->n[1], g->n[2], g->nH0, g->nH, sH, sd, g->d_chi,
-        two_bin ? g->d_chi2 : nullptr, acc, g->d_stats);
+        two_bin ? g->d_chi2 : nullptr, clear4 ? g->d_acc : nullptr,
+        clear1 ? reinterpret_cast<float*>(g->d_acc) : nullptr, g->d_stats);
     ART_TRY(cudaGetLastError());
     return ART_OK;
 }
@@ -555,7 +581,7 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     ART_TRY(cudaMemsetAsync(g->d_state, 0, sizeof(DevState), g->stream));
     rc = prepare_trace(g, p, false);
     if (rc) return rc;
-    rc = run_opacity(g, p, g->two_bin, g->d_acc);
+    rc = run_opacity(g, p, g->two_bin, d_force != nullptr, d_force == nullptr);
     if (rc) return rc;
     const int ns = (int)g->L.size();
     const int l0 = p->level0;
@@ -563,9 +589,7 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     TraceArgs A = make_args(g, p);
     if (p->schedule == ART_SCHED_PLAIN) {
         int per_sm = 0;
-        const bool cut = p->d_max > 0.0;
-        auto kern = g->two_bin ? (cut ? k_trace_level<float2, true> : k_trace_level<float2, false>)
-                               : (cut ? k_trace_level<float, true> : k_trace_level<float, false>);
+        const auto kern = level_kernel(g->two_bin, p->d_max > 0.0, d_force != nullptr);
         ART_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0));
         if (per_sm < 1) return ART_EINVAL;
         const int grid = per_sm * g->sms;
@@ -577,10 +601,7 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
         ART_TRY(cudaGetLastError());
     } else {
         int per_sm = 0;
-        const bool cut = p->d_max > 0.0;
-        auto kern = g->two_bin
-                        ? (cut ? k_trace_persistent<float2, true> : k_trace_persistent<float2, false>)
-                        : (cut ? k_trace_persistent<float, true> : k_trace_persistent<float, false>);
+        const auto kern = persistent_kernel(g->two_bin, p->d_max > 0.0, d_force != nullptr);
         ART_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0));
         if (per_sm < 1) return ART_EINVAL;
         if (p->blocks_per_sm > 0 && p->blocks_per_sm < per_sm) per_sm = p->blocks_per_sm;
@@ -600,12 +621,17 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     const float gscale = (float)(p->sigma_H * g->dx / dV);
     const float fscale = (float)(1.0 / dV);
     const float escale = (float)(g->dx / dV);
-    k_finalize<<<cell_blocks(g->ncell), 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2], g->d_acc,
-                                                             gscale, fscale, escale, d_gamma,
-                                                             d_force, d_energy);
+    const int blocks = cell_blocks(g->ncell);
+    if (d_force)
+        k_finalize<<<blocks, 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2], g->d_acc, gscale,
+                                                  fscale, escale, d_gamma, d_force, d_energy, g->d_stats,
+                                                  g->h_stats);
+    else
+        k_finalize<<<blocks, 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2],
+                                                  reinterpret_cast<const float*>(g->d_acc), gscale,
+                                                  fscale, escale, d_gamma, d_force, d_energy, g->d_stats,
+                                                  g->h_stats);
     ART_TRY(cudaGetLastError());
-    ART_TRY(cudaMemcpyAsync(g->h_stats, g->d_stats, sizeof(DevStats), cudaMemcpyDeviceToHost,
-                            g->stream));
     double Lin = 0.0;
     for (double v : g->L) Lin += v;
     g->last_L_in = Lin;

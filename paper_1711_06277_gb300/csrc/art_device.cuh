@@ -155,6 +155,16 @@ struct DevStats {
     int error;
 };
 
+// Copies the counters to pinned host memory from a kernel that runs anyway (a copy of 224 bytes
+// of its own took 2 us of the stream).
+__device__ __forceinline__ void publish_stats(const DevStats* stats, DevStats* host)
+{
+    static_assert(sizeof(DevStats) % 8 == 0 && sizeof(DevStats) / 8 <= 32, "one warp copies it");
+    if (blockIdx.x == 0 && threadIdx.x < sizeof(DevStats) / 8)
+        reinterpret_cast<unsigned long long*>(host)[threadIdx.x] =
+            reinterpret_cast<const unsigned long long*>(stats)[threadIdx.x];
+}
+
 // Scheduler state of the persistent trace and of the plain per-level launches.
 struct Sched {
     unsigned long long count[kNL];   // rays held in the level buffer (a stack, top = count)
@@ -502,7 +512,7 @@ __device__ __forceinline__ V phi_dphi(V x, V& dphi)
 // joined before the advance, with the predicates of both paths, every step paid 18 more
 // instructions (14.3 against 12.2 ms on 256^3 / 16 sources).
 //   operands: 0-2 t, 3 tc, 4 idx, 5 ncross, 6 ds, 7 key, 8 x, 9 chi, 10-12 d, 13-15 ss,
-//   16 rend, 17 unit, 18 none, 19 npad, 20 depth, 21 limit
+//   16 rend, 17 unit, 18 none, 19 npad, 20 alive, 21 earliest high word
 #define ART_LENGTH "cvt.rn.f32.s64 fl, mv;\n\t"
 #define ART_LENGTH_PARTS \
     "cvt.rn.f32.s64 fm, m;\n\t" \
@@ -516,6 +526,13 @@ __device__ __forceinline__ V phi_dphi(V x, V& dphi)
     "sub.rn.f32 fm, fm, fc;\n\t" \
     "sub.rn.f32 gm, gm, gc;\n\t" \
     "add.rn.f32 fl, fm, gm;\n\t"
+#define ART_MOVE_REGS \
+    "{\n\t" \
+    ".reg .pred p0, p1, p2, ps, po, pa;\n\t" \
+    ".reg .b32 l0, l1, l2, lr, h0, h1, h2, hr, lm;\n\t" \
+    ".reg .f32 fl, fm, fc, gm, gc;\n\t" \
+    ".reg .b64 m, tol, d, mv, at;\n\t" \
+    "setp.ne.s32 po, %20, 0;\n\t"
 #define ART_MOVE_ADVANCE(LENGTH) \
     "sub.s64 mv, m, %3;\n\t" \
     LENGTH \
@@ -533,44 +550,24 @@ __device__ __forceinline__ V phi_dphi(V x, V& dphi)
     "@p1 add.s32 %4, %4, %14;\n\t" \
     "@p2 add.s32 %4, %4, %15;\n\t" \
     "@ps mov.b32 %4, %19;\n\t"
-#define ART_MOVE_PTX(LENGTH) \
-    "{\n\t" \
-    ".reg .pred p0, p1, p2, ps, ta, tb, tc, po, pa;\n\t" \
-    ".reg .b32 l0, l1, l2, lr, h0, h1, h2, hr, hm, lm, cl, ch;\n\t" \
-    ".reg .f32 fl, fm, fc, gm, gc;\n\t" \
-    ".reg .b64 m, tol, d, mv, at;\n\t" \
+#define ART_MOVE_FAST(LENGTH) \
+    ART_MOVE_REGS \
     "mov.b64 {l0, h0}, %0;\n\t" \
     "mov.b64 {l1, h1}, %1;\n\t" \
     "mov.b64 {l2, h2}, %2;\n\t" \
     "mov.b64 {lr, hr}, %16;\n\t" \
-    "mov.b64 {cl, ch}, %3;\n\t" \
-    "setp.geu.f32 po, %9, 0f00000000;\n\t" \
-    "setp.leu.and.f32 po, %20, %21, po;\n\t" \
-    "min.s32 hm, h0, h1;\n\t" \
-    "min.s32 hm, hm, h2;\n\t" \
-    "min.s32 hm, hm, hr;\n\t" \
-    "setp.eq.s32 p0, h0, hm;\n\t" \
-    "setp.eq.s32 p1, h1, hm;\n\t" \
-    "setp.eq.s32 p2, h2, hm;\n\t" \
-    "setp.eq.s32 ps, hr, hm;\n\t" \
-    "and.pred ta, p0, p1;\n\t" \
-    "or.pred tb, p0, p1;\n\t" \
-    "and.pred tc, tb, p2;\n\t" \
-    "or.pred ta, ta, tc;\n\t" \
-    "or.pred tb, tb, p2;\n\t" \
-    "and.pred tc, tb, ps;\n\t" \
-    "or.pred ta, ta, tc;\n\t" \
-    "setp.le.or.s32 ta, hm, ch, ta;\n\t" \
-    "and.pred ta, ta, po;\n\t" \
-    "@ta bra tie_%=;\n\t" \
+    "setp.eq.s32 p0, h0, %21;\n\t" \
+    "setp.eq.s32 p1, h1, %21;\n\t" \
+    "setp.eq.s32 p2, h2, %21;\n\t" \
+    "setp.eq.s32 ps, hr, %21;\n\t" \
     "selp.b32 lm, l2, lr, p2;\n\t" \
     "selp.b32 lm, l1, lm, p1;\n\t" \
     "selp.b32 lm, l0, lm, p0;\n\t" \
-    "mov.b64 m, {lm, hm};\n\t" \
+    "mov.b64 m, {lm, %21};\n\t" \
     "mov.pred pa, po;\n\t" \
-    ART_MOVE_ADVANCE(LENGTH) \
-    "bra moved_%=;\n\t" \
-    "tie_%=:\n\t" \
+    ART_MOVE_ADVANCE(LENGTH)
+#define ART_MOVE_EXACT(LENGTH) \
+    ART_MOVE_REGS \
     "min.s64 m, %0, %1;\n\t" \
     "min.s64 m, m, %2;\n\t" \
     "shr.s64 tol, m, 40;\n\t" \
@@ -583,37 +580,53 @@ __device__ __forceinline__ V phi_dphi(V x, V& dphi)
     "setp.le.s64 ps, %16, m;\n\t" \
     "selp.b64 m, %16, m, ps;\n\t" \
     "setp.gt.and.s64 pa, m, %3, po;\n\t" \
-    ART_MOVE_ADVANCE(LENGTH) \
-    "moved_%=:\n\t"
+    ART_MOVE_ADVANCE(LENGTH)
 #define ART_MOVE_OPERANDS                                                                      \
         : "+l"(W.t[0]), "+l"(W.t[1]), "+l"(W.t[2]), "+l"(W.tc), "+r"(W.idx), "+r"(ncross),     \
           "=&f"(ds), "=&r"(key), "=&f"(x), "+f"(chi)                                           \
         : "l"(W.d[0]), "l"(W.d[1]), "l"(W.d[2]), "r"(W.ss[0]), "r"(W.ss[1]), "r"(W.ss[2]),     \
-          "l"(rend), "f"(unit), "r"(none), "r"(npad), "f"(depth), "f"(limit)
+          "l"(rend), "f"(unit), "r"(none), "r"(npad), "r"((int)alive), "r"(high)
 
-// kParts: the length is the difference of the ends' leading 24 bits plus that of the rest. Both
-// forms round alike but for segments that more than double the distance from the source, the
-// first few of a ray.
-template <bool kParts>
-__device__ __forceinline__ void walk_move(Path& W, fix rend, float unit, float chi, float depth,
-                                          float limit, int none, int npad, float& ds, float& x,
-                                          int& key, unsigned& ncross)
+// High word of the earliest of the three faces and the end radius; exact says that the high
+// words do not decide the step of a ray that is alive.
+__device__ __forceinline__ int earliest(const Path& W, fix rend, bool alive, bool& exact)
 {
-    if constexpr (kParts) asm(ART_MOVE_PTX(ART_LENGTH_PARTS) "}" ART_MOVE_OPERANDS);
-    else asm(ART_MOVE_PTX(ART_LENGTH) "}" ART_MOVE_OPERANDS);
+    const int h0 = (int)(W.t[0] >> 32), h1 = (int)(W.t[1] >> 32), h2 = (int)(W.t[2] >> 32);
+    const int hr = (int)(rend >> 32), hc = (int)(W.tc >> 32);
+    const int a = min(h0, h1), b = max(h0, h1), c = min(h2, hr), d = max(h2, hr);
+    const int first = min(a, c), second = min(max(a, c), min(b, d));
+    exact = alive & ((second == first) | (first <= hc));
+    return first;
 }
 
-template <class Cell>
+// kExact: with the 64-bit comparison. kParts: the length is the difference of the ends' leading
+// 24 bits plus that of the rest; both forms round alike but for segments that more than double
+// the distance from the source, the first few of a ray.
+template <bool kExact, bool kParts>
+__device__ __forceinline__ void walk_move(Path& W, fix rend, float unit, float chi, bool alive,
+                                          int high, int none, int npad, float& ds, float& x,
+                                          int& key, unsigned& ncross)
+{
+    if constexpr (kExact && kParts) asm(ART_MOVE_EXACT(ART_LENGTH_PARTS) "}" ART_MOVE_OPERANDS);
+    else if constexpr (kExact) asm(ART_MOVE_EXACT(ART_LENGTH) "}" ART_MOVE_OPERANDS);
+    else if constexpr (kParts) asm(ART_MOVE_FAST(ART_LENGTH_PARTS) "}" ART_MOVE_OPERANDS);
+    else asm(ART_MOVE_FAST(ART_LENGTH) "}" ART_MOVE_OPERANDS);
+}
+
+#define ART_MOVE_LOAD                   \
+    "mad.wide.s32 at, %4, %22, %23;\n\t" \
+    "@po ld.global.nc.f32 %9, [at];\n\t" \
+    "}"
+template <bool kExact, class Cell>
 __device__ __forceinline__ void walk_move_load(Path& W, fix rend, float unit, float& chi,
-                                               float depth, float limit, int none, int npad,
+                                               bool alive, int high, int none, int npad,
                                                const Cell* cells, float& ds, float& x, int& key,
                                                unsigned& ncross)
 {
-    asm(ART_MOVE_PTX(ART_LENGTH)
-        "mad.wide.s32 at, %4, %22, %23;\n\t"
-        "@po ld.global.nc.f32 %9, [at];\n\t"
-        "}"
-        ART_MOVE_OPERANDS, "n"((int)sizeof(Cell)), "l"(cells));
+    if constexpr (kExact)
+        asm(ART_MOVE_EXACT(ART_LENGTH) ART_MOVE_LOAD ART_MOVE_OPERANDS, "n"((int)sizeof(Cell)), "l"(cells));
+    else
+        asm(ART_MOVE_FAST(ART_LENGTH) ART_MOVE_LOAD ART_MOVE_OPERANDS, "n"((int)sizeof(Cell)), "l"(cells));
 }
 
 // Merges the deposits of lanes that hit the same cell (runs of equal cell index in lane
@@ -621,7 +634,19 @@ __device__ __forceinline__ void walk_move_load(Path& W, fix rend, float unit, fl
 // first segment of base-level rays, which all start in their source's cell: at l0 = 8 that is
 // 786,432 deposits into one cell per source, whose FP32 sum the merge keeps accurate.
 // Warp-uniform.
-__device__ __forceinline__ void merge_lanes(int& cell, float4& v)
+__device__ __forceinline__ float shifted(float v, int off) { return __shfl_down_sync(kFull, v, off); }
+__device__ __forceinline__ float4 shifted(float4 v, int off)
+{
+    return make_float4(shifted(v.x, off), shifted(v.y, off), shifted(v.z, off), shifted(v.w, off));
+}
+__device__ __forceinline__ void add_to(float& a, float b) { a += b; }
+__device__ __forceinline__ void add_to(float4& a, float4 b)
+{
+    a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+}
+
+template <class D>
+__device__ __forceinline__ void merge_lanes(int& cell, D& v)
 {
     const unsigned lane = threadIdx.x & 31u;
     const int prev = __shfl_up_sync(kFull, cell, 1);
@@ -631,13 +656,8 @@ __device__ __forceinline__ void merge_lanes(int& cell, float4& v)
     const int run_end = after ? __ffs(after) - 1 : 32;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const float ox = __shfl_down_sync(kFull, v.x, off);
-        const float oy = __shfl_down_sync(kFull, v.y, off);
-        const float oz = __shfl_down_sync(kFull, v.z, off);
-        const float ow = __shfl_down_sync(kFull, v.w, off);
-        if ((int)lane + off < run_end) {
-            v.x += ox; v.y += oy; v.z += oz; v.w += ow;
-        }
+        const D o = shifted(v, off);
+        if ((int)lane + off < run_end) add_to(v, o);
     }
     if (dup) cell = -1;
 }
@@ -654,8 +674,21 @@ __device__ __forceinline__ void merge_pair(int key_a, float4& a, int& key_b, con
         : "r"(key_a), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w), "r"(none));
 }
 
+__device__ __forceinline__ void merge_pair(int key_a, float& a, int& key_b, const float& b, int none)
+{
+    asm("{\n\t.reg .pred q;\n\tsetp.eq.s32 q, %2, %1;\n\t@q add.f32 %0, %0, %3;\n\t"
+        "@q mov.b32 %1, %4;\n\t}"
+        : "+f"(a), "+r"(key_b) : "r"(key_a), "f"(b), "r"(none));
+}
+
 // One reduction into the accumulator of cell `key`, none if it is negative.
-__device__ __forceinline__ void red_v4_if(float4* __restrict__ acc, int key, float4 v)
+__device__ __forceinline__ void red_if(float* base, int key, float v)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %1, 0;\n\t"
+                 "@q red.global.add.f32 [%0], %2;\n\t}"
+                 :: "l"(base + key), "r"(key), "f"(v) : "memory");
+}
+__device__ __forceinline__ void red_if(float4* __restrict__ acc, int key, float4 v)
 {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %1, 0;\n\t"
                  "@q red.global.add.v4.f32 [%0], {%2, %3, %4, %5};\n\t}"

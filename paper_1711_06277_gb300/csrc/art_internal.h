@@ -54,8 +54,8 @@ struct art_grid {
 
     // device buffers owned by the grid
     float* d_chi = nullptr;      // opacity per cell length (padded layout)
-    float4* d_acc = nullptr;     // per-cell accumulator (padded layout); the reverse sweep
-                                 // sums its gradient in the first npad floats
+    float4* d_acc = nullptr;     // per-cell accumulator (padded layout); traces without a force
+                                 // and the reverse sweep's gradient use the first npad floats
     art::SrcDev* d_src = nullptr;
     size_t src_cap = 0;
     art::LevelInfo* d_levels = nullptr;
@@ -109,7 +109,7 @@ struct art_grid {
 namespace art {
 int check_params(const art_params* p);
 int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto);
-int run_opacity(art_grid* g, const art_params* p, bool two_bin, float4* acc);
+int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, bool clear1);
 int trace_threads(const art_params* p);
 int cell_blocks(long long n);
 double rmax_cells(double m_ray, int level);

@@ -128,13 +128,14 @@ __global__ void k_directions(int level, unsigned long long npix, double r0, doub
 }
 
 // chi per cell length (dx) in FP32 from the density fields, in the padded layout with the
-// sentinel ring; flags bad densities and clears the accumulator (if given).
+// sentinel ring; flags bad densities and clears the accumulator (acc4 with force, acc1 without).
 __global__ void __launch_bounds__(256) k_opacity(int nx, int ny, int nz,
                                                  const float* __restrict__ nH0,
                                                  const float* __restrict__ nH, Coef sH, Coef sd,
                                                  float* __restrict__ chi,
                                                  float2* __restrict__ chi2,
-                                                 float4* __restrict__ acc,
+                                                 float4* __restrict__ acc4,
+                                                 float* __restrict__ acc1,
                                                  DevStats* __restrict__ st)
 {
     bool bad = false;
@@ -153,7 +154,8 @@ __global__ void __launch_bounds__(256) k_opacity(int nx, int ny, int nz,
             }
             chi[q] = c;
             if (chi2) chi2[q] = make_float2(c, dust);
-            if (acc) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (acc4) acc4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (acc1) acc1[q] = 0.f;
         });
     if (bad) atomicCAS(&st->error, 0, -1);
 }
@@ -195,10 +197,22 @@ __device__ __forceinline__ void lose(V& L, V& Lc, V dL)
 }
 
 // Deposits of the first segments of second groups, one slot per thread.
-__device__ __forceinline__ float4* second_slots()
+template <class D>
+__device__ __forceinline__ D* second_slots()
 {
-    __shared__ float4 s[kTraceMaxThreads];
+    __shared__ D s[kTraceMaxThreads];
     return s;
+}
+
+// What a segment adds to its cell: (sum L ds phi, sum dL n), or the first alone in traces
+// without a force, whose accumulator is a quarter as large and holds eight cells per sector
+// instead of two.
+template <bool kForce> struct DepositOf { using type = float4; };
+template <> struct DepositOf<false> { using type = float; };
+template <bool kForce>
+__device__ __forceinline__ typename DepositOf<kForce>::type* accumulator(const TraceArgs& A)
+{
+    return reinterpret_cast<typename DepositOf<kForce>::type*>(A.acc);
 }
 
 // Walks kWidth (1 or 2) rays per lane: the rays of quads [begin, end) of level l, taken 32
@@ -206,7 +220,7 @@ __device__ __forceinline__ float4* second_slots()
 // implied by their index (src0 is the first source), deeper ones are records. strided says that
 // base rays come in whole groups of 64: a lane takes two rays 32 apart instead of neighbours,
 // or two batches make a group. Warp-uniform.
-template <class Cell, bool kCut, int kWidth>
+template <class Cell, bool kCut, bool kForce, int kWidth>
 __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, int l,
                            unsigned long long* cursor, unsigned long long begin,
                            unsigned long long end, unsigned src0, bool strided)
@@ -219,7 +233,9 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
     const LevelInfo& LV = A.levels[l];
     const bool base = l == A.level0;
     BlockTally& T = block_tally();
-    float4* const s_second = second_slots();
+    using D = typename DepositOf<kForce>::type;
+    D* const s_second = second_slots<D>();
+    D* const acc = accumulator<kForce>(A);
     const unsigned items = (unsigned)end * kPerQuad;  // front ends below 2^29 quads
     const unsigned first = (unsigned)begin * kPerQuad;
     Batches batches(cursor, first, items);
@@ -311,35 +327,61 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
         auto step = [&](auto first) {
             int key[kWidth];
             V ds, x, xn = vset<V>(0.f);
+            bool alive[kWidth], exact = false;
+            int high[kWidth];
 #pragma unroll
             for (int j = 0; j < kWidth; ++j) {
-                const float depth = vget(two ? P.taun : P.tau, j);
-                [[maybe_unused]] const bool alive = !(cell[j] < 0.f) & !(depth > A.tau_max);
-                walk_move_load(W[j], rend, A.unit, cell[j], depth, A.tau_max, -1 - j,
-                               (int)A.npad, cells, vget(ds, j), vget(x, j), key[j], ncross);
-                if constexpr (two) {
+                bool e;
+                alive[j] = !(cell[j] < 0.f) & !(vget(two ? P.taun : P.tau, j) > A.tau_max);
+                high[j] = earliest(W[j], rend, alive[j], e);
+                exact |= e;
+            }
+            if (exact) {
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j)
+                    walk_move_load<true>(W[j], rend, A.unit, cell[j], alive[j], high[j], -1 - j,
+                                         (int)A.npad, cells, vget(ds, j), vget(x, j), key[j],
+                                         ncross);
+            } else {
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j)
+                    walk_move_load<false>(W[j], rend, A.unit, cell[j], alive[j], high[j], -1 - j,
+                                          (int)A.npad, cells, vget(ds, j), vget(x, j), key[j],
+                                          ncross);
+            }
+            if constexpr (two) {
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j) {
                     vget(xn, j) = celln[j] * vget(ds, j);
-                    if (alive) celln[j] = __ldg(&cells[W[j].idx].y);
+                    if (alive[j]) celln[j] = __ldg(&cells[W[j].idx].y);
                 }
             }
             // deposit and loss
             P.tau = vadd(P.tau, x);
             const V ph = phi_of(x);
-            const V G = vmul(vmul(P.L, ds), ph);
+            const V Lds = vmul(P.L, ds);
             const V dL = vmul(vmul(P.L, x), ph);
             lose(P.L, P.Lc, dL);
-            V dm = dL;  // momentum of both bins
+            [[maybe_unused]] V dm = dL;  // momentum of both bins
             if constexpr (two) {
                 P.taun = vadd(P.taun, xn);
                 const V dLn = vmul(vmul(P.Ln, xn), phi_of(xn));
                 lose(P.Ln, P.Lnc, dLn);
                 dm = vadd(dm, dLn);
             }
-            const V f0 = vmul(dm, P.n[0]), f1 = vmul(dm, P.n[1]), f2 = vmul(dm, P.n[2]);
-            float4 v[kWidth];
+            // (the parts of a reduction need registers in a row: formed one by one, they need no
+            // moves out of the pairs of two rays, 3 % of the trace)
+            D v[kWidth];
 #pragma unroll
-            for (int j = 0; j < kWidth; ++j)
-                v[j] = make_float4(vget(G, j), vget(f0, j), vget(f1, j), vget(f2, j));
+            for (int j = 0; j < kWidth; ++j) {
+                const float G = __fmul_rn(vget(Lds, j), vget(ph, j));
+                if constexpr (kForce)
+                    v[j] = make_float4(G, __fmul_rn(vget(dm, j), vget(P.n[0], j)),
+                                       __fmul_rn(vget(dm, j), vget(P.n[1], j)),
+                                       __fmul_rn(vget(dm, j), vget(P.n[2], j)));
+                else
+                    v[j] = G;
+            }
             if constexpr (decltype(first)::value) {
                 // the second of two groups of 32 waits until the walk is done
                 const bool later = kWidth == 1 && strided && (b / 32u) % 2u == 1u;
@@ -347,13 +389,13 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
                     if (!strided) merge_pair(key[0], v[0], key[1], v[1], -2);
 #pragma unroll
                 for (int j = 0; j < kWidth; ++j) merge_lanes(key[j], v[j]);
-                if (!later) red_v4_if(A.acc, key[0], v[0]);
+                if (!later) red_if(acc, key[0], v[0]);
                 second_key = kWidth == 2 ? key[kWidth - 1] : (later ? key[0] : -1);
                 s_second[threadIdx.x] = v[kWidth - 1];
             } else {
                 if constexpr (kWidth == 2) merge_pair(key[0], v[0], key[1], v[1], -2);
 #pragma unroll
-                for (int j = 0; j < kWidth; ++j) red_v4_if(A.acc, key[j], v[j]);
+                for (int j = 0; j < kWidth; ++j) red_if(acc, key[j], v[j]);
             }
         };
         // The first segments of base rays all lie in their source's cell: those of 32 rays are
@@ -369,7 +411,7 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
 #pragma unroll 1
             for (int k = 0; k < kCheckSteps; ++k) step(std::false_type{});
         }
-        if (base) red_v4_if(A.acc, second_key, s_second[threadIdx.x]);
+        if (base) red_if(acc, second_key, s_second[threadIdx.x]);
 
         // ---- ends: the children of split rays, and tallies (while the reservation of the
         // children's slots is on its way)
@@ -454,17 +496,17 @@ __device__ __forceinline__ bool front_strided(const TraceArgs& A, bool base,
     return base && A.base_quads % 16u == 0u && begin % 16u == 0u && end % 16u == 0u;
 }
 
-template <class Cell, bool kCut>
+template <class Cell, bool kCut, bool kForce>
 __device__ __forceinline__ void run_front(const TraceArgs& A, int l, int width,
                                           unsigned long long* cursor, unsigned long long begin,
                                           unsigned long long end, unsigned src0, bool strided)
 {
-    if (width == 2) walk_front<Cell, kCut, 2>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, strided);
-    else walk_front<Cell, kCut, 1>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, false);
+    if (width == 2) walk_front<Cell, kCut, kForce, 2>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, strided);
+    else walk_front<Cell, kCut, kForce, 1>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, false);
 }
 
 // Plain schedule: the whole front of level l of source s.
-template <class Cell, bool kCut>
+template <class Cell, bool kCut, bool kForce>
 __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_level(const __grid_constant__ TraceArgs A, int l, unsigned s)
 {
     block_tally_init();
@@ -472,7 +514,7 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_lev
     const unsigned long long end =
         l == A.level0 ? (unsigned long long)A.base_quads
                       : min(*((volatile unsigned long long*)&A.sched->count[l]), A.quad[l].cap);
-    run_front<Cell, kCut>(A, l, front_width(end), &A.sched->cursor[l], 0, end, s,
+    run_front<Cell, kCut, kForce>(A, l, front_width(end), &A.sched->cursor[l], 0, end, s,
                           front_strided(A, l == A.level0, 0, end));
     block_tally_flush(A.stats);
 }
@@ -529,7 +571,7 @@ __device__ __forceinline__ void next_phase(const TraceArgs& A)
 }
 
 // Persistent schedule: all sources, all levels, one cooperative launch.
-template <class Cell, bool kCut>
+template <class Cell, bool kCut, bool kForce>
 __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_persistent(const __grid_constant__ TraceArgs A)
 {
     block_tally_init();
@@ -548,24 +590,27 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_per
         __syncthreads();
         const int l = s_level;
         if (l < 0) break;
-        run_front<Cell, kCut>(A, l, s_width, &sc->cursor[l], s_begin, s_end, 0u, s_strided != 0);
+        run_front<Cell, kCut, kForce>(A, l, s_width, &sc->cursor[l], s_begin, s_end, 0u, s_strided != 0);
     }
     block_tally_flush(A.stats);
 }
 
 // Gamma, force and energy from the accumulator (padded layout) into the caller's SoA
 // outputs (nx*ny*nz layout), four cells per thread and round.
+template <class D>
 __global__ void __launch_bounds__(256) k_finalize(int nx, int ny, int nz,
-                                                  const float4* __restrict__ acc, float gscale,
+                                                  const D* __restrict__ acc, float gscale,
                                                   float fscale, float escale,
                                                   float* __restrict__ gamma,
                                                   float* __restrict__ force,
-                                                  float* __restrict__ energy)
+                                                  float* __restrict__ energy,
+                                                  const DevStats* stats, DevStats* host)
 {
+    publish_stats(stats, host);
     const unsigned ncell = (unsigned)nx * (unsigned)ny * (unsigned)nz;
     const unsigned long long step = 4ull * gridDim.x * blockDim.x;
     for (unsigned long long base = 4ull * blockIdx.x * blockDim.x + threadIdx.x; base < ncell; base += step) {
-        float4 a[4];
+        D a[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const unsigned long long i = base + (unsigned)k * blockDim.x;
@@ -575,13 +620,17 @@ __global__ void __launch_bounds__(256) k_finalize(int nx, int ny, int nz,
         for (int k = 0; k < 4; ++k) {
             const unsigned long long i = base + (unsigned)k * blockDim.x;
             if (i >= ncell) break;
-            gamma[i] = gscale * a[k].x;
-            if (force) {
+            float G;
+            if constexpr (std::is_same<D, float4>::value) {
+                G = a[k].x;
                 force[i] = fscale * a[k].y;
                 force[(size_t)ncell + i] = fscale * a[k].z;
                 force[2 * (size_t)ncell + i] = fscale * a[k].w;
+            } else {
+                G = a[k];
             }
-            if (energy) energy[i] = escale * a[k].x;
+            gamma[i] = gscale * G;
+            if (energy) energy[i] = escale * G;
         }
     }
 }

@@ -57,7 +57,12 @@ __global__ void k_reach(int nx, int ny, int nz, const float* __restrict__ chi,
     for (int k = 0; k < bound; ++k) {
         float ds, x;
         int key;
-        walk_move_load(W, dmax, unit, cell, tau, tau_max, -1, npad, chi, ds, x, key, count);
+        bool exact;
+        const int high = earliest(W, dmax, true, exact);
+        if (exact)
+            walk_move_load<true>(W, dmax, unit, cell, true, high, -1, npad, chi, ds, x, key, count);
+        else
+            walk_move_load<false>(W, dmax, unit, cell, true, high, -1, npad, chi, ds, x, key, count);
         tau += x;
         // left the grid or reached the cutoff, or used up
         if (cell < 0.f || tau > tau_max) break;
@@ -88,7 +93,7 @@ int art_estimate_work(art_grid* g, const art_params* p, double* h_work)
         hs[s] = source_record(g, u, 0.0, 0);
     }
     if ((rc = ensure_directions(g, p, le, le))) return rc;
-    if ((rc = run_opacity(g, p, false, nullptr))) return rc;
+    if ((rc = run_opacity(g, p, false, false, false))) return rc;
     SrcDev* d_src = nullptr;
     float* d_reach = nullptr;
     const size_t nray = (size_t)ns * npix;
