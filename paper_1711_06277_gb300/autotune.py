@@ -1,8 +1,9 @@
 """Autotuner for the launch knobs of the persistent trace.
 
-Knobs: rays a warp takes from the queue at a time (``chunk``), threads per block
-(``block_threads``) and the level-buffer capacity (``queue_capacity``, which sets how many
-rays one phase of the persistent schedule holds). Each candidate is timed with CUDA events on
+Knobs: threads per block (``block_threads``) and the level-buffer capacity
+(``queue_capacity``, which sets how many rays one phase of the persistent schedule holds);
+``chunk`` is still accepted in a search space, but the kernels take a warp's worth of rays at a
+time whatever its value. Each candidate is timed with CUDA events on
 a sample of the grid's sources (the cost of a trace is a sum over sources, so a sample ranks
 the candidates like the whole set). A small sample separates the candidates that differ by
 several percent but not the close ones, whose order can change with the number of sources in
@@ -26,9 +27,8 @@ from . import art as A
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "tune_cache.json")
 
 DEFAULT_SPACE = {
-    "chunk": [32, 64, 96, 128],
-    "block_threads": [128, 256, 512],
-    "queue_capacity": [16 << 20, 64 << 20, 256 << 20],  # rays per deep-level buffer (16 B each)
+    "block_threads": [320, 640],
+    "queue_capacity": [16 << 20, 64 << 20, 256 << 20],  # rays per deep-level buffer (4 B each)
 }
 
 

@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_backward_
 // Per-cell records of the reverse sweep in the padded layout, one gather per crossing, with
 // the opacity and its neutral-H part formed exactly as k_opacity forms the forward trace's
 // opacity; the sentinel ring and the end marker hold zero weights. The same pass clears the
-// gradient and flags bad densities.
+// gradient and dL and flags bad densities.
 struct CellIn {
     float a, b, w, v0, v1, v2;
 };
@@ -539,8 +539,11 @@ __global__ void __launch_bounds__(256) k_pack_cells(int nx, int ny, int nz,
                                                     const float* __restrict__ v,
                                                     Cell* __restrict__ rec,
                                                     float* __restrict__ grad,
+                                                    double* __restrict__ dL, int nsrc,
                                                     DevStats* __restrict__ st)
 {
+    if (blockIdx.x == 0)
+        for (int s = threadIdx.x; s < nsrc; s += blockDim.x) dL[s] = 0.0;
     const size_t ncell = (size_t)nx * ny * nz;
     bool bad = false;
     if (blockIdx.x == 0 && threadIdx.x == 0)
@@ -572,9 +575,9 @@ __global__ void __launch_bounds__(256) k_pack_cells(int nx, int ny, int nz,
 __global__ void __launch_bounds__(256) k_unpad_grad(int nx, int ny, int nz,
                                                     const float* __restrict__ src,
                                                     float* __restrict__ dst,
-                                                    const DevStats* stats, DevStats* host)
+                                                    DevState* state, DevStats* host)
 {
-    publish_stats(stats, host);
+    finish_state(state, host);
     const unsigned ncell = (unsigned)nx * (unsigned)ny * (unsigned)nz;
     const unsigned long long step = 4ull * gridDim.x * blockDim.x;
     for (unsigned long long base = 4ull * blockIdx.x * blockDim.x + threadIdx.x; base < ncell; base += step) {
@@ -615,26 +618,10 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     if (ns == 0) return ART_ESTATE;
     if (g->two_bin) return ART_EINVAL;  // the reverse sweep covers one-bin traces
     cudaStream_t st = g->stream;
-    if ((rc = status_of(cudaMemsetAsync(g->d_state, 0, sizeof(DevState), st)))) return rc;
+    if ((rc = begin_trace(g))) return rc;
     rc = prepare_trace(g, p, true);
     if (rc) return rc;
-    if ((size_t)ns > g->srcL_cap) {
-        if (g->d_srcL) cudaFree(g->d_srcL);
-        if (g->d_dL_scratch) cudaFree(g->d_dL_scratch);
-        g->d_srcL = nullptr;
-        g->d_dL_scratch = nullptr;
-        g->srcL_cap = 0;
-        if ((rc = status_of(cudaMalloc((void**)&g->d_srcL, sizeof(float) * ns)))) return rc;
-        if ((rc = status_of(cudaMalloc((void**)&g->d_dL_scratch, sizeof(double) * ns)))) return rc;
-        g->srcL_cap = ns;
-    }
-    g->h_srcL.resize(ns);
-    for (int s = 0; s < ns; ++s) g->h_srcL[s] = (float)g->L[s];
-    if ((rc = status_of(cudaMemcpyAsync(g->d_srcL, g->h_srcL.data(), sizeof(float) * ns,
-                                        cudaMemcpyHostToDevice, st))))
-        return rc;
     double* dL = d_dL ? d_dL : g->d_dL_scratch;
-    if ((rc = status_of(cudaMemsetAsync(dL, 0, sizeof(double) * ns, st)))) return rc;
     // the gradient is summed in the padded layout, in the (otherwise idle) accumulator
     float* grad_pad = reinterpret_cast<float*>(g->d_acc);
     const int pack_blocks = cell_blocks(g->npad);
@@ -647,17 +634,19 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
         if (!g->d_recw && (rc = status_of(cudaMalloc((void**)&g->d_recw, sizeof(CellW) * (g->npad + 1)))))
             return rc;
         k_pack_cells<CellW><<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH, sd, d_w,
-                                                         nullptr, g->d_recw, grad_pad, g->d_stats);
+                                                         nullptr, g->d_recw, grad_pad, dL, ns,
+                                                         g->d_stats);
     } else if (d_v) {
         if (!g->d_recf && (rc = status_of(cudaMalloc((void**)&g->d_recf, sizeof(CellF) * (g->npad + 1)))))
             return rc;
         k_pack_cells<CellF><<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH, sd, d_w,
-                                                         d_v, g->d_recf, grad_pad, g->d_stats);
+                                                         d_v, g->d_recf, grad_pad, dL, ns,
+                                                         g->d_stats);
     } else {
         if (!g->d_rec && (rc = status_of(cudaMalloc((void**)&g->d_rec, sizeof(float4) * (g->npad + 1)))))
             return rc;
         k_pack_cells<float4><<<pack_blocks, 256, 0, st>>>(nx, ny, nz, g->nH0, g->nH, sH, sd, d_w,
-                                                          nullptr, g->d_rec, grad_pad,
+                                                          nullptr, g->d_rec, grad_pad, dL, ns,
                                                           g->d_stats);
     }
     if ((rc = status_of(cudaGetLastError()))) return rc;
@@ -693,8 +682,9 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     cfg.numAttrs = 1;
     if ((rc = status_of(cudaLaunchKernelEx(&cfg, kern, A)))) return rc;
     k_unpad_grad<<<cell_blocks(g->ncell), 256, 0, st>>>(nx, ny, nz, grad_pad, d_dlog_nH0,
-                                                       g->d_stats, g->h_stats);
+                                                       g->d_state, g->h_stats);
     if ((rc = status_of(cudaGetLastError()))) return rc;
+    end_trace(g);
     g->last_L_in = 0.0;
     for (double v : g->L) g->last_L_in += v;
     g->last_lmax = g->lmax_glob;

@@ -278,6 +278,26 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
                                 cudaMemcpyHostToDevice, g->stream));
     }
     g->lmax_glob = lmax_glob;
+    if (adjoint) {
+        const bool grow = (size_t)ns > g->srcL_cap;
+        if (grow) {
+            dev_free(g->d_srcL);
+            dev_free(g->d_dL_scratch);
+            g->d_srcL = nullptr;
+            g->d_dL_scratch = nullptr;
+            g->srcL_cap = 0;
+            int rc = dev_alloc(&g->d_srcL, ns);
+            if (!rc) rc = dev_alloc(&g->d_dL_scratch, ns);
+            if (rc) return rc;
+            g->srcL_cap = ns;
+        }
+        if (!same || grow) {
+            g->h_srcL.resize(ns);
+            for (int s = 0; s < ns; ++s) g->h_srcL[s] = (float)g->L[s];
+            ART_TRY(cudaMemcpyAsync(g->d_srcL, g->h_srcL.data(), ns * sizeof(float),
+                                    cudaMemcpyHostToDevice, g->stream));
+        }
+    }
     if (g->two_bin && !adjoint) {
         if ((size_t)ns > g->srcLn_cap) {
             dev_free(g->d_srcLn);
@@ -356,6 +376,25 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
     g->prep_two_bin = g->two_bin;
     return ART_OK;
 }
+
+// Scheduler state and counters are clear when a trace begins: they are from the start, and the
+// last kernel of every trace leaves them so. After a call that failed on the way they are
+// cleared here (a clearing that is only captured into a graph leaves them marked as they are).
+int begin_trace(art_grid* g)
+{
+    g->state_dirty_captured = false;
+    if (!g->state_clean) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        ART_TRY(cudaMemsetAsync(g->d_state, 0, sizeof(DevState), g->stream));
+        ART_TRY(cudaStreamIsCapturing(g->stream, &cs));
+        g->state_dirty_captured = cs != cudaStreamCaptureStatusNone;
+    }
+    g->state_clean = false;
+    return ART_OK;
+}
+
+// The kernels of a trace are enqueued, the last of which clears the state.
+void end_trace(art_grid* g) { g->state_clean = !g->state_dirty_captured; }
 
 // Block size of the trace kernels: the caller's, at most (and by default) what they are built
 // for.
@@ -503,6 +542,8 @@ int art_create_grid(art_grid** out, int nx, int ny, int nz, const double box_lo[
     if (!rc) {
         g->d_sched = &g->d_state->sched;
         g->d_stats = &g->d_state->stats;
+        rc = cuda_status(cudaMemsetAsync(g->d_state, 0, sizeof(DevState), g->stream));
+        g->state_clean = rc == ART_OK;
     }
     if (!rc) rc = cuda_status(cudaMallocHost((void**)&g->h_stats, sizeof(DevStats)));
     if (!rc) rc = cuda_status(cudaMallocHost((void**)&g->h_levels, sizeof(LevelInfo) * kNL));
@@ -578,7 +619,7 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     int rc = check_params(p);
     if (rc) return rc;
     if (g->L.empty()) return ART_ESTATE;
-    ART_TRY(cudaMemsetAsync(g->d_state, 0, sizeof(DevState), g->stream));
+    if ((rc = begin_trace(g))) return rc;
     rc = prepare_trace(g, p, false);
     if (rc) return rc;
     rc = run_opacity(g, p, g->two_bin, d_force != nullptr, d_force == nullptr);
@@ -624,14 +665,15 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     const int blocks = cell_blocks(g->ncell);
     if (d_force)
         k_finalize<<<blocks, 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2], g->d_acc, gscale,
-                                                  fscale, escale, d_gamma, d_force, d_energy, g->d_stats,
+                                                  fscale, escale, d_gamma, d_force, d_energy, g->d_state,
                                                   g->h_stats);
     else
         k_finalize<<<blocks, 256, 0, g->stream>>>(g->n[0], g->n[1], g->n[2],
                                                   reinterpret_cast<const float*>(g->d_acc), gscale,
-                                                  fscale, escale, d_gamma, d_force, d_energy, g->d_stats,
+                                                  fscale, escale, d_gamma, d_force, d_energy, g->d_state,
                                                   g->h_stats);
     ART_TRY(cudaGetLastError());
+    end_trace(g);
     double Lin = 0.0;
     for (double v : g->L) Lin += v;
     g->last_L_in = Lin;

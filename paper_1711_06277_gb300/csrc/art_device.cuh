@@ -155,16 +155,6 @@ struct DevStats {
     int error;
 };
 
-// Copies the counters to pinned host memory from a kernel that runs anyway (a copy of 224 bytes
-// of its own took 2 us of the stream).
-__device__ __forceinline__ void publish_stats(const DevStats* stats, DevStats* host)
-{
-    static_assert(sizeof(DevStats) % 8 == 0 && sizeof(DevStats) / 8 <= 32, "one warp copies it");
-    if (blockIdx.x == 0 && threadIdx.x < sizeof(DevStats) / 8)
-        reinterpret_cast<unsigned long long*>(host)[threadIdx.x] =
-            reinterpret_cast<const unsigned long long*>(stats)[threadIdx.x];
-}
-
 // Scheduler state of the persistent trace and of the plain per-level launches.
 struct Sched {
     unsigned long long count[kNL];   // rays held in the level buffer (a stack, top = count)
@@ -180,6 +170,20 @@ struct DevState {
     Sched sched;
     DevStats stats;
 };
+
+// Run by the last kernel of a trace: copies the counters to pinned host memory and leaves the
+// state cleared for the next trace (a copy and a clearing of their own took 2 us each).
+__device__ __forceinline__ void finish_state(DevState* state, DevStats* host)
+{
+    static_assert(sizeof(DevStats) % 8 == 0 && sizeof(DevState) % 8 == 0, "copied in words");
+    if (blockIdx.x != 0) return;
+    const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&state->stats);
+    unsigned long long* to = reinterpret_cast<unsigned long long*>(host);
+    unsigned long long* all = reinterpret_cast<unsigned long long*>(state);
+    for (unsigned i = threadIdx.x; i < sizeof(DevStats) / 8; i += blockDim.x) to[i] = from[i];
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < sizeof(DevState) / 8; i += blockDim.x) all[i] = 0ull;
+}
 
 // Everything the trace kernels read.
 struct CellF;

@@ -60,6 +60,8 @@ struct art_grid {
     size_t src_cap = 0;
     art::LevelInfo* d_levels = nullptr;
     art::DevState* d_state = nullptr;  // scheduler and counters, cleared together
+    bool state_clean = false;          // d_state is clear once the stream gets here
+    bool state_dirty_captured = false; // this trace's clearing of it is only captured
     art::Sched* d_sched = nullptr;     // in d_state
     art::DevStats* d_stats = nullptr;  // in d_state
     art::DevStats* h_stats = nullptr;  // pinned
@@ -110,6 +112,8 @@ namespace art {
 int check_params(const art_params* p);
 int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto);
 int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, bool clear1);
+int begin_trace(art_grid* g);
+void end_trace(art_grid* g);
 int trace_threads(const art_params* p);
 int cell_blocks(long long n);
 double rmax_cells(double m_ray, int level);

@@ -604,9 +604,9 @@ __global__ void __launch_bounds__(256) k_finalize(int nx, int ny, int nz,
                                                   float* __restrict__ gamma,
                                                   float* __restrict__ force,
                                                   float* __restrict__ energy,
-                                                  const DevStats* stats, DevStats* host)
+                                                  DevState* state, DevStats* host)
 {
-    publish_stats(stats, host);
+    finish_state(state, host);
     const unsigned ncell = (unsigned)nx * (unsigned)ny * (unsigned)nz;
     const unsigned long long step = 4ull * gridDim.x * blockDim.x;
     for (unsigned long long base = 4ull * blockIdx.x * blockDim.x + threadIdx.x; base < ncell; base += step) {
