@@ -24,8 +24,8 @@
 // fronts, and every part without children) need no collapse.
 //
 // Before, each lane ran its own state machine of both passes with refills, atomic count-downs of
-// the parents and completions in between, with 21 of 32 lanes active. Against that: 9.28 ->
-// 4.73 ms on 128^3 / 16 sources with a force term, 1.69 -> 0.81 ms on an odd box with force and
+// the parents and completions in between, with 21 of 32 lanes active. Against that: 9.55 ->
+// 4.50 ms on 128^3 / 16 sources with a force term, 1.81 -> 0.69 ms on an odd box with force and
 // dust. What bounds it now is the issue of its instructions (69 % of cycles, 104 per ray and
 // step), then the latency of the record gathers (20 warps per SM hold 40 rays' worth).
 #include <cmath>

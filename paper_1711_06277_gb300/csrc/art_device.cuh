@@ -4,9 +4,9 @@
 //   fixed-point numbers with TraceArgs::fbits fraction bits, as many as the box diagonal
 //   leaves room for (51 at 512^3): a face 500 cells from the source sits within 1e-12 cells
 //   of its place, an advance is one 64-bit integer add and an order decision one compare.
-//   Against pairs of floats this took the reverse sweep, which is bound by its instructions,
-//   from 9.82 to 8.91 ms (128^3, 16 sources) and the forward trace, which is bound by its
-//   deposits, from 83.6 to 81.9 ms (256^3, 64 sources).
+//   Against pairs of floats this alone took a reverse sweep bound by its instructions from
+//   9.82 to 8.91 ms (128^3, 16 sources) and a forward trace bound by one deposit per crossing
+//   from 83.6 to 81.9 ms (256^3, 64 sources).
 // * Double-float ("df") arithmetic (an unevaluated sum hi + lo of two floats, ~44 significant
 //   bits) places the start of a ray: FP64 throughput on this part is a small fraction of FP32.
 // * The ray-walk state and one crossing step of Sec. 2.1 (Kim et al. 2017): next face
@@ -495,26 +495,26 @@ __device__ __forceinline__ V phi_dphi(V x, V& dphi)
 
 // The geometric part of a step: the segment from tc to the next face or to the end radius
 // rend (split or cutoff, kNoEnd if at none), and the advance of the walk to its end; at rend
-// the next cell is the end marker npad. ds is the length (cell units; unit = 2^-fbits) and key
-// the cell of the segment, 0 and `none` where there is nothing to deposit: the length is not
-// positive or the ray has ended (chi < 0, or depth > limit). Deposits are counted in ncross;
-// x is chi ds, 0 with ds (also where chi is infinite). walk_move_load also replaces chi by the opacity at the start of the next
-// cell's record, unless the ray has ended.
+// the next cell is the end marker npad. ds is the length (cell units; unit = 2^-fbits), x is
+// chi ds and key the cell of the segment; ds and x are 0 and key is `none` where there is
+// nothing to deposit: the ray is no longer alive, or the length is not positive. Deposits are
+// counted in ncross. walk_move_load also replaces chi by the opacity at the start of the next
+// cell's record, unless the ray is no longer alive.
 //
 // The earliest of the three faces and the end radius is decided on the high words (2^-19
-// cells at 512^3): different high words order the distances exactly. Equal ones (exact ties,
-// near ties, a face at the end radius), and segments too short to show in the high words,
-// take the exact 64-bit comparison on the side path, where axes that cross within 2^-40 of
-// the distance of the earliest one step together (a diagonal step). Two distances within that
-// tolerance can still have different high words when they straddle a boundary; the walk then
-// crosses the two faces in two steps with a segment far below the 1e-5-cell near-tie
+// cells at 512^3): different high words order the distances exactly. Where two are equal
+// (exact ties, near ties, a face at the end radius), or the segment is too short to show in
+// them (earliest() says both), the exact 64-bit comparison decides, and axes that cross within
+// 2^-40 of the distance of the earliest one step together (a diagonal step). Two distances
+// within that tolerance can still have different high words when they straddle a boundary; the
+// walk then crosses the two faces in two steps with a segment far below the 1e-5-cell near-tie
 // threshold between them, a ray the oracle flags as near-tie.
 //
 // Written in PTX because the predicates of the choice then also predicate the advance: from
-// C++ the compiler made branches of it (15 per ray and step instead of the one for ties,
-// 97.0 against 65.7 ms on 256^3 / 64 sources). The side path finishes the move by itself:
-// joined before the advance, with the predicates of both paths, every step paid 18 more
-// instructions (14.3 against 12.2 ms on 256^3 / 16 sources).
+// C++ the compiler made branches of it (15 per ray and step instead of one for both rays of a
+// lane, 97.0 against 65.7 ms on 256^3 / 64 sources with four rays per lane). Each form carries
+// its own advance: with the exact choice joined before a common advance, by the predicates of
+// both, every step paid 18 more instructions (14.3 against 12.2 ms on 256^3 / 16 sources).
 //   operands: 0-2 t, 3 tc, 4 idx, 5 ncross, 6 ds, 7 key, 8 x, 9 chi, 10-12 d, 13-15 ss,
 //   16 rend, 17 unit, 18 none, 19 npad, 20 alive, 21 earliest high word
 #define ART_LENGTH "cvt.rn.f32.s64 fl, mv;\n\t"
@@ -704,7 +704,8 @@ __device__ __forceinline__ void red_if(float4* __restrict__ acc, int key, float4
 // helpers shared by the forward and backward kernels
 // ---------------------------------------------------------------------------------------
 // Threads per block of the trace kernels at most: one block of 20 warps per SM (65536 / 640 =
-// 102 registers a thread: two walks), so that a grid barrier has 152 arrivals and not 760.
+// 102 registers a thread: two walks), so that a grid barrier has 152 arrivals and not 760. 24
+// warps (80 registers) gain 5 % at 256^3 and lose 2 % at 512^3 and 3 % in the sweep.
 constexpr int kTraceMaxThreads = 640;
 constexpr int kTraceMinBlocks = 1;
 // Steps between checks whether a warp still has rays.
