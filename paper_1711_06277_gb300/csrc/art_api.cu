@@ -92,6 +92,12 @@ void dev_free(void* p)
     if (p) cudaFree(p);
 }
 
+void free_retired(art_grid* g)
+{
+    for (void* p : g->retired) dev_free(p);
+    g->retired.clear();
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------------------
@@ -157,7 +163,8 @@ SrcDev source_record(const art_grid* g, const double u[3], double base_L, int lm
     d.hi = make_float4(h[0], h[1], h[2], (float)base_L);
     d.lo = make_float4(lo[0], lo[1], lo[2], lmf);
     d.xy = make_longlong2(to_fix(u[0], g->fbits), to_fix(u[1], g->fbits));
-    d.z_ = make_longlong2(to_fix(u[2], g->fbits), 0);
+    d.z_ = make_longlong2(to_fix(u[2], g->fbits),
+                          pad_index((long long)u[0], (long long)u[1], (long long)u[2], g->n[0], g->n[1]));
     return d;
 }
 
@@ -256,13 +263,31 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         const double lb = adjoint ? 1.0 / (double)npix0 : g->L[s] / (double)npix0;
         hs[s] = source_record(g, u, lb, lm);
     }
-    if ((size_t)ns > g->src_cap) {
-        dev_free(g->d_src);
+    // The sums of first segments are kept for a fixed order of addition where base rays come in
+    // whole groups of 64 of one source (from l0 = 2; every phase of the base front then ends on such
+    // a group unless it is 16 quads or less, see below) and up to l0 = 6, 1536 sums per source: the
+    // one warp that adds them takes longer beyond, and they are added as they come. They share
+    // the allocation of the source table (freeing one more block costs a grid's end 0.1 ms). A block
+    // that has become too small for them alone may be in use by a captured trace and is kept.
+    const size_t groups = !adjoint && l0 >= 2 && l0 <= 6 ? (size_t)ns * (npix0 / 32) : 0;
+    if ((size_t)ns > g->src_cap || groups > g->first_cap) {
+        const size_t cap = std::max((size_t)ns, g->src_cap), gcap = std::max(groups, g->first_cap);
+        if ((size_t)ns > g->src_cap) {
+            dev_free(g->d_src);
+            free_retired(g);
+        } else {
+            g->retired.push_back(g->d_src);
+        }
         g->d_src = nullptr;
-        g->src_cap = 0;
-        int rc = dev_alloc(&g->d_src, ns);
+        g->src_cap = g->first_cap = 0;
+        g->prep_valid = false;
+        char* block = nullptr;
+        int rc = dev_alloc(&block, cap * sizeof(SrcDev) + gcap * 8 * sizeof(float4));
         if (rc) return rc;
-        g->src_cap = ns;
+        g->d_src = reinterpret_cast<SrcDev*>(block);
+        g->d_first = reinterpret_cast<float*>(g->d_src + cap);
+        g->src_cap = cap;
+        g->first_cap = gcap;
     }
     // uploads only when the sources or the parameters that shape the tables changed, so an
     // unchanged trace enqueues no host-to-device copy (and can be captured in a CUDA graph)
@@ -365,6 +390,7 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         }
         if (rc) return rc;
     }
+    g->first_ordered = groups > 0 && (plain || l0 == lmax_glob || g->quad[l0 + 1].cap / 4 > 16);
     g->prep_valid = true;
     g->prep_version = g->src_version;
     g->prep_level0 = l0;
@@ -445,6 +471,7 @@ TraceArgs make_args(art_grid* g, const art_params* p)
         A.quad[l] = g->quad[l];
         if (l > g->lmax_glob) A.adj[l].cap = A.quad[l].cap = 0;
     }
+    if (g->first_ordered) A.first = g->d_first;
     A.base_quads = 3u << (2 * p->level0);
     A.nsrc = (unsigned)g->L.size();
     A.npad = (unsigned)g->npad;
@@ -639,6 +666,11 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
             for (int l = l0; l <= g->src_lmax[s]; ++l)
                 kern<<<grid, threads, 0, g->stream>>>(A, l, (unsigned)s);
         }
+        if (A.first) {
+            const int blocks = std::min((ns + 7) / 8, 16 * g->sms);
+            if (d_force) k_add_first<true><<<blocks, 256, 0, g->stream>>>(A);
+            else k_add_first<false><<<blocks, 256, 0, g->stream>>>(A);
+        }
         ART_TRY(cudaGetLastError());
     } else {
         int per_sm = 0;
@@ -702,6 +734,7 @@ void art_destroy_grid(art_grid* g)
     dev_free(g->d_chi);
     dev_free(g->d_acc);
     dev_free(g->d_src);
+    free_retired(g);
     dev_free(g->d_levels);
     dev_free(g->d_state);
     dev_free(g->d_srcL);

@@ -113,8 +113,11 @@ struct SrcDev {
     float4 hi;  // u_x, u_y, u_z (hi parts), L / N_ray(l0)
     float4 lo;  // u_x, u_y, u_z (lo parts), l_max (int bits)
     longlong2 xy;  // u_x, u_y (fixed-point)
-    longlong2 z_;  // u_z (fixed-point), unused
+    longlong2 z_;  // u_z (fixed-point), the cell that the source lies in, on a face the upper one
+                   // (index in the padded layout)
 };
+
+__device__ __forceinline__ int source_cell(const SrcDev& d) { return (int)__ldg(&d.z_).y; }
 
 // Per level constants of a trace.
 struct LevelInfo {
@@ -204,6 +207,8 @@ struct TraceArgs {
     const LevelInfo* levels;
     AdjBuf adj[kNL];         // adjoint fronts
     QuadBuf quad[kNL];       // forward fronts (levels beyond l0)
+    float* first;            // sums of the base rays' first segments, 8 per group of 32 rays
+                             // (see keep_first); null where they are added as they come
     unsigned base_quads;     // quads of level l0 per source (3 * 4^l0)
     unsigned nsrc;
     unsigned npad;           // cells of the padded layout; cell npad is the end marker
@@ -643,10 +648,41 @@ __device__ __forceinline__ float4 shifted(float4 v, int off)
 {
     return make_float4(shifted(v.x, off), shifted(v.y, off), shifted(v.z, off), shifted(v.w, off));
 }
+__device__ __forceinline__ float from_lane(float v, int lane) { return __shfl_sync(kFull, v, lane); }
+__device__ __forceinline__ float4 from_lane(float4 v, int lane)
+{
+    return make_float4(from_lane(v.x, lane), from_lane(v.y, lane), from_lane(v.z, lane),
+                       from_lane(v.w, lane));
+}
+__device__ __forceinline__ float across(float v, int mask) { return __shfl_xor_sync(kFull, v, mask); }
+__device__ __forceinline__ float4 across(float4 v, int mask)
+{
+    return make_float4(across(v.x, mask), across(v.y, mask), across(v.z, mask), across(v.w, mask));
+}
+__device__ __forceinline__ bool is_zero(float v) { return v == 0.f; }
+__device__ __forceinline__ bool is_zero(float4 v)
+{
+    return v.x == 0.f && v.y == 0.f && v.z == 0.f && v.w == 0.f;
+}
 __device__ __forceinline__ void add_to(float& a, float b) { a += b; }
 __device__ __forceinline__ void add_to(float4& a, float4 b)
 {
     a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+}
+
+// sum + rest += b, the rounding error of sum collected in rest
+__device__ __forceinline__ void add_pair(float& sum, float& rest, float b)
+{
+    const df r = df_two_sum(sum, b);
+    sum = r.hi;
+    rest += r.lo;
+}
+__device__ __forceinline__ void add_pair(float4& sum, float4& rest, float4 b)
+{
+    add_pair(sum.x, rest.x, b.x);
+    add_pair(sum.y, rest.y, b.y);
+    add_pair(sum.z, rest.z, b.z);
+    add_pair(sum.w, rest.w, b.w);
 }
 
 template <class D>
@@ -779,12 +815,15 @@ __device__ __forceinline__ void df_accumulate(df& s, float v)
 // address had taken microseconds.
 __device__ __forceinline__ unsigned warps_in_grid() { return gridDim.x * (blockDim.x >> 5); }
 
+// Place of this warp in the grid: the warps of an SM are far apart.
+__device__ __forceinline__ unsigned warp_in_grid() { return (threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
+
 struct Batches {
     unsigned long long* cursor;
     unsigned next, items;
     bool first;
     __device__ __forceinline__ Batches(unsigned long long* c, unsigned begin, unsigned n)
-        : cursor(c), next(begin + 32u * ((threadIdx.x >> 5) * gridDim.x + blockIdx.x)), items(n),
+        : cursor(c), next(begin + 32u * warp_in_grid()), items(n),
           first(true) {}
     // First item of the warp's next batch, or a value >= items when there is none. Warp-uniform.
     __device__ __forceinline__ unsigned take(unsigned begin)

@@ -75,6 +75,12 @@ struct art_grid {
     art::QuadBuf quad[art::kNL] = {};
     unsigned long long quad_cap[art::kNL] = {};      // allocated quads per level
 
+    // sums of the base rays' first segments, kept for a fixed order of addition
+    float* d_first = nullptr;        // behind the source table, in its allocation
+    size_t first_cap = 0;            // groups of 32 rays that it holds
+    bool first_ordered = false;      // the prepared trace keeps them
+    std::vector<void*> retired;      // former blocks of the table and the sums (see prepare_trace)
+
     // adjoint fronts
     art::AdjBuf adj[art::kNL] = {};
     unsigned long long adj_cap[art::kNL] = {};       // allocated quads per level

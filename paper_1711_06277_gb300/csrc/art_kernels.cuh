@@ -196,14 +196,6 @@ __device__ __forceinline__ void lose(V& L, V& Lc, V dL)
     L = Lnew;
 }
 
-// Deposits of the first segments of second groups, one slot per thread.
-template <class D>
-__device__ __forceinline__ D* second_slots()
-{
-    __shared__ D s[kTraceMaxThreads];
-    return s;
-}
-
 // What a segment adds to its cell: (sum L ds phi, sum dL n), or the first alone in traces
 // without a force, whose accumulator is a quarter as large and holds eight cells per sector
 // instead of two.
@@ -215,11 +207,111 @@ __device__ __forceinline__ typename DepositOf<kForce>::type* accumulator(const T
     return reinterpret_cast<typename DepositOf<kForce>::type*>(A.acc);
 }
 
+// The first segments of base rays lie in their source's cell, or in the up to eight cells around
+// it where it sits on a face, an edge or a corner. The sum of each group of 32 rays and cell is
+// kept until the base front is done, and one warp per source then adds them up, so that the rate
+// next to a single source, the largest of the field, and with it the substep size are the same in
+// every run; added as the warps got to them, 96 sums at l0 = 4 differed by 1e-7 to 6e-7 from run to
+// run. They are added in two floats: their order in one float leaves up to 8e-7 (equal sums of
+// symmetric directions in a row are rounded alike). The six sums of l0 = 2 are added in one, those
+// of even number first, which is what the former walk (64 base rays per warp, the first half of
+// each first) came to in every run.
+template <class D>
+struct FirstSegments {  // of the rays of a block on their way
+    D value[2][kTraceMaxThreads];
+    int key[2][kTraceMaxThreads];
+};
+template <class D>
+__device__ __forceinline__ FirstSegments<D>& first_segments()
+{
+    __shared__ FirstSegments<D> f;
+    return f;
+}
+template <class D>
+__device__ __forceinline__ D* first_sums(const TraceArgs& A)
+{
+    return reinterpret_cast<D*>(A.first);
+}
+
+// Keeps the sums of one group at `to`, one per cell (bit a of a cell's number says that it is the
+// lower of the two on axis a). A lane's ray lies `below` cells of the padded layout below the
+// source's cell, if it has a segment at all (some). Warp-uniform.
+template <class D>
+__device__ __forceinline__ void keep_first(D* to, int sy, int sz, int below, bool some, D v)
+{
+    const unsigned lane = threadIdx.x & 31u;
+    int o = 0;
+    if (below >= sz) { o |= 4; below -= sz; }
+    if (below >= sy) { o |= 2; below -= sy; }
+    o |= below;
+    D mine{};  // lane o keeps the sum of cell o
+    unsigned left = __ballot_sync(kFull, some);
+    while (left) {
+        const int cell = __shfl_sync(kFull, o, __ffs(left) - 1);
+        const bool in = some && o == cell;
+        D sum = in ? v : D{};
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) add_to(sum, shifted(sum, off));  // lane 0's is whole
+        sum = from_lane(sum, 0);
+        if ((int)lane == cell) mine = sum;
+        left &= ~__ballot_sync(kFull, in);
+    }
+    if (lane < 8u) __stcg(to + lane, mine);
+}
+
+// The sum of a source's kept sums for cell `lane % 8`, in every lane; `from` are its first group's.
+// Four groups side by side. Warp-uniform.
+template <class D>
+__device__ __forceinline__ D sum_first(const D* from, unsigned groups)
+{
+    const unsigned lane = threadIdx.x & 31u;
+    from += lane % 8u;
+    D sum{}, rest{};
+    if (groups <= 6u) {
+        for (unsigned t = 0; t < groups; ++t) add_to(sum, __ldcg(from + 8u * (t < 3u ? 2u * t : 2u * t - 5u)));
+        return sum;
+    }
+    for (unsigned t = lane / 8u; t < groups; t += 32u) {
+        D v[8];  // eight loads in flight
+#pragma unroll
+        for (unsigned k = 0; k < 8u; ++k) v[k] = t + 4u * k < groups ? __ldcg(from + 8u * (t + 4u * k)) : D{};
+#pragma unroll
+        for (unsigned k = 0; k < 8u; ++k) add_pair(sum, rest, v[k]);
+    }
+#pragma unroll
+    for (int off = 8; off < 32; off <<= 1) {
+        const D s2 = across(sum, off), r2 = across(rest, off);
+        add_pair(sum, rest, s2);
+        add_to(rest, r2);
+    }
+    add_to(sum, rest);
+    return sum;
+}
+
+// Adds the kept sums of all sources to the accumulator, a warp per source, the warps with the last
+// batches, if any, of a front first. In the persistent schedule every warp gets here after its share
+// of the front that follows the base, while others still walk; as a function apart, and called
+// after the walk, it costs nothing measurable (in line or before the walk 2 to 3 %, by the walk's
+// registers; as a kernel of its own 7 us; in the last kernel, by the blocks of the sources' cells, 7 us
+// with one source and 46 us with 64).
+template <class D>
+__device__ __noinline__ void add_first(const TraceArgs& A, D* acc)
+{
+    const unsigned o = threadIdx.x % 8u;  // the lane's cell
+    const unsigned groups = A.base_quads / 8u;
+    for (unsigned s = warps_in_grid() - 1u - warp_in_grid(); s < A.nsrc; s += warps_in_grid()) {
+        const D sum = sum_first(first_sums<D>(A) + 8ull * groups * s, groups);
+        if (threadIdx.x % 32u < 8u && !is_zero(sum))
+            red_if(acc, source_cell(A.src[s]) - (int)(o & 1u) -
+                            (A.nx + 2) * ((int)(o >> 1 & 1u) + (A.ny + 2) * (int)(o >> 2)), sum);
+    }
+}
+
 // Walks kWidth (1 or 2) rays per lane: the rays of quads [begin, end) of level l, taken 32
 // lanes at a time from `cursor`, which counts items of kWidth rays. Base-level quads are
 // implied by their index (src0 is the first source), deeper ones are records. strided says that
-// base rays come in whole groups of 64: a lane takes two rays 32 apart instead of neighbours,
-// or two batches make a group. Warp-uniform.
+// base rays come in whole groups of 64: where a lane takes two, they are 32 apart instead of
+// neighbours, so that a group of 32 is the same at both widths. Warp-uniform.
 template <class Cell, bool kCut, bool kForce, int kWidth>
 __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, int l,
                            unsigned long long* cursor, unsigned long long begin,
@@ -234,8 +326,8 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
     const bool base = l == A.level0;
     BlockTally& T = block_tally();
     using D = typename DepositOf<kForce>::type;
-    D* const s_second = second_slots<D>();
     D* const acc = accumulator<kForce>(A);
+    FirstSegments<D>& F = first_segments<D>();
     const unsigned items = (unsigned)end * kPerQuad;  // front ends below 2^29 quads
     const unsigned first = (unsigned)begin * kPerQuad;
     Batches batches(cursor, first, items);
@@ -323,7 +415,6 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
         // ring where it left the grid, the end marker where it reached its end radius) or has
         // passed tau_max, and does nothing more. In two-bin traces the packet is used up once
         // its dust-only depth (never the larger one) passes tau_max.
-        int second_key = -1;
         auto step = [&](auto first) {
             int key[kWidth];
             V ds, x, xn = vset<V>(0.f);
@@ -383,24 +474,17 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
                     v[j] = G;
             }
             if constexpr (decltype(first)::value) {
-                // the second of two groups of 32 waits until the walk is done
-                const bool later = kWidth == 1 && strided && (b / 32u) % 2u == 1u;
-                if constexpr (kWidth == 2)
-                    if (!strided) merge_pair(key[0], v[0], key[1], v[1], -2);
 #pragma unroll
-                for (int j = 0; j < kWidth; ++j) merge_lanes(key[j], v[j]);
-                if (!later) red_if(acc, key[0], v[0]);
-                second_key = kWidth == 2 ? key[kWidth - 1] : (later ? key[0] : -1);
-                s_second[threadIdx.x] = v[kWidth - 1];
+                for (int j = 0; j < kWidth; ++j) {
+                    F.value[j][threadIdx.x] = v[j];
+                    F.key[j][threadIdx.x] = key[j];
+                }
             } else {
                 if constexpr (kWidth == 2) merge_pair(key[0], v[0], key[1], v[1], -2);
 #pragma unroll
                 for (int j = 0; j < kWidth; ++j) red_if(acc, key[j], v[j]);
             }
         };
-        // The first segments of base rays all lie in their source's cell: those of 32 rays are
-        // deposited as one sum, in every second such group when the walk is done, so that the
-        // additions to that one cell are spread over the phase.
         if (base) step(std::true_type{});
         for (;;) {
             bool any = false;
@@ -411,7 +495,32 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
 #pragma unroll 1
             for (int k = 0; k < kCheckSteps; ++k) step(std::false_type{});
         }
-        if (base) red_if(acc, second_key, s_second[threadIdx.x]);
+
+        // ---- first segments of base rays (here, where the walk's registers are free)
+        if (base) {
+            D v[kWidth];
+            int key[kWidth];
+#pragma unroll
+            for (int j = 0; j < kWidth; ++j) {
+                v[j] = F.value[j][threadIdx.x];
+                key[j] = F.key[j][threadIdx.x];
+            }
+            if (strided && A.first) {
+                const int at = source_cell(A.src[s]);
+                D* const to = first_sums<D>(A) + 8u * (src0 * (A.base_quads / 8u) + kWidth * b / 32u);
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j)
+                    keep_first(to + 8 * j, A.nx + 2, (A.nx + 2) * (A.ny + 2), at - key[j], key[j] >= 0, v[j]);
+            } else {
+                if constexpr (kWidth == 2)
+                    if (!strided) merge_pair(key[0], v[0], key[1], v[1], -2);
+#pragma unroll
+                for (int j = 0; j < kWidth; ++j) {
+                    merge_lanes(key[j], v[j]);
+                    red_if(acc, key[j], v[j]);
+                }
+            }
+        }
 
         // ---- ends: the children of split rays, and tallies (while the reservation of the
         // children's slots is on its way)
@@ -502,7 +611,7 @@ __device__ __forceinline__ void run_front(const TraceArgs& A, int l, int width,
                                           unsigned long long end, unsigned src0, bool strided)
 {
     if (width == 2) walk_front<Cell, kCut, kForce, 2>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, strided);
-    else walk_front<Cell, kCut, kForce, 1>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, false);
+    else walk_front<Cell, kCut, kForce, 1>(A, cells_of<Cell>(A), l, cursor, begin, end, src0, strided);
 }
 
 // Plain schedule: the whole front of level l of source s.
@@ -517,6 +626,13 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_lev
     run_front<Cell, kCut, kForce>(A, l, front_width(end), &A.sched->cursor[l], 0, end, s,
                           front_strided(A, l == A.level0, 0, end));
     block_tally_flush(A.stats);
+}
+
+// The kept sums of first segments in the plain schedule.
+template <bool kForce>
+__global__ void __launch_bounds__(256) k_add_first(const __grid_constant__ TraceArgs A)
+{
+    add_first(A, accumulator<kForce>(A));
 }
 
 // Resets the per-level counters of the plain schedule before the next source, whose launches
@@ -576,11 +692,13 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_per
 {
     block_tally_init();
     Sched* sc = A.sched;
-    __shared__ int s_level, s_width, s_strided;
+    __shared__ int s_level, s_width, s_strided, s_base_done;
     __shared__ unsigned long long s_begin, s_end;
+    if (threadIdx.x == 0) s_level = -1;
     for (;;) {
         if (!grid_barrier(sc, A.stats, A.wait_ns, [&] { next_phase(A); })) break;
         if (threadIdx.x == 0) {
+            s_base_done = s_level == A.level0 && s_begin == 0;  // the phase before
             s_level = __ldcg(&sc->done) ? -1 : __ldcg(&sc->phase_level);
             s_width = __ldcg(&sc->phase_width);
             s_strided = __ldcg(&sc->phase_strided);
@@ -589,8 +707,9 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace_per
         }
         __syncthreads();
         const int l = s_level;
+        if (l >= 0) run_front<Cell, kCut, kForce>(A, l, s_width, &sc->cursor[l], s_begin, s_end, 0u, s_strided != 0);
+        if (s_base_done && A.first) add_first(A, accumulator<kForce>(A));
         if (l < 0) break;
-        run_front<Cell, kCut, kForce>(A, l, s_width, &sc->cursor[l], s_begin, s_end, 0u, s_strided != 0);
     }
     block_tally_flush(A.stats);
 }
