@@ -574,20 +574,20 @@ __device__ void walk_front(const TraceArgs& A, const Cell* __restrict__ cells, i
         if (nchild) {
             const QuadBuf& C = A.quad[l + 1];
             slot = __shfl_sync(kFull, slot, 0);
-            if (slot + nchild > C.cap) {
-                atomicCAS(&A.stats->error, 0, -3);  // ART_EQUEUE_OVERFLOW
-            } else if (mine) {
+            // every slot below the capacity is written, whatever a front leaves out: the next
+            // launch of the plain schedule reads them all
+            const unsigned cap = (unsigned)C.cap, room = slot < cap ? min(nchild, cap - slot) : 0u;
+            if (room < nchild) atomicCAS(&A.stats->error, 0, -3);  // ART_EQUEUE_OVERFLOW
 #pragma unroll
-                for (int j = 0; j < kWidth; ++j) {
-                    if (child[j]) {
-                        __stcg(C.rec + slot + at[j],
-                               make_uint4(s, 4u * (pix + j * apart),
-                                          __float_as_uint(0.25f * vget(P.L, j)),
-                                          __float_as_uint(vget(P.tau, j))));
-                        if constexpr (two)
-                            __stcg(C.recn + slot + at[j],
-                                   make_float2(0.25f * vget(P.Ln, j), vget(P.taun, j)));
-                    }
+            for (int j = 0; j < kWidth; ++j) {
+                if (child[j] && at[j] < room) {
+                    __stcg(C.rec + slot + at[j],
+                           make_uint4(s, 4u * (pix + j * apart),
+                                      __float_as_uint(0.25f * vget(P.L, j)),
+                                      __float_as_uint(vget(P.tau, j))));
+                    if constexpr (two)
+                        __stcg(C.recn + slot + at[j],
+                               make_float2(0.25f * vget(P.Ln, j), vget(P.taun, j)));
                 }
             }
         }
