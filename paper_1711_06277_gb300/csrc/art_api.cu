@@ -433,15 +433,16 @@ int trace_threads(const art_params* p)
 int cell_blocks(long long n) { return (int)((n + 1023) / 1024); }
 
 // Opacity per cell length (padded layout) into d_chi, and the two-bin pairs into d_chi2; clears
-// the accumulator of a trace with a force (clear4) or without (clear1).
-int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, bool clear1)
+// the accumulator of a trace with a force (clear4) or without (clear1). Bad densities are flagged in
+// st, if given: a pass outside a trace must leave the trace state as it is.
+int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, bool clear1, DevStats* st)
 {
     const Coef sH = coef_of(p->sigma_H * g->dx);
     const Coef sd = coef_of(g->nH ? p->sigma_d * g->dx : 0.0);
     k_opacity<<<cell_blocks(g->npad), 256, 0, g->stream>>>(
         g->n[0], g->n[1], g->n[2], g->nH0, g->nH, sH, sd, g->d_chi,
         two_bin ? g->d_chi2 : nullptr, clear4 ? g->d_acc : nullptr,
-        clear1 ? reinterpret_cast<float*>(g->d_acc) : nullptr, g->d_stats);
+        clear1 ? reinterpret_cast<float*>(g->d_acc) : nullptr, st);
     ART_TRY(cudaGetLastError());
     return ART_OK;
 }
@@ -649,7 +650,7 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     if ((rc = begin_trace(g))) return rc;
     rc = prepare_trace(g, p, false);
     if (rc) return rc;
-    rc = run_opacity(g, p, g->two_bin, d_force != nullptr, d_force == nullptr);
+    rc = run_opacity(g, p, g->two_bin, d_force != nullptr, d_force == nullptr, g->d_stats);
     if (rc) return rc;
     const int ns = (int)g->L.size();
     const int l0 = p->level0;

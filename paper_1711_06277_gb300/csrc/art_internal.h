@@ -117,7 +117,7 @@ struct art_grid {
 namespace art {
 int check_params(const art_params* p);
 int ensure_directions(art_grid* g, const art_params* p, int lfrom, int lto);
-int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, bool clear1);
+int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, bool clear1, DevStats* st);
 int begin_trace(art_grid* g);
 void end_trace(art_grid* g);
 int trace_threads(const art_params* p);

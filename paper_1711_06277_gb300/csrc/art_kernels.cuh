@@ -128,7 +128,8 @@ __global__ void k_directions(int level, unsigned long long npix, double r0, doub
 }
 
 // chi per cell length (dx) in FP32 from the density fields, in the padded layout with the
-// sentinel ring; flags bad densities and clears the accumulator (acc4 with force, acc1 without).
+// sentinel ring; flags bad densities in st (if given) and clears the accumulator (acc4 with force,
+// acc1 without).
 __global__ void __launch_bounds__(256) k_opacity(int nx, int ny, int nz,
                                                  const float* __restrict__ nH0,
                                                  const float* __restrict__ nH, Coef sH, Coef sd,
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(256) k_opacity(int nx, int ny, int nz,
             if (acc4) acc4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (acc1) acc1[q] = 0.f;
         });
-    if (bad) atomicCAS(&st->error, 0, -1);
+    if (bad && st) atomicCAS(&st->error, 0, -1);
 }
 
 // The per-cell records a trace gathers: opacities (one bin) or opacity pairs (two bins).

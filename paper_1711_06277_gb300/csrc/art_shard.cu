@@ -93,7 +93,7 @@ int art_estimate_work(art_grid* g, const art_params* p, double* h_work)
         hs[s] = source_record(g, u, 0.0, 0);
     }
     if ((rc = ensure_directions(g, p, le, le))) return rc;
-    if ((rc = run_opacity(g, p, false, false, false))) return rc;
+    if ((rc = run_opacity(g, p, false, false, false, nullptr))) return rc;
     SrcDev* d_src = nullptr;
     float* d_reach = nullptr;
     const size_t nray = (size_t)ns * npix;
