@@ -621,7 +621,7 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
     if ((rc = begin_trace(g))) return rc;
     rc = prepare_trace(g, p, true);
     if (rc) return rc;
-    double* dL = d_dL ? d_dL : g->d_dL_scratch;
+    double* dL = d_dL ? d_dL : g->tables[1].dL;
     // the gradient is summed in the padded layout, in the (otherwise idle) accumulator
     float* grad_pad = reinterpret_cast<float*>(g->d_acc);
     const int pack_blocks = cell_blocks(g->npad);
@@ -650,13 +650,12 @@ extern "C" int art_trace_backward(art_grid* g, const art_params* p, const float*
                                                           g->d_stats);
     }
     if ((rc = status_of(cudaGetLastError()))) return rc;
-    TraceArgs A = make_args(g, p);
+    TraceArgs A = make_args(g, p, true);
     A.rec = g->d_rec;
     A.recf = d_v ? g->d_recf : nullptr;
     A.recw = light ? g->d_recw : nullptr;
     A.grad = grad_pad;
     A.dL = dL;
-    A.srcL = g->d_srcL;
     const double dV = g->dx * g->dx * g->dx;
     A.gscale = (float)(p->sigma_H * g->dx / dV);
     A.fscale = (float)(1.0 / dV);

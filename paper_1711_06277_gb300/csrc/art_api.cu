@@ -241,6 +241,54 @@ static int ensure_quads(art_grid* g, int l, unsigned long long need, bool two_bi
     return ART_OK;
 }
 
+// Words of a table that travel as a kernel's parameter.
+template <int kWords>
+struct Words {
+    uint4 w[kWords];
+};
+template <int kWords>
+__global__ void k_store(const __grid_constant__ Words<kWords> from, uint4* __restrict__ to, unsigned n)
+{
+    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) to[i] = from.w[i];
+}
+template <int kWords>
+static cudaError_t store_words(const unsigned char* from, size_t bytes, uint4* to, cudaStream_t st)
+{
+    Words<kWords> w;
+    std::memcpy(w.w, from, bytes);
+    k_store<kWords><<<1, 64, 0, st>>>(w, to, (unsigned)(bytes / sizeof(uint4)));
+    return cudaGetLastError();
+}
+
+// Brings a table of the device up to date. An unchanged one enqueues nothing (such a trace can be
+// captured in a graph without it). The bytes travel as kernel parameters, which the launch
+// takes over: a staging buffer may be written again while an earlier copy from it still waits in
+// the stream, and a graph would read it at every replay.
+static int send_table(art_grid* g, HostTable& t, const void* data, size_t bytes, void* to)
+{
+    const unsigned char* from = static_cast<const unsigned char*>(data);
+    if (t.known && t.sent.size() == bytes && std::memcmp(t.sent.data(), from, bytes) == 0) return ART_OK;
+    t.known = false;
+    constexpr int kSmall = 64, kLarge = 1024;  // words of 16 bytes
+    for (size_t at = 0; at < bytes;) {
+        uint4* const dst = reinterpret_cast<uint4*>(static_cast<unsigned char*>(to) + at);
+        const bool small = bytes - at <= kSmall * sizeof(uint4);
+        const size_t n = std::min(bytes - at, kLarge * sizeof(uint4));
+        ART_TRY(small ? store_words<kSmall>(from + at, n, dst, g->stream)
+                      : store_words<kLarge>(from + at, n, dst, g->stream));
+        at += n;
+    }
+    // captured into a graph, the table changes whenever the graph runs: no call can tell any more
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    ART_TRY(cudaStreamIsCapturing(g->stream, &cs));
+    t.in_graph = t.in_graph || cs != cudaStreamCaptureStatusNone;
+    if (!t.in_graph) {
+        t.sent.assign(from, from + bytes);
+        t.known = true;
+    }
+    return ART_OK;
+}
+
 // Source table, per-source l_max, direction tables, level constants and ray buffers for a
 // trace with parameters p. Allocates only when something grew or changed.
 int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
@@ -270,88 +318,41 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
     // the allocation of the source table (freeing one more block costs a grid's end 0.1 ms). A block
     // that has become too small for them alone may be in use by a captured trace and is kept.
     const size_t groups = !adjoint && l0 >= 2 && l0 <= 6 ? (size_t)ns * (npix0 / 32) : 0;
-    if ((size_t)ns > g->src_cap || groups > g->first_cap) {
-        const size_t cap = std::max((size_t)ns, g->src_cap), gcap = std::max(groups, g->first_cap);
-        if ((size_t)ns > g->src_cap) {
-            dev_free(g->d_src);
-            free_retired(g);
+    SourceTables& T = g->tables[adjoint ? 1 : 0];
+    if ((size_t)ns > T.cap || groups > T.first_cap) {
+        const size_t cap = (std::max((size_t)ns, T.cap) + 3) & ~(size_t)3;
+        const size_t gcap = std::max(groups, T.first_cap);
+        if ((size_t)ns > T.cap) {
+            dev_free(T.src);
+            if (!adjoint) free_retired(g);
         } else {
-            g->retired.push_back(g->d_src);
+            g->retired.push_back(T.src);
         }
-        g->d_src = nullptr;
-        g->src_cap = g->first_cap = 0;
-        g->prep_valid = false;
+        T = SourceTables{nullptr, nullptr, nullptr, nullptr, 0, 0, {}, {}, T.levels_sent};
         char* block = nullptr;
-        int rc = dev_alloc(&block, cap * sizeof(SrcDev) + gcap * 8 * sizeof(float4));
+        const int rc = dev_alloc(&block, cap * (sizeof(SrcDev) + sizeof(double) + sizeof(float)) +
+                                             gcap * 8 * sizeof(float4));
         if (rc) return rc;
-        g->d_src = reinterpret_cast<SrcDev*>(block);
-        g->d_first = reinterpret_cast<float*>(g->d_src + cap);
-        g->src_cap = cap;
-        g->first_cap = gcap;
+        T.src = reinterpret_cast<SrcDev*>(block);
+        T.first = reinterpret_cast<float*>(T.src + cap);
+        T.dL = reinterpret_cast<double*>(T.first + gcap * 8 * 4);
+        T.lum = reinterpret_cast<float*>(T.dL + cap);
+        T.cap = cap;
+        T.first_cap = gcap;
     }
-    // uploads only when the sources or the parameters that shape the tables changed, so an
-    // unchanged trace enqueues no host-to-device copy (and can be captured in a CUDA graph)
-    const bool same = g->prep_valid && g->prep_version == g->src_version &&
-                      g->prep_level0 == l0 && g->prep_level_max == p->level_max &&
-                      g->prep_m_ray == p->m_ray && g->prep_adjoint == adjoint &&
-                      g->prep_schedule == p->schedule && g->prep_qcap == p->queue_capacity &&
-                      g->prep_two_bin == g->two_bin;
-    if (!same) {
-        g->h_src_stage.assign(hs.data(), hs.data() + hs.size());
-        if (!g->h_src_stage.data()) return ART_ENOMEM;
-        ART_TRY(cudaMemcpyAsync(g->d_src, g->h_src_stage.data(), ns * sizeof(SrcDev),
-                                cudaMemcpyHostToDevice, g->stream));
-    }
+    int rc = send_table(g, T.src_sent, hs.data(), ns * sizeof(SrcDev), T.src);
+    if (rc) return rc;
     g->lmax_glob = lmax_glob;
-    if (adjoint) {
-        const bool grow = (size_t)ns > g->srcL_cap;
-        if (grow) {
-            dev_free(g->d_srcL);
-            dev_free(g->d_dL_scratch);
-            g->d_srcL = nullptr;
-            g->d_dL_scratch = nullptr;
-            g->srcL_cap = 0;
-            int rc = dev_alloc(&g->d_srcL, ns);
-            if (!rc) rc = dev_alloc(&g->d_dL_scratch, ns);
-            if (rc) return rc;
-            g->srcL_cap = ns;
-        }
-        if (!same || grow) {
-            g->h_srcL.resize(ns);
-            for (int s = 0; s < ns; ++s) g->h_srcL[s] = (float)g->L[s];
-            ART_TRY(cudaMemcpyAsync(g->d_srcL, g->h_srcL.data(), ns * sizeof(float),
-                                    cudaMemcpyHostToDevice, g->stream));
-        }
+    if (adjoint || g->two_bin) {
+        std::vector<float> lum((ns + 3) & ~3, 0.f);  // whole words of 16 bytes
+        for (int s = 0; s < ns; ++s) lum[s] = (float)(adjoint ? g->L[s] : g->Ln[s] / (double)npix0);
+        if ((rc = send_table(g, T.lum_sent, lum.data(), lum.size() * sizeof(float), T.lum))) return rc;
     }
-    if (g->two_bin && !adjoint) {
-        if ((size_t)ns > g->srcLn_cap) {
-            dev_free(g->d_srcLn);
-            g->d_srcLn = nullptr;
-            g->srcLn_cap = 0;
-            int rc = dev_alloc(&g->d_srcLn, ns);
-            if (rc) return rc;
-            g->srcLn_cap = ns;
-            g->prep_valid = false;
-        }
-        if (!same || !g->prep_valid) {
-            g->h_Ln_stage.resize(ns);
-            for (int s = 0; s < ns; ++s) g->h_Ln_stage[s] = (float)(g->Ln[s] / (double)npix0);
-            g->h_srcLn_pin.assign(g->h_Ln_stage.data(), g->h_Ln_stage.data() + ns);
-            if (!g->h_srcLn_pin.data()) return ART_ENOMEM;
-            ART_TRY(cudaMemcpyAsync(g->d_srcLn, g->h_srcLn_pin.data(), ns * sizeof(float),
-                                    cudaMemcpyHostToDevice, g->stream));
-        }
-        if (!g->d_chi2) {
-            int rc = dev_alloc(&g->d_chi2, g->npad + 1);
-            if (rc) return rc;
-        }
-    }
+    if (g->two_bin && !adjoint && !g->d_chi2 && (rc = dev_alloc(&g->d_chi2, g->npad + 1))) return rc;
     // --- direction tables (FP64 HEALPix, rotated), rebuilt when the rotation changes
-    {
-        const int rc = ensure_directions(g, p, l0, lmax_glob);
-        if (rc) return rc;
-    }
+    if ((rc = ensure_directions(g, p, l0, lmax_glob))) return rc;
     // --- level constants
+    static_assert(sizeof(SrcDev) % 16 == 0 && sizeof(LevelInfo) * kNL % 16 == 0, "stored in words");
     LevelInfo lv[kNL];
     std::memset(lv, 0, sizeof(lv));
     const double unit = rmax_unit(p->m_ray);
@@ -364,11 +365,7 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         lv[l].dir = g->dir[l];
         lv[l].destroy_w = 1ull << (2 * (lmax_glob - l));
     }
-    if (!same || std::memcmp(lv, g->h_levels, sizeof(lv)) != 0) {
-        std::memcpy(g->h_levels, lv, sizeof(lv));
-        ART_TRY(cudaMemcpyAsync(g->d_levels, g->h_levels, sizeof(lv), cudaMemcpyHostToDevice,
-                                g->stream));
-    }
+    if ((rc = send_table(g, T.levels_sent, lv, sizeof(lv), g->d_levels + (adjoint ? kNL : 0)))) return rc;
     // --- fronts: deeper levels hold at most the queue capacity (persistent) or one source's
     // whole front (plain); the base level of a forward trace needs no storage
     const bool plain = p->schedule == ART_SCHED_PLAIN;
@@ -380,7 +377,6 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         else if (plain) need = p->queue_capacity > 0 ? (unsigned long long)qcap : front;
         else need = std::min<unsigned long long>((unsigned long long)qcap, (unsigned long long)ns * front);
         need = (need + 3) & ~3ull;
-        int rc = ART_OK;
         if (adjoint) {
             rc = ensure_adjoint_front(g, l, std::max(need / 4, 4ull));
         } else if (l > l0) {
@@ -391,15 +387,6 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         if (rc) return rc;
     }
     g->first_ordered = groups > 0 && (plain || l0 == lmax_glob || g->quad[l0 + 1].cap / 4 > 16);
-    g->prep_valid = true;
-    g->prep_version = g->src_version;
-    g->prep_level0 = l0;
-    g->prep_level_max = p->level_max;
-    g->prep_m_ray = p->m_ray;
-    g->prep_adjoint = adjoint;
-    g->prep_schedule = p->schedule;
-    g->prep_qcap = p->queue_capacity;
-    g->prep_two_bin = g->two_bin;
     return ART_OK;
 }
 
@@ -447,8 +434,9 @@ int run_opacity(art_grid* g, const art_params* p, bool two_bin, bool clear4, boo
     return ART_OK;
 }
 
-TraceArgs make_args(art_grid* g, const art_params* p)
+TraceArgs make_args(art_grid* g, const art_params* p, bool adjoint)
 {
+    const SourceTables& T = g->tables[adjoint ? 1 : 0];
     TraceArgs A;
     std::memset(&A, 0, sizeof(A));
     // the d_max cutoff (read only by the kernels built for a cutoff)
@@ -463,16 +451,17 @@ TraceArgs make_args(art_grid* g, const art_params* p)
     A.tau_max = (float)p->tau_max;
     A.chi = g->d_chi;
     A.chi2 = g->d_chi2;
-    A.srcLn = g->d_srcLn;
+    A.srcLn = T.lum;
     A.acc = g->d_acc;
-    A.src = g->d_src;
-    A.levels = g->d_levels;
+    A.srcL = T.lum;
+    A.src = T.src;
+    A.levels = g->d_levels + (adjoint ? kNL : 0);
     for (int l = 0; l < kNL; ++l) {
         A.adj[l] = g->adj[l];
         A.quad[l] = g->quad[l];
         if (l > g->lmax_glob) A.adj[l].cap = A.quad[l].cap = 0;
     }
-    if (g->first_ordered) A.first = g->d_first;
+    if (g->first_ordered) A.first = T.first;
     A.base_quads = 3u << (2 * p->level0);
     A.nsrc = (unsigned)g->L.size();
     A.npad = (unsigned)g->npad;
@@ -565,7 +554,7 @@ int art_create_grid(art_grid** out, int nx, int ny, int nz, const double box_lo[
     if (!rc) rc = cuda_status(cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device));
     if (!rc) rc = dev_alloc(&g->d_chi, npad + 1);
     if (!rc) rc = dev_alloc(&g->d_acc, npad);
-    if (!rc) rc = dev_alloc(&g->d_levels, kNL);
+    if (!rc) rc = dev_alloc(&g->d_levels, 2 * kNL);
     if (!rc) rc = dev_alloc(&g->d_state, 1);
     if (!rc) {
         g->d_sched = &g->d_state->sched;
@@ -574,7 +563,6 @@ int art_create_grid(art_grid** out, int nx, int ny, int nz, const double box_lo[
         g->state_clean = rc == ART_OK;
     }
     if (!rc) rc = cuda_status(cudaMallocHost((void**)&g->h_stats, sizeof(DevStats)));
-    if (!rc) rc = cuda_status(cudaMallocHost((void**)&g->h_levels, sizeof(LevelInfo) * kNL));
     if (rc) {
         art_destroy_grid(g);
         return rc;
@@ -605,7 +593,6 @@ int art_add_sources(art_grid* g, int n, const double* h_pos, const double* h_L)
     g->pos.insert(g->pos.end(), h_pos, h_pos + 3 * (size_t)n);
     g->L.insert(g->L.end(), h_L, h_L + (size_t)n);
     if (g->two_bin) g->Ln.insert(g->Ln.end(), (size_t)n, 0.0);
-    g->src_version += 1;
     return ART_OK;
 }
 
@@ -616,7 +603,6 @@ int art_clear_sources(art_grid* g)
     g->L.clear();
     g->Ln.clear();
     g->two_bin = false;
-    g->src_version += 1;
     return ART_OK;
 }
 
@@ -626,7 +612,6 @@ int art_set_nonionizing(art_grid* g, const double* h_Ln)
     if (!h_Ln) {
         g->two_bin = false;
         g->Ln.clear();
-        g->src_version += 1;
         return ART_OK;
     }
     if (g->L.empty()) return ART_ESTATE;
@@ -634,7 +619,6 @@ int art_set_nonionizing(art_grid* g, const double* h_Ln)
         if (!(h_Ln[s] >= 0.0) || !std::isfinite(h_Ln[s])) return ART_EINVAL;
     g->Ln.assign(h_Ln, h_Ln + g->L.size());
     g->two_bin = true;
-    g->src_version += 1;
     return ART_OK;
 }
 
@@ -655,7 +639,7 @@ int art_trace(art_grid* g, const art_params* p, float* d_gamma, float* d_force, 
     const int ns = (int)g->L.size();
     const int l0 = p->level0;
     const int threads = trace_threads(p);
-    TraceArgs A = make_args(g, p);
+    TraceArgs A = make_args(g, p, false);
     if (p->schedule == ART_SCHED_PLAIN) {
         int per_sm = 0;
         const auto kern = level_kernel(g->two_bin, p->d_max > 0.0, d_force != nullptr);
@@ -734,17 +718,15 @@ void art_destroy_grid(art_grid* g)
     cudaStreamSynchronize(g->stream);
     dev_free(g->d_chi);
     dev_free(g->d_acc);
-    dev_free(g->d_src);
+    dev_free(g->tables[0].src);
+    dev_free(g->tables[1].src);
     free_retired(g);
     dev_free(g->d_levels);
     dev_free(g->d_state);
-    dev_free(g->d_srcL);
     dev_free(g->d_rec);
     dev_free(g->d_recf);
     dev_free(g->d_recw);
     dev_free(g->d_chi2);
-    dev_free(g->d_srcLn);
-    dev_free(g->d_dL_scratch);
     for (int l = 0; l < kNL; ++l) {
         dev_free(g->dir[l]);
         dev_free(g->quad[l].rec);
@@ -753,7 +735,6 @@ void art_destroy_grid(art_grid* g)
         dev_free(b.rec); dev_free(b.parent); dev_free(b.own); dev_free(b.sub);
     }
     if (g->h_stats) cudaFreeHost(g->h_stats);
-    if (g->h_levels) cudaFreeHost(g->h_levels);
     delete g;
 }
 

@@ -8,27 +8,29 @@
 #include "art.h"
 #include "art_device.cuh"
 
-// A growable array in pinned host memory (copies from it can be captured in a graph).
-template <class T>
-struct PinnedVec {
-    T* data_ = nullptr;
-    size_t n_ = 0, cap_ = 0;
-    ~PinnedVec() { if (data_) cudaFreeHost(data_); }
-    T* data() { return data_; }
-    void assign(const T* b, const T* e)
-    {
-        size_t n = (size_t)(e - b);
-        if (n > cap_) {
-            if (data_) cudaFreeHost(data_);
-            data_ = nullptr;
-            cap_ = 0;
-            if (cudaMallocHost((void**)&data_, n * sizeof(T)) != cudaSuccess) { data_ = nullptr; n_ = 0; return; }
-            cap_ = n;
-        }
-        for (size_t i = 0; i < n; ++i) data_[i] = b[i];
-        n_ = n;
-    }
+namespace art {
+
+// A table in device memory that the host writes: what was last stored there, while that is known.
+struct HostTable {
+    std::vector<unsigned char> sent;
+    bool known = false;
+    bool in_graph = false;   // a graph holds a store to it
 };
+
+// What the device holds per source, once per direction: a forward trace and a reverse sweep need
+// different luminosities, and alternating calls would replace each other's tables. One block of
+// device memory.
+struct SourceTables {
+    SrcDev* src = nullptr;   // start of the block
+    float* first = nullptr;  // forward: sums of first segments, kept for a fixed order of addition
+    double* dL = nullptr;    // reverse: dloss/dL of callers that pass no buffer
+    float* lum = nullptr;    // forward: base-ray non-ionizing luminosities; reverse: luminosities
+    size_t cap = 0;          // sources
+    size_t first_cap = 0;    // groups of 32 base rays
+    HostTable src_sent, lum_sent, levels_sent;
+};
+
+}  // namespace art
 
 struct art_grid {
     int device = 0;
@@ -46,19 +48,16 @@ struct art_grid {
     std::vector<double> Ln;      // non-ionizing luminosities (two-bin traces)
     bool two_bin = false;
     float2* d_chi2 = nullptr;    // {chi_i, chi_n} per cell length (two-bin traces, padded)
-    float* d_srcLn = nullptr;    // base-ray non-ionizing luminosity per source
-    size_t srcLn_cap = 0;
-    std::vector<float> h_Ln_stage;
-    PinnedVec<float> h_srcLn_pin;
     std::vector<int> src_lmax;
+    art::SourceTables tables[2];     // forward, reverse
+    art::LevelInfo* d_levels = nullptr;  // level constants, kNL per direction
+    std::vector<void*> retired;      // former blocks of the forward tables (see prepare_trace)
+    bool first_ordered = false;      // the prepared trace keeps its first segments
 
     // device buffers owned by the grid
     float* d_chi = nullptr;      // opacity per cell length (padded layout)
     float4* d_acc = nullptr;     // per-cell accumulator (padded layout); traces without a force
                                  // and the reverse sweep's gradient use the first npad floats
-    art::SrcDev* d_src = nullptr;
-    size_t src_cap = 0;
-    art::LevelInfo* d_levels = nullptr;
     art::DevState* d_state = nullptr;  // scheduler and counters, cleared together
     bool state_clean = false;          // d_state is clear once the stream gets here
     bool state_dirty_captured = false; // this trace's clearing of it is only captured
@@ -66,7 +65,7 @@ struct art_grid {
     art::DevStats* d_stats = nullptr;  // in d_state
     art::DevStats* h_stats = nullptr;  // pinned
 
-    float4* dir[art::kNL] = {};     // per level: 3 float4 per pixel (n and 1/n as df)
+    float4* dir[art::kNL] = {};     // per level: 3 float4 per pixel (n as df, face spacing codes)
     bool dir_built[art::kNL] = {};
     bool dir_rotate = false;
     double dir_rot[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
@@ -75,34 +74,14 @@ struct art_grid {
     art::QuadBuf quad[art::kNL] = {};
     unsigned long long quad_cap[art::kNL] = {};      // allocated quads per level
 
-    // sums of the base rays' first segments, kept for a fixed order of addition
-    float* d_first = nullptr;        // behind the source table, in its allocation
-    size_t first_cap = 0;            // groups of 32 rays that it holds
-    bool first_ordered = false;      // the prepared trace keeps them
-    std::vector<void*> retired;      // former blocks of the table and the sums (see prepare_trace)
-
     // adjoint fronts
     art::AdjBuf adj[art::kNL] = {};
     unsigned long long adj_cap[art::kNL] = {};       // allocated quads per level
 
-    // adjoint: source luminosities and a dL buffer for callers that pass none
-    float* d_srcL = nullptr;
+    // adjoint: cell records
     float4* d_rec = nullptr;     // per-cell {chi, chi_H, w, 0} of the reverse sweep (padded)
     art::CellF* d_recf = nullptr;  // the same with the force weight (loss with a force term)
     art::CellW* d_recw = nullptr;  // {chi, w} per cell (loss without dust or force term)
-    double* d_dL_scratch = nullptr;
-    size_t srcL_cap = 0;
-    std::vector<float> h_srcL;
-
-    // what the device copies of the source table and level constants were built from
-    art::LevelInfo* h_levels = nullptr;          // pinned staging of the level constants
-    PinnedVec<art::SrcDev> h_src_stage;          // pinned staging of the source table
-    unsigned long long src_version = 0;
-    unsigned long long prep_version = 0;
-    bool prep_valid = false, prep_adjoint = false, prep_two_bin = false;
-    int prep_level0 = -1, prep_level_max = -2, prep_schedule = -1;
-    double prep_m_ray = 0.0;
-    long long prep_qcap = -1;
 
     int lmax_glob = 0;
     int last_lmax = 0;
@@ -127,6 +106,6 @@ fix to_fix(double cells, int fbits);
 Coef coef_of(double v);
 SrcDev source_record(const art_grid* g, const double u[3], double base_L, int lmax);
 int prepare_trace(art_grid* g, const art_params* p, bool adjoint);
-TraceArgs make_args(art_grid* g, const art_params* p);
+TraceArgs make_args(art_grid* g, const art_params* p, bool adjoint);
 int finish_stats(art_grid* g, art_stats* out);
 }  // namespace art
