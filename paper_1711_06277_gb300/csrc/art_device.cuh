@@ -439,8 +439,6 @@ __device__ __forceinline__ float2 vrcp_max1(float2 v)
 {
     return make_float2(rcp_ftz(fmaxf(v.x, 1.f)), rcp_ftz(fmaxf(v.y, 1.f)));
 }
-__device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ float2 vmax(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
 // a where x < 1, else b
 __device__ __forceinline__ float vbelow1(float x, float a, float b) { return x < 1.f ? a : b; }
 __device__ __forceinline__ float2 vbelow1(float2 x, float2 a, float2 b)
@@ -454,9 +452,9 @@ __device__ __forceinline__ float vget(const float2& v, int j) { return j ? v.y :
 
 // phi(x) = (1 - e^-x)/x for x >= 0. Below 1 as E sinh(y)/y with y = x/2 and E = e^{-y}, the even
 // series of sinh(y)/y to y^8 (truncation < 3e-11 for y < 1/2, no cancellation); above 1 as
-// (1 - E^2)/x. One exponential serves both. The first form falls below phi above 1 (its series
-// is cut short; NaN where it overflows against E = 0) and the second, with x replaced by
-// max(x, 1), falls below phi below 1, so phi is the larger of the two and lanes never diverge.
+// (1 - E^2)/x. One exponential serves both, and both are formed: lanes never diverge. Chosen by x,
+// not as the larger of the two: up to x = 2 they differ by rounding (the error of E enters them with
+// opposite signs), and the larger would bias a sum of many (2e-8 of the photons absorbed there).
 template <class V>
 __device__ __forceinline__ V phi_of(V x)
 {
@@ -467,13 +465,13 @@ __device__ __forceinline__ V phi_of(V x)
     S = vfma(S, x2, vset<V>(1.f / 24.f));
     S = vfma(S, x2, vset<V>(1.f));
     const V large = vmul(vfma(vmul(E, vset<V>(-1.f)), E, vset<V>(1.f)), vrcp_max1(x));
-    return vmax(vmul(E, S), large);
+    return vbelow1(x, vmul(E, S), large);
 }
 
 // phi(x) and phi'(x) of a ray of the reverse sweep, which needs both. Below 1, with y = x/2,
 // E = e^{-y} and S = sinh(y)/y: phi = E S and phi' = E (S'(y) - S) / 2, S' to y^7 (S' - S stays
-// near -1, so nothing cancels); above 1, phi' = (e^{-x} - phi)/x. Chosen by x, not as the larger
-// of the two: near 1 they differ by rounding, and the larger would bias a sum of many.
+// near -1, so nothing cancels); above 1, phi' = (e^{-x} - phi)/x. Chosen by x as in
+// phi_of.
 template <bool kDerivative, class V>
 __device__ __forceinline__ V phi_dphi(V x, V& dphi)
 {
