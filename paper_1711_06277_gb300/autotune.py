@@ -8,13 +8,16 @@ a sample of the grid's sources (the cost of a trace is a sum over sources, so a 
 the candidates like the whole set). A small sample separates the candidates that differ by
 several percent but not the close ones, whose order can change with the number of sources in
 flight, so the fastest few are timed again on a larger sample when the workload has more
-sources than the first one. The winner is cached in a JSON file keyed by the grid shape, the
-number of sources and the base level, so later runs of the same workload shape skip the
-search.
+sources than the first one. Candidates are timed with the outputs that the caller will ask for
+(traces with and without a force are kernels of their own). The winner is cached in a JSON file
+keyed by the grid shape, the number of sources, the base level, what selects the kernel (force,
+cutoff) and the kernels' sources, so later runs of the same workload shape skip the search and
+knobs found for other kernels are not used.
 """
 from __future__ import annotations
 
 import dataclasses
+import hashlib
 import itertools
 import json
 import os
@@ -23,6 +26,7 @@ import numpy as np
 import torch
 
 from . import art as A
+from . import build
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "tune_cache.json")
 
@@ -32,8 +36,18 @@ DEFAULT_SPACE = {
 }
 
 
-def _key(shape, nsrc, params: A.Params) -> str:
-    return f"{shape[0]}x{shape[1]}x{shape[2]}|src{nsrc}|l0{params.level0}|m{params.m_ray}"
+def _kernel_version() -> str:
+    """Digest of the trace kernels' sources."""
+    h = hashlib.sha256()
+    for name in ("art_kernels.cuh", "art_device.cuh"):
+        with open(os.path.join(build.CSRC, name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
+def _key(shape, nsrc, params: A.Params, force: bool = True) -> str:
+    return (f"{shape[0]}x{shape[1]}x{shape[2]}|src{nsrc}|l0{params.level0}|m{params.m_ray}"
+            f"|cut{int(params.d_max > 0)}|force{int(force)}|{_kernel_version()}")
 
 
 def _load_cache(path):
@@ -44,17 +58,17 @@ def _load_cache(path):
         return {}
 
 
-def _time_knobs(g, params: A.Params, knobs: dict, repeats: int, stream) -> float:
+def _time_knobs(g, params: A.Params, knobs: dict, repeats: int, stream, force: bool) -> float:
     """Best of ``repeats`` timed traces with these knobs (after one untimed trace, which also
     allocates); inf if the trace reports an error."""
     p = dataclasses.replace(params, schedule="persistent", **knobs)
-    g.trace(p, force=False)
+    g.trace(p, force=force)
     best = float("inf")
     for _ in range(repeats):
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         e0.record(stream)
-        g.trace(p, force=False, stats=False)
+        g.trace(p, force=force, stats=False)
         e1.record(stream)
         e1.synchronize()
         best = min(best, e0.elapsed_time(e1))
@@ -64,13 +78,14 @@ def _time_knobs(g, params: A.Params, knobs: dict, repeats: int, stream) -> float
 def tune(nH0: torch.Tensor, dx: float, pos, L, params: A.Params, sample: int = 16,
          space: dict | None = None, repeats: int = 2, cache_path: str | None = CACHE,
          nH: torch.Tensor | None = None, lo=(0.0, 0.0, 0.0), verbose: bool = False,
-         refine_sample: int = 128, finalists: int = 3) -> A.Params:
+         refine_sample: int = 128, finalists: int = 3, force: bool = True) -> A.Params:
     """Returns ``params`` with the fastest knobs for this workload shape: every candidate
     timed on ``sample`` sources, then the ``finalists`` fastest on ``refine_sample`` sources
-    (when the workload has more sources than the first sample)."""
+    (when the workload has more sources than the first sample). ``force``: whether the traces to
+    come ask for the force."""
     pos = np.asarray(pos, dtype=np.float64).reshape(-1, 3)
     L = np.asarray(L, dtype=np.float64).reshape(-1)
-    key = _key(tuple(nH0.shape), len(L), params)
+    key = _key(tuple(nH0.shape), len(L), params, force)
     cache = _load_cache(cache_path) if cache_path else {}
     if key in cache:
         return dataclasses.replace(params, **cache[key]["knobs"])
@@ -84,7 +99,7 @@ def tune(nH0: torch.Tensor, dx: float, pos, L, params: A.Params, sample: int = 1
     names = list(space)
     for combo in itertools.product(*(space[n] for n in names)):
         knobs = dict(zip(names, combo))
-        best = _time_knobs(g, params, knobs, repeats, stream)
+        best = _time_knobs(g, params, knobs, repeats, stream, force)
         if best == float("inf"):
             continue
         results.append((best, knobs))
@@ -101,7 +116,7 @@ def tune(nH0: torch.Tensor, dx: float, pos, L, params: A.Params, sample: int = 1
         g.add_sources(pos[idx2], L[idx2])
         refined = []
         for _, knobs in results[:finalists]:
-            best = _time_knobs(g, params, knobs, repeats, stream)
+            best = _time_knobs(g, params, knobs, repeats, stream, force)
             if best < float("inf"):
                 refined.append((best, knobs))
             if verbose:
