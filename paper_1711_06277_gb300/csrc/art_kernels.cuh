@@ -110,6 +110,14 @@ __global__ void k_directions(int level, unsigned long long npix, double r0, doub
     } else {
         w[0] = v[0]; w[1] = v[1]; w[2] = v[2];
     }
+    // Distances along directions of length 1/2 or more stay below kFar inside the box, and every
+    // step of a walk moves its ray. Where a matrix that is no rotation makes them shorter, they
+    // are lengthened to 1: a ray whose faces all lie beyond kFar would never end.
+    const double len2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+    if (!(len2 >= 0.25)) {
+        const double scale = len2 > 0.0 ? 1.0 / sqrt(len2) : 0.0;
+        for (int a = 0; a < 3; ++a) w[a] = scale > 0.0 ? w[a] * scale : (a == 0 ? 1.0 : 0.0);
+    }
     float h[3], l[3];
     fix d[3];
 #pragma unroll
