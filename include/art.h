@@ -83,7 +83,8 @@ typedef struct {
                             whose phases run longer than the bound need a larger value
                             (the trace then fails with ART_ETIMEOUT, results incomplete) */
     int blocks_per_sm;   /* resident blocks per SM of the persistent trace (0 = as many as
-                            fit); fewer blocks keep fewer rays in flight */
+                            fit); fewer blocks keep fewer rays in flight. At the default block
+                            size one block fills an SM: matters with smaller blocks only */
     double d_max;        /* > 0: every ray ends at this distance from its source (the cutoff
                             of the weak-scaling test, Sec. 3.1), its remaining L counted as
                             escaped; at d_max = r_max(l) the cut wins over the split.

@@ -49,7 +49,6 @@ __device__ __forceinline__ df df_add(df a, df b)
     df s = df_two_sum(a.hi, b.hi);
     return df_quick(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
-__device__ __forceinline__ df df_neg(df a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ df df_mul(df a, df b)
 {
     float p = __fmul_rn(a.hi, b.hi);
@@ -160,8 +159,8 @@ struct DevStats {
 
 // Scheduler state of the persistent trace and of the plain per-level launches.
 struct Sched {
-    unsigned long long count[kNL];   // rays held in the level buffer (a stack, top = count)
-    unsigned long long cursor[kNL];  // next ray of the current phase / launch
+    unsigned long long count[kNL];   // quads held in the level's front (a stack, top = count)
+    unsigned long long cursor[kNL];  // next item (one or two rays) of the current phase / launch
     unsigned long long phase_begin, phase_end;
     int phase_level, phase_width, phase_strided, phase_kind, done, started;
     // adjoint: quads of a level whose descendants are still being swept
@@ -230,19 +229,11 @@ struct TraceArgs {
 // ---------------------------------------------------------------------------------------
 // Per-cell record gathered at every step: the opacity alone (forward), or
 // {opacity, its neutral-H part, loss weight, unused} (adjoint).
-__device__ __forceinline__ float chi_of(const float& c) { return c; }
 __device__ __forceinline__ float chi_of(const float4& c) { return c.x; }
-__device__ __forceinline__ float chi_of(const float2& c) { return c.x; }
 // A cell record of two floats marks a two-bin trace: {chi_i, chi_n}.
 template <class Cell> struct TwoBin { static constexpr bool value = false; };
 template <> struct TwoBin<float2> { static constexpr bool value = true; };
-__device__ __forceinline__ float load_cell(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float4 load_cell(const float4* p) { return __ldg(p); }
-__device__ __forceinline__ float2 load_cell(const float2* p) { return __ldg(p); }
-template <class Cell> __device__ __forceinline__ Cell cell_zero();
-template <> __device__ __forceinline__ float cell_zero<float>() { return 0.f; }
-template <> __device__ __forceinline__ float4 cell_zero<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-template <> __device__ __forceinline__ float2 cell_zero<float2>() { return make_float2(0.f, 0.f); }
 // Cell record of a reverse sweep whose loss has a force term: {chi, chi_H, w, 0} and the
 // force weight {v_x, v_y, v_z, 0} (32 bytes, two 16-byte gathers per step).
 struct CellF {
@@ -260,11 +251,6 @@ __device__ __forceinline__ CellW load_cell(const CellW* p)
 {
     const float2 v = __ldg(reinterpret_cast<const float2*>(p));
     return {v.x, v.y};
-}
-template <> __device__ __forceinline__ CellW cell_zero<CellW>() { return {0.f, 0.f}; }
-template <> __device__ __forceinline__ CellF cell_zero<CellF>()
-{
-    return {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
 }
 
 // Where a ray is on its way through the grid.
@@ -738,7 +724,7 @@ __device__ __forceinline__ void red_if(float4* __restrict__ acc, int key, float4
 // helpers shared by the forward and backward kernels
 // ---------------------------------------------------------------------------------------
 // Threads per block of the trace kernels at most: one block of 20 warps per SM (65536 / 640 =
-// 102 registers a thread: two walks), so that a grid barrier has 152 arrivals and not 760. 24
+// 102 registers a thread, 96 in steps of eight: two walks), so that a grid barrier has 152 arrivals and not 760. 24
 // warps (80 registers) gain 5 % at 256^3 and lose 2 % at 512^3 and 3 % in the sweep.
 constexpr int kTraceMaxThreads = 640;
 constexpr int kTraceMinBlocks = 1;

@@ -342,6 +342,7 @@ int art_dt_substep_static(void* stream, long long ncell, const float* d_gamma, c
     // block in this call, so nothing carries over from an earlier call
     const int tiles = (int)((ncell + 255) / 256);
     cudaStream_t s = (cudaStream_t)stream;
+    // (a cell per thread: four at a time, a tile would use a quarter of its block's threads)
     k_dt_partial<<<tiles, 256, 0, s>>>(ncell, false, d_gamma, d_nH, d_xn, (float)alpha_B, partials);
     k_dt_final<<<1, 1024, 0, s>>>(tiles, partials, C, d_dt);
     return cudaGetLastError() == cudaSuccess ? ART_OK : ART_ECUDA;
