@@ -669,6 +669,17 @@ __device__ __forceinline__ void add_pair(float4& sum, float4& rest, float4 b)
     add_pair(sum.w, rest.w, b.w);
 }
 
+// sum + rest; a sum that has overflowed (its error is no number then) stays as it is
+__device__ __forceinline__ float with_rest(float sum, float rest)
+{
+    return fabsf(rest) <= 3.4e38f ? sum + rest : sum;
+}
+__device__ __forceinline__ float4 with_rest(float4 sum, float4 rest)
+{
+    return make_float4(with_rest(sum.x, rest.x), with_rest(sum.y, rest.y), with_rest(sum.z, rest.z),
+                       with_rest(sum.w, rest.w));
+}
+
 template <class D>
 __device__ __forceinline__ void merge_lanes(int& cell, D& v)
 {

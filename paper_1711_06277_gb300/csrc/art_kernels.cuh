@@ -293,8 +293,7 @@ __device__ __forceinline__ D sum_first(const D* from, unsigned groups)
         add_pair(sum, rest, s2);
         add_to(rest, r2);
     }
-    add_to(sum, rest);
-    return sum;
+    return with_rest(sum, rest);
 }
 
 // Adds the kept sums of all sources to the accumulator, a warp per source, the warps with the last

@@ -51,3 +51,19 @@ def test_substep_size_repeats():
     got = {float(art.dt_substep(g.trace(p, force=False, stats=False)["gamma"], nH, x, 1.0).cpu()) for _ in range(12)}
     assert len(got) == 1
     g.close()
+
+
+@pytest.mark.parametrize("level0", [2, 3, 4])
+@pytest.mark.parametrize("force", [False, True])
+def test_overflowing_rate_is_infinite(level0, force):
+    """The rate of the source's cell beyond the largest float: plus infinity, and no NaN."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1711_06277_gb300 import art
+    rho = torch.full((N, N, N), 1e-6, device="cuda")
+    g = art.Grid(rho, 1.0)
+    g.add_sources([[10.5, 12.5, 11.5]], [2e38 * 12 * 4 ** level0])   # every base ray is a float
+    gamma = g.trace(art.Params(level0=level0, sigma_H=1.0), force=force)["gamma"]
+    assert float(gamma[11, 12, 10]) == float("inf")
+    assert not bool(torch.isnan(gamma).any())
+    g.close()
