@@ -222,9 +222,10 @@ __device__ __forceinline__ typename DepositOf<kForce>::type* accumulator(const T
 // next to a single source, the largest of the field, and with it the substep size are the same in
 // every run; added as the warps got to them, 96 sums at l0 = 4 differed by 1e-7 to 6e-7 from run to
 // run. They are added in two floats: their order in one float leaves up to 8e-7 (equal sums of
-// symmetric directions in a row are rounded alike). The six sums of l0 = 2 are added in one, those
-// of even number first, which is what the former walk (64 base rays per warp, the first half of
-// each first) came to in every run.
+// symmetric directions in a row are rounded alike). The 6 and 24 sums of l0 = 2 and 3 are added in
+// one, where the former walk (64 base rays per warp, the first half of each first) came to one
+// value in nearly every run, and in the order that gives it most often: the last groups first, those
+// of odd number at l0 = 3 one place late.
 template <class D>
 struct FirstSegments {  // of the rays of a block on their way
     D value[2][kTraceMaxThreads];
@@ -276,8 +277,16 @@ __device__ __forceinline__ D sum_first(const D* from, unsigned groups)
     const unsigned lane = threadIdx.x & 31u;
     from += lane % 8u;
     D sum{}, rest{};
-    if (groups <= 6u) {
-        for (unsigned t = 0; t < groups; ++t) add_to(sum, __ldcg(from + 8u * (t < 3u ? 2u * t : 2u * t - 5u)));
+    if (groups <= 24u) {
+        const int last = (int)groups / 2 - 1, late = groups > 6u ? 1 : 0;
+#pragma unroll 6
+        for (int t = 0; t < (int)groups; ++t) {
+            // even groups from the last down, each followed by the odd one of its pair (l0 = 2) or
+            // of the pair before; at l0 = 3 the last even one begins and the first odd one ends
+            const int u = t - late, odd = u & 1;
+            const int i = odd ? last - (u >> 1) : last - late - (u >> 1);
+            add_to(sum, __ldcg(from + 8 * (u < 0 ? 2 * last : i < 0 ? 1 : 2 * i + odd)));
+        }
         return sum;
     }
     for (unsigned t = lane / 8u; t < groups; t += 32u) {
