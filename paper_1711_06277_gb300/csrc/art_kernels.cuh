@@ -17,7 +17,7 @@
 // per lane merge more (0.51 against 0.68 sectors per crossing) but leave 12 instead of 20 warps
 // per SM (16.7 against 14.3 ms on 256^3 / 16 sources, before the step was trimmed further).
 // Against one ray per lane with refills (and floating-point pairs for the distances):
-// 85.1 -> 51.4 ms on 256^3 / 64 sources, 620 -> 415 ms on 512^3 / 64 sources, 3.52 -> 0.27 ms on
+// 85.5 -> 51.6 ms on 256^3 / 64 sources, 619 -> 409 ms on 512^3 / 64 sources, 3.55 -> 0.28 ms on
 // 128^3 / 64 sources cut at 19 cells, where rays of 7 steps had waited for refills every 64.
 //
 // Two schedules share that routine:
