@@ -24,10 +24,11 @@
 // fronts, and every part without children) need no collapse.
 //
 // Before, each lane ran its own state machine of both passes with refills, atomic count-downs of
-// the parents and completions in between, with 21 of 32 lanes active. Against that: 9.55 ->
-// 4.50 ms on 128^3 / 16 sources with a force term, 1.81 -> 0.69 ms on an odd box with force and
-// dust. What bounds it now is the issue of its instructions (69 % of cycles, 104 per ray and
-// step), then the latency of the record gathers (20 warps per SM hold 40 rays' worth).
+// the parents and completions in between, with 21 of 32 lanes active. Against that: 9.9 -> 4.6 ms
+// on 128^3 / 16 sources with a force term, 1.89 -> 0.70 ms on an odd box with force and dust. What
+// bounds it now: without a force term the issue of its instructions (68 % of cycles), with one the
+// latency of the 32-byte record gathers first (20 warps per SM hold 40 rays' worth; issue 60 %, and
+// the one form of the kernel that spills, 148 bytes).
 #include <cmath>
 #include <algorithm>
 #include <cstring>

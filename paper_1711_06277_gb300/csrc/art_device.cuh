@@ -622,11 +622,7 @@ __device__ __forceinline__ void walk_move_load(Path& W, fix rend, float unit, fl
         asm(ART_MOVE_FAST(ART_LENGTH) ART_MOVE_LOAD ART_MOVE_OPERANDS, "n"((int)sizeof(Cell)), "l"(cells));
 }
 
-// Merges the deposits of lanes that hit the same cell (runs of equal cell index in lane
-// order) into the first lane of each run and takes them from the others. Used only for the
-// first segment of base-level rays, which all start in their source's cell: at l0 = 8 that is
-// 786,432 deposits into one cell per source, whose FP32 sum the merge keeps accurate.
-// Warp-uniform.
+// Deposits (float or float4) across the lanes of a warp, and their sums.
 __device__ __forceinline__ float shifted(float v, int off) { return __shfl_down_sync(kFull, v, off); }
 __device__ __forceinline__ float4 shifted(float4 v, int off)
 {
@@ -680,6 +676,11 @@ __device__ __forceinline__ float4 with_rest(float4 sum, float4 rest)
                        with_rest(sum.w, rest.w));
 }
 
+// Merges the deposits of lanes that hit the same cell (runs of equal cell index in lane
+// order) into the first lane of each run and takes them from the others. Used only for the first
+// segments of base-level rays that are not kept for a fixed order of addition, and for their
+// gradients: at l0 = 8 that is 786,432 deposits into one cell per source, whose FP32 sum the merge
+// keeps accurate. Warp-uniform.
 template <class D>
 __device__ __forceinline__ void merge_lanes(int& cell, D& v)
 {
