@@ -314,14 +314,16 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
     // The sums of first segments are kept for a fixed order of addition where base rays come in
     // whole groups of 64 of one source (from l0 = 2; every phase of the base front then ends on such
     // a group unless it is 16 quads or less, see below) and up to l0 = 6, 1536 sums per source: the
-    // one warp that adds them takes longer beyond, and they are added as they come. They share
-    // the allocation of the source table (freeing one more block costs a grid's end 0.1 ms). A block
-    // that has become too small for them alone may be in use by a captured trace and is kept.
+    // one warp that adds them takes longer beyond, and they are added as they come. They lie behind
+    // the accumulator where they fit (creating and freeing a block of their own costs 0.3 ms from
+    // 1 MB on), else in the allocation of the source table. A block of that which has become too
+    // small for them alone may be in use by a captured trace and is kept.
     const size_t groups = !adjoint && l0 >= 2 && l0 <= 6 ? (size_t)ns * (npix0 / 32) : 0;
+    const size_t own = groups * 8 <= g->first_room ? 0 : groups;
     SourceTables& T = g->tables[adjoint ? 1 : 0];
-    if ((size_t)ns > T.cap || groups > T.first_cap) {
+    if ((size_t)ns > T.cap || own > T.first_cap) {
         const size_t cap = (std::max((size_t)ns, T.cap) + 3) & ~(size_t)3;
-        const size_t gcap = std::max(groups, T.first_cap);
+        const size_t gcap = std::max(own, T.first_cap);
         if ((size_t)ns > T.cap) {
             dev_free(T.src);
             if (!adjoint) free_retired(g);
@@ -340,6 +342,7 @@ int prepare_trace(art_grid* g, const art_params* p, bool adjoint)
         T.cap = cap;
         T.first_cap = gcap;
     }
+    g->d_first = own ? T.first : reinterpret_cast<float*>(g->d_acc + g->npad);
     int rc = send_table(g, T.src_sent, hs.data(), ns * sizeof(SrcDev), T.src);
     if (rc) return rc;
     g->lmax_glob = lmax_glob;
@@ -461,7 +464,7 @@ TraceArgs make_args(art_grid* g, const art_params* p, bool adjoint)
         A.quad[l] = g->quad[l];
         if (l > g->lmax_glob) A.adj[l].cap = A.quad[l].cap = 0;
     }
-    if (g->first_ordered) A.first = T.first;
+    if (g->first_ordered) A.first = g->d_first;
     A.base_quads = 3u << (2 * p->level0);
     A.nsrc = (unsigned)g->L.size();
     A.npad = (unsigned)g->npad;
@@ -553,7 +556,8 @@ int art_create_grid(art_grid** out, int nx, int ny, int nz, const double box_lo[
     int rc = cuda_status(cudaGetDevice(&g->device));
     if (!rc) rc = cuda_status(cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device));
     if (!rc) rc = dev_alloc(&g->d_chi, npad + 1);
-    if (!rc) rc = dev_alloc(&g->d_acc, npad);
+    g->first_room = (size_t)npad / 32;
+    if (!rc) rc = dev_alloc(&g->d_acc, npad + g->first_room);
     if (!rc) rc = dev_alloc(&g->d_levels, 2 * kNL);
     if (!rc) rc = dev_alloc(&g->d_state, 1);
     if (!rc) {

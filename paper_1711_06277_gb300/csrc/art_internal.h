@@ -22,7 +22,7 @@ struct HostTable {
 // device memory.
 struct SourceTables {
     SrcDev* src = nullptr;   // start of the block
-    float* first = nullptr;  // forward: sums of first segments, kept for a fixed order of addition
+    float* first = nullptr;  // forward: sums of first segments that do not fit behind the accumulator
     double* dL = nullptr;    // reverse: dloss/dL of callers that pass no buffer
     float* lum = nullptr;    // forward: base-ray non-ionizing luminosities; reverse: luminosities
     size_t cap = 0;          // sources
@@ -53,6 +53,8 @@ struct art_grid {
     art::LevelInfo* d_levels = nullptr;  // level constants, kNL per direction
     std::vector<void*> retired;      // former blocks of the forward tables (see prepare_trace)
     bool first_ordered = false;      // the prepared trace keeps its first segments
+    float* d_first = nullptr;        // where: behind the accumulator or in tables[0]
+    size_t first_room = 0;           // float4s behind the accumulator (a 32nd of it)
 
     // device buffers owned by the grid
     float* d_chi = nullptr;      // opacity per cell length (padded layout)
